@@ -213,12 +213,14 @@ def run_gpu(args):
     ms = barrier_max(ms, ws)
     ok = all(i["status"] == "ok" and i["relres_true"] <= cfg.tol for i in infos)
     iters = [i["iters"] for i in infos]
-    # per launch of the loop: configure, init, tail; the 5 kernels of an
-    # iteration run in passes of 4 iterations (graph) or 16 (host-driven loop),
-    # and the kernels of a pass's iterations after convergence launch and
-    # return at once
-    per_pass = 4 if args.launch == "graph" else 16
-    launches = sum(3 * (i["restarts"] + 1) + 5 * per_pass * (-(-i["iters"] // per_pass)) for i in infos)
+    # on the device: configure and one persistent kernel per solve, restarts
+    # included.  Host-driven loop: configure, init, tail per start; the 5
+    # kernels of an iteration run in passes of 16 iterations, and those of a
+    # pass's iterations after convergence launch and return at once
+    if args.launch == "graph":
+        launches = 2 * len(infos)
+    else:
+        launches = sum(3 * (i["restarts"] + 1) + 5 * 16 * (-(-i["iters"] // 16)) for i in infos)
     solves = args.steps * ws
     value = solves / (ms / 1e3)
     # independent check of the last solution with the CPU SpMV of the generator data

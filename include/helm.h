@@ -204,8 +204,11 @@ typedef enum {
 } helm_precision;
 /* How the iteration loop is driven on the device. */
 typedef enum {
-  HELM_LAUNCH_AUTO = 0,       /* graph; the host-driven loop if the graph
-                                 cannot be built */
+  HELM_LAUNCH_AUTO = 0,       /* BiCGStab (the whole FP64 solve; the complex64
+                                 inner solves of mixed precision): persistent
+                                 where the device can launch it, else as the
+                                 other methods: graph; the host-driven loop if
+                                 the graph cannot be built */
   HELM_LAUNCH_GRAPH = 1,      /* CUDA graph with a device-driven while node;
                                  HELM_ERR_CUDA if it cannot be built */
   HELM_LAUNCH_PERSISTENT = 2, /* FP64 BiCGStab only (HELM_ERR_INVALID for
@@ -214,9 +217,11 @@ typedef enum {
                                  cooperative kernel whose phases are separated
                                  by grid barriers; the same arithmetic as the
                                  graph, bit for bit.  Every barrier wait gives
-                                 up after 2 s: the block sets a device error
-                                 flag of the handle, every block leaves the
-                                 kernel, and the solve returns HELM_ERR_CUDA.
+                                 up after a fixed number of polls (at least 2 s
+                                 of the kernel's running time): the block sets
+                                 a device error flag of the handle, every block
+                                 leaves the kernel, and the solve returns
+                                 HELM_ERR_CUDA.
                                  Every solve clears that flag when it starts,
                                  so a later solve on the handle is unaffected;
                                  helm_spmv has no waits and never sets it.
@@ -248,7 +253,9 @@ typedef struct {
                           most tol; when the recurrence met tol but the
                           recomputed residual did not, the solve restarts
                           from the current x while iterations remain
-                          (BiCGStab, BiCGStab(l), TFQMR) */
+                          (BiCGStab, BiCGStab(l), TFQMR); FP64 BiCGStab
+                          also when (r^, r) of its recurrence came to exactly
+                          zero after an iteration */
   int32_t maxit;       /* iteration cap (Section 4 uses 1000); each BiCGStab
                           or TFQMR iteration applies A twice */
   int32_t use_x0;      /* 0: start from x = 0 (Section 4); 1: start from d_x */

@@ -55,8 +55,9 @@ __device__ __forceinline__ double cabs2_acc(double2 a, double acc) {
   acc = fma(a.x, a.x, acc);
   return fma(a.y, a.y, acc);
 }
-__device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-  // Smith's algorithm (Smith 1962) for robustness against overflow.
+__device__ __noinline__ inline double2 cdiv(double2 a, double2 b) {
+  // Smith's algorithm (Smith 1962) for robustness against overflow.  Out of
+  // line: most callers reach it only when |b|^2 under- or overflows.
   if (fabs(b.x) >= fabs(b.y)) {
     double r = b.y / b.x, d = b.x + b.y * r;
     return make_double2((a.x + a.y * r) / d, (a.y - a.x * r) / d);
@@ -65,13 +66,18 @@ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
     return make_double2((a.x * r + a.y) / d, (a.y * r - a.x) / d);
   }
 }
+// Division and square root of the scalar steps, out of line: inlined, they make
+// up most of a solver kernel's code (each a kilobyte at every use), which has
+// to stay in the instruction cache.
+__device__ __noinline__ inline double sc_div(double a, double b) { return a / b; }
+__device__ __noinline__ inline double sc_sqrt(double a) { return sqrt(a); }
 // a / b with one real division: a conj(b) / |b|^2 (the scalar recurrences run
 // in one thread between kernels, where every dependent division is latency);
 // Smith's algorithm when |b|^2 under- or overflows.
 __device__ __forceinline__ double2 cdiv_fast(double2 a, double2 b) {
   const double d = fma(b.x, b.x, b.y * b.y);
   if (!(d > 0.0) || !isfinite(d) || d < 1e-290) return cdiv(a, b);
-  const double inv = 1.0 / d;
+  const double inv = sc_div(1.0, d);
   return make_double2(fma(a.x, b.x, a.y * b.y) * inv, fma(a.y, b.x, -a.x * b.y) * inv);
 }
 __device__ __forceinline__ bool cfinite(double2 a) { return isfinite(a.x) && isfinite(a.y); }

@@ -38,6 +38,7 @@
 
 #include "common.cuh"
 #include "internal.hpp"
+#include "persist.cuh"
 #include "spmv.cuh"
 
 namespace helm {
@@ -98,7 +99,35 @@ __device__ __forceinline__ double nrm_acc(double acc, float2 a) {
   return acc + static_cast<double>(fmaf(a.x, a.x, a.y * a.y));
 }
 
-// Every kernel of the solver: at most 1024 threads, one block per SM.
+// Solver shapes, by the slices of the mesh per SM (krylov_shapes).  The shape
+// fixes which thread owns which row, in how many parts a row is summed, and so
+// the rounding of every reduction: every form of a solve takes the same one, and
+// it depends on nothing but the size, so that a solve gives the same bits on
+// every run.
+//   small: one block per SM; a row is summed in kParts parts, which the
+//          persistent kernel gives to three warps;
+//   mid:   one block per SM of at most 640 threads (96 registers a thread);
+//   large: two blocks per SM of at most 512 threads (64 registers).
+// complex64 (the inner solves of mixed precision): mid or large (us per inner
+// iteration, persistent / before: 20^3 29.9 / 44.5, 60x30x25 29.7 / 37.1,
+// 80x40x32 38.4 / 47, 120x60x50 70.2 / 77.9, 200x100x80 192.7 / 204.8).
+// Measured (BiCGStab, us per iteration: persistent / graph kernels; before, on
+// one shape with graph kernels):
+//   20^3 box      (2 slices per SM)  small 25.7 / 42.8                       (39.7)
+//   60x30x25      (10)               mid   37.7 / 39.0, large 50.1 / 47.6    (43.6)
+//   80x40x32      (23)               mid   57.1 / 59.4, large 60.0 / 67.0    (65.1)
+//   120x60x50     (77)               mid  122.0 / 136.2, large 135.4 / 140.2 (134.0)
+//   200x100x80    (338)              mid  504 (512 threads), large 470 / 500 (478)
+enum : int { SHAPE_SMALL = 0, SHAPE_MID = 1, SHAPE_LARGE = 2 };
+constexpr int kMidSlices = 150;  // slices per SM from which the shape is large
+template <int S> struct SolverBounds {
+  static constexpr int threads = S == SHAPE_SMALL ? 384 : S == SHAPE_MID ? 640 : 512;  // warps of a split persistent kernel included
+  static constexpr int blocks = S == SHAPE_LARGE ? 2 : 1;
+  static constexpr int parts = S == SHAPE_SMALL ? kParts : 1;
+  // entries per pipeline stage of the persistent kernel's products
+  static constexpr int persist_u = S == SHAPE_LARGE ? 2 : 3;
+};
+// The other kernels on an SpMV grid (init, tail, refinement steps).
 constexpr int kSolverThreads = Engine<double2>::kThreads;
 constexpr int kSolverMinBlocks = Engine<double2>::kMinBlocks;
 
@@ -153,40 +182,123 @@ __device__ __forceinline__ void pdl_enter() {
 
 // ---------------------------------------------------------------- reductions
 
-// Fixed-order total of the block partials partials[b K + k], b < G: thread j
-// adds blocks j, j + T, j + 2T, ... in that order, then the fixed block tree.
-// Valid in thread 0.
-template <int K>
+// Two orders of a grid's sums.  One is chosen for latency (a dependent FP64 add
+// is 64 clocks): trees over warps and blocks with the components side by side
+// on the warps; partials: component k of block b at k G + b (every block of a
+// persistent solve reads them all: neighbours share a sector).  The other, for
+// complex64 on the large shape: warps in order, then blocks in thread order;
+// whether the inner solves of mixed precision converge on a strongly indefinite
+// system of that size (200x100x80 at 10 points per wavelength) hangs on the last
+// bits of these sums, so their order stays.
+template <class V, int S>
+constexpr bool kOrderedSums = std::is_same<V, float2>::value && S == SHAPE_LARGE;
+
+// Sums of the first `width` lanes (a power of two) into lane 0, in the order
+// that the pattern fixes.
+__device__ __forceinline__ double lanes_sum(double v, int width) {
+#pragma unroll 1
+  for (int off = width >> 1; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
+// This block's K sums into its partials (global memory; a barrier of the block
+// or a fence has to follow).  `red` holds 32 * K doubles.
+template <class V, int S, int K>
+__device__ __forceinline__ void put_block_partials(double (&v)[K], double* red, double* partials) {
+  if constexpr (kOrderedSums<V, S>) {
+    block_sum<K>(v, red);
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int k = 0; k < K; ++k) partials[static_cast<size_t>(blockIdx.x) * K + k] = v[k];
+  } else {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = static_cast<int>(blockDim.x >> 5);
+    const double ws = warp_sum_t<K>(v);
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (lane == warp_sum_lane<K>(k)) red[warp * K + k] = ws;
+    __syncthreads();
+    const int width = nwarps > 1 ? 1 << (32 - __clz(nwarps - 1)) : 1;
+#pragma unroll 1
+    for (int k = warp; k < K; k += nwarps) {
+      const double s = lanes_sum(lane < nwarps ? red[lane * K + k] : 0.0, width);
+      if (lane == 0) partials[static_cast<size_t>(k) * gridDim.x + blockIdx.x] = s;
+    }
+  }
+}
+
+// Fixed-order totals of all blocks' partials, valid in thread 0: one warp per
+// component, lane j adds blocks j, j + 32, j + 64, ... (five loaded at a time) in
+// that order, then the lanes' tree; or thread j adds blocks j, j + T, ..., then
+// the block tree.
+template <class V, int S, int K>
 __device__ __forceinline__ void sum_block_partials(const double* partials, int G, double* red, double (&tot)[K]) {
-  double acc[K];
+  if constexpr (kOrderedSums<V, S>) {
+    double acc[K];
 #pragma unroll
-  for (int k = 0; k < K; ++k) acc[k] = 0.0;
-  for (int b = threadIdx.x; b < G; b += blockDim.x)
+    for (int k = 0; k < K; ++k) acc[k] = 0.0;
+    for (int b = threadIdx.x; b < G; b += blockDim.x)
 #pragma unroll
-    for (int k = 0; k < K; ++k) acc[k] += ld_cg(&partials[static_cast<size_t>(b) * K + k]);
-  block_sum<K>(acc, red);
+      for (int k = 0; k < K; ++k) acc[k] += ld_cg(&partials[static_cast<size_t>(b) * K + k]);
+    block_sum<K>(acc, red);
 #pragma unroll
-  for (int k = 0; k < K; ++k) tot[k] = acc[k];
+    for (int k = 0; k < K; ++k) tot[k] = acc[k];
+  } else {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = static_cast<int>(blockDim.x >> 5);
+    __shared__ double out[K];
+#pragma unroll 1
+    for (int k = warp; k < K; k += nwarps) {
+      double acc = 0.0;
+#pragma unroll 1
+      for (int j0 = lane; j0 < G; j0 += 5 * 32) {
+        double w[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+          w[u] = j0 + 32 * u < G ? ld_cg(&partials[static_cast<size_t>(k) * G + j0 + 32 * u]) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+          if (j0 + 32 * u < G) acc += w[u];
+      }
+      acc = lanes_sum(acc, 32);
+      if (lane == 0) out[k] = acc;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int k = 0; k < K; ++k) tot[k] = out[k];
+    }
+  }
 }
 
 // Graph path: publish this block's K sums; the last block to arrive forms
 // the totals (valid in its thread 0) and returns true.
-template <int K>
+template <class V, int S, int K>
 __device__ __forceinline__ bool grid_total_last(double (&v)[K], double* partials, unsigned int* ticket, double* red,
                                                 double (&tot)[K]) {
   __shared__ bool s_last;
-  block_sum<K>(v, red);
+  put_block_partials<V, S, K>(v, red, partials);
+  __syncthreads();
   if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) partials[static_cast<size_t>(blockIdx.x) * K + k] = v[k];
     __threadfence();
     s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
   __syncthreads();
   if (!s_last) return false;
   __threadfence();
-  sum_block_partials<K>(partials, gridDim.x, red, tot);
+  sum_block_partials<V, S, K>(partials, gridDim.x, red, tot);
   if (threadIdx.x == 0) *ticket = 0u;
+  return true;
+}
+
+// Persistent path: publish this block's K sums, wait for every block, add all
+// blocks' sums in the same order (every block the same), totals valid in
+// thread 0; false when the barrier gave up.
+template <class V, int S, int K>
+__device__ __forceinline__ bool grid_total_all(double (&v)[K], double* partials, unsigned int* tickets,
+                                               unsigned int* dev_err, unsigned int* target, double* red,
+                                               double (&tot)[K]) {
+  put_block_partials<V, S, K>(v, red, partials);
+  if (!grid_barrier(tickets, dev_err, target)) return false;
+  sum_block_partials<V, S, K>(partials, gridDim.x, red, tot);
   return true;
 }
 
@@ -200,19 +312,21 @@ __device__ __forceinline__ bool grid_total_last(double (&v)[K], double* partials
 // poor or non-finite inner iterate is rejected there, and a fresh inner
 // process starts from the FP64 residual).  Returns true when the event was
 // absorbed that way; the caller then leaves the status running.
+template <class V>
 __device__ __forceinline__ bool refine_absorb(SolverState* st) {
-  if (st->method != kModeRefine) return false;
+  if (std::is_same<V, double2>::value || st->method != kModeRefine) return false;
   st->aux[1].x = 1.0;
   return true;
 }
 // A refinement step is pending: the rest of the inner iteration is skipped.
+template <class V>
 __device__ __forceinline__ bool refine_step_pending(const SolverState* st) {
-  return st->method == kModeRefine && st->aux[1].x != 0.0;
+  return !std::is_same<V, double2>::value && st->method == kModeRefine && st->aux[1].x != 0.0;
 }
 
 // after the initial residual: tot = (||b||^2, ||r||^2, (r^, r))
 __device__ __forceinline__ void sc_init(SolverState* st, const double (&tot)[4], int use_x0) {
-  const double bnorm = sqrt(tot[0]);
+  const double bnorm = sc_sqrt(tot[0]);
   st->bnorm = bnorm;
   if (use_x0) st->spmv_count += 1;
   int status = ST_RUNNING;
@@ -222,7 +336,7 @@ __device__ __forceinline__ void sc_init(SolverState* st, const double (&tot)[4],
     status = HELM_OK;  // b = 0: x = 0 (written by the tail)
     st->relres = 0.0;
   } else {
-    const double relres = sqrt(tot[1]) / bnorm;
+    const double relres = sc_div(sc_sqrt(tot[1]), bnorm);
     st->relres = relres;
     const double2 rho = make_double2(tot[2], tot[3]);
     if (!isfinite(relres)) {
@@ -250,6 +364,7 @@ __device__ __forceinline__ void sc_init(SolverState* st, const double (&tot)[4],
 }
 
 // after P2: tot = (r^, v)
+template <class V>
 __device__ __forceinline__ void sc_after_v(SolverState* st, const double (&tot)[2]) {
   st->iter += 1;
   st->spmv_count += 1;
@@ -264,22 +379,24 @@ __device__ __forceinline__ void sc_after_v(SolverState* st, const double (&tot)[
     if (!cfinite(alpha)) err = HELM_ERR_NONFINITE;
     else st->alpha = alpha;
   }
-  if (err && !refine_absorb(st)) st->status = err;
+  if (err && !refine_absorb<V>(st)) st->status = err;
 }
 
 // after P3: tot = ||s||^2; ||s|| / ||b|| <= tol compared squared
+template <class V>
 __device__ __forceinline__ void sc_after_s(SolverState* st, const double (&tot)[1]) {
   const double s2 = tot[0];
   const double bt = st->bnorm * st->tol;
   if (!isfinite(s2)) {
-    if (!refine_absorb(st)) st->status = HELM_ERR_NONFINITE;
-  } else if (st->method != kModeRefine && s2 <= bt * bt) {
+    if (!refine_absorb<V>(st)) st->status = HELM_ERR_NONFINITE;
+  } else if ((std::is_same<V, double2>::value || st->method != kModeRefine) && s2 <= bt * bt) {
     st->phase = PH_SCONV;
-    st->relres = sqrt(s2) / st->bnorm;
+    st->relres = sc_div(sc_sqrt(s2), st->bnorm);
   }
 }
 
 // after P4: tot = ((t, s), ||t||^2)
+template <class V>
 __device__ __forceinline__ void sc_after_t(SolverState* st, const double (&tot)[3]) {
   st->spmv_count += 1;
   const double2 ts = make_double2(tot[0], tot[1]);
@@ -290,19 +407,21 @@ __device__ __forceinline__ void sc_after_t(SolverState* st, const double (&tot)[
   } else if (tt == 0.0) {
     err = HELM_ERR_BREAKDOWN;
   } else {
-    const double inv_tt = 1.0 / tt;
+    const double inv_tt = sc_div(1.0, tt);
     const double2 omega = make_double2(ts.x * inv_tt, ts.y * inv_tt);
     if (!cfinite(omega)) err = HELM_ERR_NONFINITE;
     else st->omega = omega;
   }
-  if (err && !refine_absorb(st)) st->status = err;
+  if (err && !refine_absorb<V>(st)) st->status = err;
 }
 
 // after P5: tot = ((r^, r), ||r||^2); `late` = the deadline has passed.
 // With phase PH_SCONV (P5 only added alpha p to x) the solve is done.
+template <class V>
 __device__ __forceinline__ void sc_after_xr(SolverState* st, const double (&tot)[3], bool late) {
   // the inner loop of mixed precision runs on a scaled residual: b - A x ~ aux[2].x * r
-  const double sc = st->method == kModeRefine ? st->aux[2].x : 1.0;
+  constexpr bool plain = std::is_same<V, double2>::value;
+  const double sc = !plain && st->method == kModeRefine ? st->aux[2].x : 1.0;
   const int phase = st->phase;
   const double2 alpha64 = st->alpha, omega64 = st->omega;
   int status = ST_RUNNING;
@@ -315,25 +434,25 @@ __device__ __forceinline__ void sc_after_xr(SolverState* st, const double (&tot)
     const double r2 = tot[2];
     const double bt = st->bnorm * st->tol;
     bool stop_ok = r2 * (sc * sc) <= bt * bt;
-    if (st->method == kModeRefine && isfinite(r2)) {
+    if (!plain && st->method == kModeRefine && isfinite(r2)) {
       // mixed precision: the recurrence never declares convergence; it asks
       // for a refinement step (FP64 residual, fresh process) when it has
       // dropped by inner_tol since the process began, looks converged, or
       // after kInnerMax iterations (complex64 BiCGStab can stagnate on
       // strongly indefinite systems; the step's minimal-residual length
       // keeps a poor inner iterate from increasing the FP64 residual)
-      const double rn = sqrt(r2);
+      const double rn = sc_sqrt(r2);
       const double cyc = st->aux[3].y;
       const bool dropped = cyc > 0.0 && cyc < 1.0 && rn <= cyc * st->aux[0].x;
       if (stop_ok || dropped || st->iter - static_cast<int>(st->aux[0].y) >= kInnerMax) st->aux[1].x = 1.0;
       stop_ok = false;
     }
     if (!isfinite(r2)) {
-      status = refine_absorb(st) ? ST_RUNNING : HELM_ERR_NONFINITE;
+      status = refine_absorb<V>(st) ? ST_RUNNING : HELM_ERR_NONFINITE;
     } else if (stop_ok) {
       status = HELM_OK;
     } else if (czero(omega64)) {
-      status = refine_absorb(st) ? ST_RUNNING : HELM_ERR_BREAKDOWN;
+      status = refine_absorb<V>(st) ? ST_RUNNING : HELM_ERR_BREAKDOWN;
     } else if (st->iter >= st->maxit) {
       status = HELM_ERR_NOT_CONVERGED;
     } else if (late) {
@@ -343,325 +462,397 @@ __device__ __forceinline__ void sc_after_xr(SolverState* st, const double (&tot)
       // beta = (rho_new / rho) (alpha / omega) = (rho_new alpha) / (rho omega)
       const double2 beta = cdiv_fast(cmul(rho_new, alpha64), cmul(st->rho, omega64));
       if (!cfinite(rho_new) || !cfinite(beta)) {
-        status = refine_absorb(st) ? ST_RUNNING : HELM_ERR_NONFINITE;
+        status = refine_absorb<V>(st) ? ST_RUNNING : HELM_ERR_NONFINITE;
         st->iter += 1;
       } else if (czero(rho_new)) {
-        status = refine_absorb(st) ? ST_RUNNING : HELM_ERR_BREAKDOWN;
+        // (r^, r) has sunk below the rounding of its terms and they cancelled:
+        // the process can go no further, x and r stand.  Start again from x
+        // (r^ = r); what is left in (r^, r) at such a point, zero or not, is the
+        // luck of the order of the sum.
+        status = refine_absorb<V>(st) ? ST_RUNNING : ST_RESTART;
         st->iter += 1;
       } else {
         st->rho = rho_new;
         st->beta = beta;
       }
     }
-    if (status != ST_RUNNING) st->relres = sqrt(tot[2]) * sc / st->bnorm;
+    if (status != ST_RUNNING) st->relres = sc_div(sc_sqrt(tot[2]) * sc, st->bnorm);
   }
   st->status = status;
 }
 
+// after the tail: tot = ||b - A x||^2
+__device__ __forceinline__ void sc_tail(SolverState* st, const double (&tot)[1]) {
+  if (st->bnorm == 0.0) {
+    st->relres_true = 0.0;
+  } else {
+    st->relres_true = sc_div(sc_sqrt(tot[0]), st->bnorm);
+    st->spmv_count += 1;
+  }
+}
+
+// After the tail: the recurrence converged but the true residual did not, or
+// (r^, r) vanished; the solve starts again from x while iterations remain.
+__host__ __device__ __forceinline__ bool restart_due(SolverState* st) {
+  if (st->status == ST_RESTART && st->relres_true <= st->tol) st->status = HELM_OK;
+  if (st->status == ST_RESTART && st->iter >= st->maxit) st->status = HELM_ERR_NOT_CONVERGED;
+  return st->status == ST_RESTART || (st->status == HELM_OK && st->relres_true > st->tol && st->iter < st->maxit);
+}
+
 // ---------------------------------------------------------------- phases
 // The per-thread work of each phase, shared by the graph kernels and the
-// persistent kernel.  Rows are those of SliceRows; each phase returns this
-// thread's partial sums.
-
-// init without x0: x = 0, r = r^ = b, p = v = 0; (||b||^2, ||r||^2, (r^, r))
+// persistent kernels; each returns this thread's partial sums.  Rows are those
+// of SliceRows.
 template <class V>
-__device__ __forceinline__ void ph_init_zero(const KArgs<V>& a, typename Prec<V>::S (&acc)[2],
-                                             typename Prec<V>::C& d) {
-  const V z = vzero<V>();
-  for (SliceRows q(a.A.n); q.active(); q.advance()) {
-    const int32_t i = q.row();
-    if (i >= a.A.n) continue;
-    const V bi = a.b[i];
-    a.x[i] = z;
-    a.r[i] = bi;
-    a.rh[i] = bi;
-    a.p[i] = z;
-    a.v[i] = z;
-    acc[0] = nrm_acc(acc[0], bi);
-    d = dot_acc(d, bi, bi);
-  }
-  acc[1] = acc[0];
-}
+struct Phases {
+  const KArgs<V>& a;
+  PRows q;
+  Own<V, 0> v;
+  Own<V, 1> r;
+  Own<V, 2> t;
+  Own<V, 3> rh;
+  Own<V, 4> x;
+  Own<V, 5> p;  // p and s: a copy beside the one that is gathered
+  Own<V, 6> s;
+  static constexpr int kOwn = 7;
+  __device__ __forceinline__ Phases(const KArgs<V>& a_, const PLayout& L)
+      : a(a_), q(L), v{a_.v, L}, r{a_.r, L}, t{a_.t, L}, rh{a_.rh, L}, x{a_.x, L}, p{a_.p, L}, s{a_.s, L} {}
 
-// init with x0 (SpMV epilogue): r = r^ = b - A x, p = v = 0
-template <class V>
-struct InitEpi {
-  const V* b;
-  V *r, *rh, *p, *v;
-  typename Prec<V>::S part[2];
-  typename Prec<V>::C d;
-  V bpre;
-  __device__ __forceinline__ void prefetch(int32_t i) { bpre = b[i]; }
-  __device__ __forceinline__ void row(int32_t i, V ax) {
-    const V bi = bpre;
-    const V ri = csub(bi, ax);
-    r[i] = ri;
-    rh[i] = ri;
-    p[i] = vzero<V>();
-    v[i] = vzero<V>();
+  __device__ __forceinline__ int32_t n() const { return a.A.n; }
+
+  // r = r^ = ri, p = v = 0 on row i; (||b||^2, ||r||^2, (r^, r))
+  __device__ __forceinline__ void init_row(int32_t i, int li, V bi, V ri, double (&part)[4]) const {
+    const V z = vzero<V>();
+    r.st(i, li, ri);
+    rh.st(i, li, ri);
+    p.st(i, li, z);
+    v.st(i, li, z);
     part[0] = nrm_acc(part[0], bi);
     part[1] = nrm_acc(part[1], ri);
-    d = dot_acc(d, ri, ri);
+    const double2 d = dot_acc(make_double2(part[2], part[3]), ri, ri);
+    part[2] = d.x;
+    part[3] = d.y;
+  }
+  // without x0: x = 0, r = b
+  __device__ __forceinline__ void init_zero(double (&part)[4]) const {
+    for_rows(q, n(), [&](int32_t i, int li) {
+      const V bi = a.b[i];
+      x.st(i, li, vzero<V>());
+      init_row(i, li, bi, bi, part);
+    });
+  }
+  // with x0: r = b - A x
+  __device__ __forceinline__ void row_init(int32_t i, int li, V ax, double (&part)[4]) const {
+    const V bi = a.b[i];
+    if (x.shared()) x.st(i, li, a.x[i]);
+    init_row(i, li, bi, csub(bi, ax), part);
+  }
+
+  // P1: p = r + beta (p - omega v)
+  __device__ __forceinline__ void upd_p(V beta, V omega) const {
+    for_rows(q, n(), [&](int32_t i, int li) {
+      p.st_both(i, li, cfma(beta, cfms(omega, v.ld(i, li), p.ld(i, li)), r.ld(i, li)));
+    });
+  }
+
+  // P2: v = A p, (r^, v)
+  __device__ __forceinline__ void row_v(int32_t i, int li, V rhi, V ax, double (&part)[4]) const {
+    v.st(i, li, ax);
+    const double2 d = dot_acc(make_double2(part[0], part[1]), rhi, ax);
+    part[0] = d.x;
+    part[1] = d.y;
+  }
+
+  // P3: s = r - alpha v, ||s||^2
+  __device__ __forceinline__ void upd_s(V alpha, double (&part)[4]) const {
+    for_rows(q, n(), [&](int32_t i, int li) {
+      const V sn = cfms(alpha, v.ld(i, li), r.ld(i, li));
+      s.st_both(i, li, sn);
+      part[0] = nrm_acc(part[0], sn);
+    });
+  }
+
+  // P4: t = A s, (t, s), ||t||^2
+  __device__ __forceinline__ void row_t(int32_t i, int li, V si, V ax, double (&part)[4]) const {
+    t.st(i, li, ax);
+    const double2 d = dot_acc(make_double2(part[0], part[1]), ax, si);
+    part[0] = d.x;
+    part[1] = d.y;
+    part[2] = nrm_acc(part[2], ax);
+  }
+
+  // P5: x += alpha p + omega s, r = s - omega t; (r^, r), ||r||^2.  With sconv
+  // (the solve stopped at s) only x += alpha p.
+  __device__ __forceinline__ void upd_xr(V alpha, V omega, bool sconv, double (&part)[4]) const {
+    if (sconv) {
+      for_rows(q, n(), [&](int32_t i, int li) { x.st(i, li, cfma(alpha, p.ld(i, li), x.ld(i, li))); });
+      return;
+    }
+    for_rows(q, n(), [&](int32_t i, int li) {
+      const V si = s.ld(i, li);
+      x.st(i, li, cfma(omega, si, cfma(alpha, p.ld(i, li), x.ld(i, li))));
+      const V ri = cfms(omega, t.ld(i, li), si);
+      r.st(i, li, ri);
+      const double2 d = dot_acc(make_double2(part[0], part[1]), rh.ld(i, li), ri);
+      part[0] = d.x;
+      part[1] = d.y;
+      part[2] = nrm_acc(part[2], ri);
+    });
   }
 };
-template <class V>
-__device__ __forceinline__ InitEpi<V> init_epi(const KArgs<V>& a) {
-  return InitEpi<V>{a.b, a.r, a.rh, a.p, a.v, {Prec<V>::szero(), Prec<V>::szero()}, Prec<V>::czero(), vzero<V>()};
-}
-
-// P1: p = r + beta (p - omega v); the next row's loads are issued before
-// this row is computed
-template <class V>
-__device__ __forceinline__ void ph_p(const KArgs<V>& a, V beta, V omega) {
-  SliceRows q(a.A.n);
-  int32_t i = q.row();
-  if (!q.active() || i >= a.A.n) return;
-  V v0 = a.v[i], p0 = a.p[i], r0 = a.r[i];
-  for (;;) {
-    SliceRows nq = q;
-    const bool more = nq.advance() && nq.row() < a.A.n;
-    const int32_t j = nq.row();
-    V v1 = v0, p1 = p0, r1 = r0;
-    if (more) {
-      v1 = a.v[j];
-      p1 = a.p[j];
-      r1 = a.r[j];
-    }
-    a.p[i] = cfma(beta, cfms(omega, v0, p0), r0);
-    if (!more) break;
-    v0 = v1;
-    p0 = p1;
-    r0 = r1;
-    i = j;
-    q = nq;
-  }
-}
-
-// P2 epilogue: v = A p, (r^, v)
-template <class V>
-struct VEpi {
-  V* v;
-  const V* rhp;
-  typename Prec<V>::C part;
-  V rh;
-  __device__ __forceinline__ void prefetch(int32_t i) { rh = rhp[i]; }
-  __device__ __forceinline__ void row(int32_t i, V ax) {
-    v[i] = ax;
-    part = dot_acc(part, rh, ax);
-  }
-};
-template <class V>
-__device__ __forceinline__ VEpi<V> v_epi(const KArgs<V>& a) {
-  return VEpi<V>{a.v, a.rh, Prec<V>::czero(), vzero<V>()};
-}
-
-// P3: s = r - alpha v, ||s||^2
-template <class V>
-__device__ __forceinline__ typename Prec<V>::S ph_s(const KArgs<V>& a, V alpha) {
-  using S = typename Prec<V>::S;
-  S acc = Prec<V>::szero();
-  SliceRows q(a.A.n);
-  int32_t i = q.row();
-  if (!q.active() || i >= a.A.n) return acc;
-  V v0 = a.v[i], r0 = a.r[i];
-  for (;;) {
-    SliceRows nq = q;
-    const bool more = nq.advance() && nq.row() < a.A.n;
-    const int32_t j = nq.row();
-    V v1 = v0, r1 = r0;
-    if (more) {
-      v1 = a.v[j];
-      r1 = a.r[j];
-    }
-    const V s0 = cfms(alpha, v0, r0);
-    a.s[i] = s0;
-    acc = nrm_acc(acc, s0);
-    if (!more) break;
-    v0 = v1;
-    r0 = r1;
-    i = j;
-    q = nq;
-  }
-  return acc;
-}
-
-// P4 epilogue: t = A s, (t, s), ||t||^2
-template <class V>
-struct TEpi {
-  V* t;
-  const V* sp;
-  typename Prec<V>::C ts;
-  typename Prec<V>::S tt;
-  V si;
-  __device__ __forceinline__ void prefetch(int32_t i) { si = sp[i]; }
-  __device__ __forceinline__ void row(int32_t i, V ax) {
-    t[i] = ax;
-    ts = dot_acc(ts, ax, si);
-    tt = nrm_acc(tt, ax);
-  }
-};
-template <class V>
-__device__ __forceinline__ TEpi<V> t_epi(const KArgs<V>& a) {
-  return TEpi<V>{a.t, a.s, Prec<V>::czero(), Prec<V>::szero(), vzero<V>()};
-}
-
-// P5: x += alpha p + omega s, r = s - omega t; (r^, r), ||r||^2.  With
-// sconv (the solve stopped at s) only x += alpha p.
-template <class V>
-__device__ __forceinline__ void ph_xr(const KArgs<V>& a, V alpha, V omega, bool sconv, typename Prec<V>::C& rr,
-                                      typename Prec<V>::S& r2) {
-  SliceRows q(a.A.n);
-  int32_t i = q.row();
-  if (!q.active() || i >= a.A.n) return;
-  if (sconv) {
-    for (; q.active(); q.advance()) {
-      i = q.row();
-      if (i < a.A.n) a.x[i] = cfma(alpha, a.p[i], a.x[i]);
-    }
-    return;
-  }
-  V s0 = a.s[i], x0 = a.x[i], p0 = a.p[i], t0 = a.t[i], h0 = a.rh[i];
-  for (;;) {
-    SliceRows nq = q;
-    const bool more = nq.advance() && nq.row() < a.A.n;
-    const int32_t j = nq.row();
-    V sn = s0, xn = x0, pn = p0, tn = t0, hn = h0;
-    if (more) {
-      sn = a.s[j];
-      xn = a.x[j];
-      pn = a.p[j];
-      tn = a.t[j];
-      hn = a.rh[j];
-    }
-    a.x[i] = cfma(omega, s0, cfma(alpha, p0, x0));
-    const V r0 = cfms(omega, t0, s0);
-    a.r[i] = r0;
-    rr = dot_acc(rr, h0, r0);
-    r2 = nrm_acc(r2, r0);
-    if (!more) break;
-    s0 = sn;
-    x0 = xn;
-    p0 = pn;
-    t0 = tn;
-    h0 = hn;
-    i = j;
-    q = nq;
-  }
-}
 
 // ---------------------------------------------------------------- graph kernels
 
-template <class V>
-__global__ void __launch_bounds__(kSolverThreads, kSolverMinBlocks) k_init(KArgs<V> a) {
+// no shared memory: the rounds of the grid, whose blocks' warps all own rows
+__device__ __forceinline__ PLayout graph_layout(int32_t n) {
+  const int32_t wb = static_cast<int32_t>(blockDim.x >> 5), W = static_cast<int32_t>(gridDim.x) * wb;
+  PLayout L = {};
+  L.rounds = ((n + 31) / 32 + W - 1) / W;
+  L.split = 1;
+  L.warps = wb;
+  return L;
+}
+template <class V, int S, class Pre, class F>
+__device__ __forceinline__ void graph_spmv(const Phases<V>& ph, const V* x, Pre pre, F f) {
+  spmv_rows<V, kSpmvUnroll, SolverBounds<S>::parts, GatherReadOnly>(ph.q, ph.a.A, x, pre, f);
+}
+
+#define HELM_SOLVER_KERNEL __global__ void __launch_bounds__(SolverBounds<S>::threads, SolverBounds<S>::blocks)
+#define HELM_GRAPH_PHASES                     \
+  const PLayout lay = graph_layout(a.A.n);    \
+  const Phases<V> ph(a, lay);                 \
+  double part[4] = {0.0, 0.0, 0.0, 0.0};
+
+template <class V, int S>
+HELM_SOLVER_KERNEL k_init(const __grid_constant__ KArgs<V> a) {
   pdl_enter();
-  using S = typename Prec<V>::S;
-  using C = typename Prec<V>::C;
   __shared__ double red[32 * 4];
   SolverState* st = a.st;
   const int use_x0 = st->use_x0;
-  S acc[2] = {Prec<V>::szero(), Prec<V>::szero()};
-  C d = Prec<V>::czero();
+  HELM_GRAPH_PHASES
   if (use_x0) {
-    InitEpi<V> epi = init_epi<V>(a);
-    spmv_run<V>(a.A, a.x, epi, nullptr, a.dev_err);
-    acc[0] = epi.part[0];
-    acc[1] = epi.part[1];
-    d = epi.d;
+    graph_spmv<V, S>(
+        ph, a.x, [](int32_t) {}, [&](int32_t i, int li, V ax) { ph.row_init(i, li, ax, part); });
   } else {
-    ph_init_zero<V>(a, acc, d);
+    ph.init_zero(part);
   }
-  const double2 dd = to_d2(d);
-  double part[4] = {to_d(acc[0]), to_d(acc[1]), dd.x, dd.y};
   double tot[4];
-  if (!grid_total_last<4>(part, a.partials, a.tickets + TK_INIT, red, tot)) return;
+  if (!grid_total_last<V, S, 4>(part, a.partials, a.tickets + TK_INIT, red, tot)) return;
   if (threadIdx.x != 0) return;
   sc_init(st, tot, use_x0);
   set_cond(a, st->status == ST_RUNNING);
 }
 
 // K1: p = r + beta (p - omega v)
-template <class V>
-__global__ void __launch_bounds__(kSolverThreads, kSolverMinBlocks) k_p(KArgs<V> a) {
+template <class V, int S>
+HELM_SOLVER_KERNEL k_p(const __grid_constant__ KArgs<V> a) {
   pdl_enter();
   const SolverState* st = a.st;
-  if (st->status != ST_RUNNING || refine_step_pending(st)) return;
-  ph_p<V>(a, Prec<V>::cvt(st->beta), Prec<V>::cvt(st->omega));
+  if (st->status != ST_RUNNING || refine_step_pending<V>(st)) return;
+  const PLayout lay = graph_layout(a.A.n);
+  Phases<V>(a, lay).upd_p(Prec<V>::cvt(st->beta), Prec<V>::cvt(st->omega));
 }
 
 // K2: v = A p, (r^, v) -> alpha
-template <class V>
-__global__ void __launch_bounds__(kSolverThreads, kSolverMinBlocks) k_v(KArgs<V> a) {
+template <class V, int S>
+HELM_SOLVER_KERNEL k_v(const __grid_constant__ KArgs<V> a) {
   pdl_enter();
   __shared__ double red[32 * 2];
   SolverState* st = a.st;
-  if (st->status != ST_RUNNING || refine_step_pending(st)) return;
-  VEpi<V> epi = v_epi<V>(a);
-  spmv_run<V>(a.A, a.p, epi, nullptr, a.dev_err);
-  const double2 pd = to_d2(epi.part);
-  double part[2] = {pd.x, pd.y};
-  double tot[2];
-  if (!grid_total_last<2>(part, a.partials, a.tickets + TK_V, red, tot)) return;
+  if (st->status != ST_RUNNING || refine_step_pending<V>(st)) return;
+  HELM_GRAPH_PHASES
+  V rhi = vzero<V>();
+  graph_spmv<V, S>(
+      ph, a.p, [&](int32_t i) { rhi = a.rh[i]; }, [&](int32_t i, int li, V ax) { ph.row_v(i, li, rhi, ax, part); });
+  double part2[2] = {part[0], part[1]}, tot[2];
+  if (!grid_total_last<V, S, 2>(part2, a.partials, a.tickets + TK_V, red, tot)) return;
   if (threadIdx.x != 0) return;
-  sc_after_v(st, tot);
+  sc_after_v<V>(st, tot);
 }
 
 // K3: s = r - alpha v, ||s||
-template <class V>
-__global__ void __launch_bounds__(kSolverThreads, kSolverMinBlocks) k_s(KArgs<V> a) {
+template <class V, int S>
+HELM_SOLVER_KERNEL k_s(const __grid_constant__ KArgs<V> a) {
   pdl_enter();
   __shared__ double red[32];
   SolverState* st = a.st;
-  if (st->status != ST_RUNNING || refine_step_pending(st)) return;
-  double part[1] = {to_d(ph_s<V>(a, Prec<V>::cvt(st->alpha)))};
-  double tot[1];
-  if (!grid_total_last<1>(part, a.partials, a.tickets + TK_S, red, tot)) return;
+  if (st->status != ST_RUNNING || refine_step_pending<V>(st)) return;
+  HELM_GRAPH_PHASES
+  ph.upd_s(Prec<V>::cvt(st->alpha), part);
+  double part1[1] = {part[0]}, tot[1];
+  if (!grid_total_last<V, S, 1>(part1, a.partials, a.tickets + TK_S, red, tot)) return;
   if (threadIdx.x != 0) return;
-  sc_after_s(st, tot);
+  sc_after_s<V>(st, tot);
 }
 
 // K4: t = A s, (t, s), (t, t) -> omega
-template <class V>
-__global__ void __launch_bounds__(kSolverThreads, kSolverMinBlocks) k_t(KArgs<V> a) {
+template <class V, int S>
+HELM_SOLVER_KERNEL k_t(const __grid_constant__ KArgs<V> a) {
   pdl_enter();
-  using S = typename Prec<V>::S;
   __shared__ double red[32 * 3];
   SolverState* st = a.st;
-  if (st->status != ST_RUNNING || st->phase != PH_RUN || refine_step_pending(st)) return;
-  TEpi<V> epi = t_epi<V>(a);
-  spmv_run<V>(a.A, a.s, epi, nullptr, a.dev_err);
-  const double2 tsd = to_d2(epi.ts);
-  double part[3] = {tsd.x, tsd.y, to_d(epi.tt)};
-  double tot[3];
-  if (!grid_total_last<3>(part, a.partials, a.tickets + TK_T, red, tot)) return;
+  if (st->status != ST_RUNNING || st->phase != PH_RUN || refine_step_pending<V>(st)) return;
+  HELM_GRAPH_PHASES
+  V si = vzero<V>();
+  graph_spmv<V, S>(
+      ph, a.s, [&](int32_t i) { si = a.s[i]; }, [&](int32_t i, int li, V ax) { ph.row_t(i, li, si, ax, part); });
+  double part3[3] = {part[0], part[1], part[2]}, tot[3];
+  if (!grid_total_last<V, S, 3>(part3, a.partials, a.tickets + TK_T, red, tot)) return;
   if (threadIdx.x != 0) return;
-  sc_after_t(st, tot);
+  sc_after_t<V>(st, tot);
 }
 
 // K5: x += alpha p + omega s, r = s - omega t; stop test; rho, beta
-template <class V>
-__global__ void __launch_bounds__(kSolverThreads, kSolverMinBlocks) k_xr(KArgs<V> a) {
+template <class V, int S>
+HELM_SOLVER_KERNEL k_xr(const __grid_constant__ KArgs<V> a) {
   pdl_enter();
-  using S = typename Prec<V>::S;
   __shared__ double red[32 * 3];
   SolverState* st = a.st;
-  if (st->status != ST_RUNNING) {
+  // (mixed precision: a pending refinement step ends the inner loop)
+  if (st->status != ST_RUNNING || refine_step_pending<V>(st)) {
     if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(a, false);
     return;
   }
-  if (refine_step_pending(st)) {  // mixed precision: the inner loop ends for the refinement step
-    if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(a, false);
-    return;
-  }
-  typename Prec<V>::C rr = Prec<V>::czero();
-  typename Prec<V>::S r2 = Prec<V>::szero();
-  ph_xr<V>(a, Prec<V>::cvt(st->alpha), Prec<V>::cvt(st->omega), st->phase == PH_SCONV, rr, r2);
-  const double2 rrd = to_d2(rr);
-  double part[3] = {rrd.x, rrd.y, to_d(r2)};
-  double tot[3];
-  if (!grid_total_last<3>(part, a.partials, a.tickets + TK_XR, red, tot)) return;
+  HELM_GRAPH_PHASES
+  ph.upd_xr(Prec<V>::cvt(st->alpha), Prec<V>::cvt(st->omega), st->phase == PH_SCONV, part);
+  double part3[3] = {part[0], part[1], part[2]}, tot[3];
+  if (!grid_total_last<V, S, 3>(part3, a.partials, a.tickets + TK_XR, red, tot)) return;
   if (threadIdx.x != 0) return;
-  sc_after_xr(st, tot, deadline_passed(st));
-  set_cond(a, st->status == ST_RUNNING && !refine_step_pending(st));
+  sc_after_xr<V>(st, tot, deadline_passed(st));
+  set_cond(a, st->status == ST_RUNNING && !refine_step_pending<V>(st));
+}
+
+// ---------------------------------------------------------------- persistent loop
+
+// A solve as a loop over steps, each a vector update or a product, then a grid
+// barrier and (in every block the same) the sums and the scalar step that
+// chooses the next one.  complex128: the whole solve (init, iterations, tail,
+// restarts); complex64: the inner loop of mixed precision, from its start to the
+// next refinement step.  Every step does exactly what the graph kernel of that
+// name does, on the same rows of the same threads; the totals are formed from
+// the same partials in the same order, so all blocks take every decision
+// together (the deadline is decided by block 0 and carried in the last
+// reduction of each iteration).  Two partials buffers alternate, so a block may
+// publish the next step's sums while a slower block still reads the previous
+// ones.  The gathered vectors (p, s, x at the start and the end) are written by
+// other blocks of the same launch: they are read with coherent loads.  The
+// others stay in the block's shared memory as far as they fit (Phases).
+// One product, one reduction and one copy of each update in the code: see
+// persist.cuh on registers and code size.
+enum : int { STEP_INIT = 0, STEP_INIT_X0, STEP_LOAD, STEP_P, STEP_V, STEP_S, STEP_T, STEP_XR, STEP_FLUSH, STEP_TAIL,
+             STEP_END };
+template <class V, int S>
+__device__ __forceinline__ void persist_loop(const KArgs<V>& a, const PLayout& L) {
+  constexpr bool whole = std::is_same<V, double2>::value;
+  constexpr bool SPLIT = whole && SolverBounds<S>::parts > 1;
+  using G = GatherCoherent;
+  __shared__ double red[32 * 4];
+  __shared__ SolverState sst;
+  __shared__ unsigned int s_target;  // arrivals of the barriers passed
+  __shared__ int s_step;
+  const Phases<V> ph(a, L);
+  copy_state(&sst, a.st);
+  if (threadIdx.x == 0) s_target = 0u;
+  persist_table<V>(ph.q, a.A);
+  HeldPart held;
+  if constexpr (SPLIT) held.load(ph.q, a.A);
+  int buf = 0;
+  int step = sst.use_x0 ? STEP_INIT_X0 : STEP_INIT;
+  if (!whole) step = sst.status == ST_RUNNING && !refine_step_pending<V>(&sst) ? STEP_LOAD : STEP_END;
+  while (step != STEP_END) {
+    double part[4] = {0.0, 0.0, 0.0, 0.0};
+    if (step == STEP_P) {
+      ph.upd_p(Prec<V>::cvt(sst.beta), Prec<V>::cvt(sst.omega));
+    } else if (step == STEP_S) {
+      ph.upd_s(Prec<V>::cvt(sst.alpha), part);
+    } else if (step == STEP_XR) {
+      ph.upd_xr(Prec<V>::cvt(sst.alpha), Prec<V>::cvt(sst.omega), sst.phase == PH_SCONV, part);
+      part[3] = (blockIdx.x == 0 && threadIdx.x == 0 && deadline_passed(&sst)) ? 1.0 : 0.0;
+    } else if (whole && step == STEP_INIT) {
+      ph.init_zero(part);
+    } else if (!whole && step == STEP_LOAD) {  // the vectors of the inner solve's start
+      for_rows(ph.q, a.A.n, [&](int32_t i, int li) {
+        if (ph.v.shared()) ph.v.st(i, li, a.v[i]);
+        if (ph.r.shared()) ph.r.st(i, li, a.r[i]);
+        if (ph.rh.shared()) ph.rh.st(i, li, a.rh[i]);
+        if (ph.x.shared()) ph.x.st(i, li, a.x[i]);
+        if (ph.p.shared()) ph.p.st(i, li, a.p[i]);
+      });
+      step = STEP_P;
+      continue;
+    } else if (step == STEP_FLUSH) {  // x is complete once every block is here
+      if (sst.bnorm == 0.0) for_rows(ph.q, a.A.n, [&](int32_t i, int) { a.x[i] = vzero<V>(); });
+      else if (ph.x.shared()) for_rows(ph.q, a.A.n, [&](int32_t i, int li) { a.x[i] = *ph.x.at(li); });
+      if (!whole) break;
+    } else if (step != STEP_TAIL || sst.bnorm != 0.0) {  // a product
+      const V* in = step == STEP_V ? a.p : step == STEP_T ? a.s : a.x;
+      auto row = [&](int32_t i, int li, V ax) {
+        const int st = opaque(step);
+        if (st == STEP_V) ph.row_v(i, li, ph.rh.ld(i, li), ax, part);
+        else if (st == STEP_T) ph.row_t(i, li, ph.s.ld(i, li), ax, part);
+        else if (st == STEP_TAIL) part[0] = nrm_acc(part[0], csub(a.b[i], ax));
+        else ph.row_init(i, li, ax, part);
+      };
+      if constexpr (SPLIT) spmv_split<G>(ph.q, a.A, held, in, row);
+      else spmv_rows<V, SolverBounds<S>::persist_u, 1, G>(ph.q, a.A, in, [](int32_t) {}, row);
+    }
+    if (step == STEP_P || step == STEP_FLUSH) {
+      if (!grid_barrier(a.tickets, a.dev_err, &s_target)) return;
+      step = step == STEP_P ? STEP_V : STEP_TAIL;
+      continue;
+    }
+    buf ^= 1;
+    double tot[4];
+    if (!grid_total_all<V, S, 4>(part, a.partials + static_cast<size_t>(buf) * gridDim.x * 4, a.tickets, a.dev_err, &s_target,
+                           red, tot))
+      return;
+    if (threadIdx.x == 0) {
+      int next = STEP_P;
+      if (step == STEP_V) {
+        const double t2[2] = {tot[0], tot[1]};
+        sc_after_v<V>(&sst, t2);
+        next = STEP_S;
+      } else if (step == STEP_S) {
+        const double t1[1] = {tot[0]};
+        sc_after_s<V>(&sst, t1);
+        next = sst.phase == PH_RUN ? STEP_T : STEP_XR;
+      } else if (step == STEP_T) {
+        const double t3[3] = {tot[0], tot[1], tot[2]};
+        sc_after_t<V>(&sst, t3);
+        next = STEP_XR;
+      } else if (step == STEP_XR) {
+        const double t3[3] = {tot[0], tot[1], tot[2]};
+        sc_after_xr<V>(&sst, t3, tot[3] > 0.0);
+      } else if (step != STEP_TAIL) {
+        sc_init(&sst, tot, step == STEP_INIT_X0);
+      }
+      if (sst.status != ST_RUNNING || refine_step_pending<V>(&sst)) next = STEP_FLUSH;
+      if (step == STEP_TAIL) {
+        const double t1[1] = {tot[0]};
+        sc_tail(&sst, t1);
+        next = STEP_END;
+        // (as the host does for the graph)
+        if (restart_due(&sst)) {
+          next = STEP_INIT_X0;
+          sst.restarts += 1;
+          sst.use_x0 = 1;
+          sst.status = ST_RUNNING;
+          sst.phase = PH_RUN;
+          sst.relres = 0.0;
+          sst.relres_true = 0.0;
+          const double2 one = make_double2(1.0, 0.0);
+          sst.rho = one;
+          sst.alpha = one;
+          sst.omega = one;
+          sst.beta = make_double2(0.0, 0.0);
+        }
+      }
+      s_step = next;
+    }
+    __syncthreads();
+    step = s_step;
+  }
+  if (blockIdx.x == 0) copy_state(a.st, &sst);
 }
 
 // Solver grid: one wave of the solver kernels -- the blocks that fit on every
@@ -688,12 +879,9 @@ template <class V>
 struct KShapes {
   int grid;     // every kernel of the loop, init and tail included
   int threads;  // threads per block (a multiple of 32)
+  int bps;      // blocks per SM the grid is sized for
+  int shape;    // SHAPE_*
 };
-
-template <class V>
-inline void enqueue_init(const KArgs<V>& a, const KShapes<V>& sh, cudaStream_t s) {
-  k_init<V><<<sh.grid, sh.threads, 0, s>>>(a);
-}
 
 // A loop kernel launched with programmatic stream serialization (a
 // programmatic edge from the kernel before it when captured into a graph);
@@ -717,18 +905,31 @@ inline void launch_loop_kernel(void (*kernel)(KArgs<V>), const KArgs<V>& a, cons
 #endif
 }
 
-template <class V>
-inline void enqueue_body(const KArgs<V>& a, const KShapes<V>& sh, cudaStream_t s) {
-  launch_loop_kernel<V>(k_p<V>, a, sh, s);
-  launch_loop_kernel<V>(k_v<V>, a, sh, s);
-  launch_loop_kernel<V>(k_s<V>, a, sh, s);
-  launch_loop_kernel<V>(k_t<V>, a, sh, s);
-  launch_loop_kernel<V>(k_xr<V>, a, sh, s);
+template <class V, int S>
+inline void enqueue_body_s(const KArgs<V>& a, const KShapes<V>& sh, cudaStream_t s) {
+  launch_loop_kernel<V>(k_p<V, S>, a, sh, s);
+  launch_loop_kernel<V>(k_v<V, S>, a, sh, s);
+  launch_loop_kernel<V>(k_s<V, S>, a, sh, s);
+  launch_loop_kernel<V>(k_t<V, S>, a, sh, s);
+  launch_loop_kernel<V>(k_xr<V, S>, a, sh, s);
 }
 
+// f(shape constant) for the shape of a solve
+template <class V, class F>
+inline void with_shape(const KShapes<V>& sh, F f) {
+  if constexpr (std::is_same<V, double2>::value) {
+    if (sh.shape == SHAPE_SMALL) return f(std::integral_constant<int, SHAPE_SMALL>());
+  }
+  if (sh.shape == SHAPE_MID) return f(std::integral_constant<int, SHAPE_MID>());
+  f(std::integral_constant<int, SHAPE_LARGE>());
+}
 template <class V>
-inline helm_status prepare_krylov_kernels() {
-  return HELM_OK;
+inline void enqueue_init(const KArgs<V>& a, const KShapes<V>& sh, cudaStream_t s) {
+  with_shape(sh, [&](auto S) { k_init<V, S.value><<<sh.grid, sh.threads, 0, s>>>(a); });
+}
+template <class V>
+inline void enqueue_body(const KArgs<V>& a, const KShapes<V>& sh, cudaStream_t s) {
+  with_shape(sh, [&](auto S) { enqueue_body_s<V, S.value>(a, sh, s); });
 }
 
 // Shape of a slice-parallel grid: one block per SM (blocks_per_sm with
@@ -749,43 +950,16 @@ inline SliceShape slice_shape(int32_t n, int num_sms, int max_threads, int block
   return SliceShape{static_cast<int>(grid), static_cast<int>(32 * std::max<int64_t>(warps, 1))};
 }
 
-// Shape of the solver's grid: blocks of at most HELM_SOLVER_THREADS threads,
-// HELM_SOLVER_BPS blocks per SM.  A build-time choice, not a run-time one:
-// the shape fixes which thread owns which row and so the rounding of every
-// reduction, and a solve must give the same bits on every run.
-// Measured on the 120x60x50 cavity (graph loop, us per iteration): 1024 x 1
-// (832 threads used) 144.6, 512 x 2 138.4, 256 x 4 140.8.
-#ifndef HELM_SOLVER_THREADS
-#define HELM_SOLVER_THREADS 512
-#endif
-#ifndef HELM_SOLVER_BPS
-#define HELM_SOLVER_BPS 2
-#endif
-// The complex64 solver (the inner solves of mixed precision, HBM-bound) may
-// take another shape.
-#ifndef HELM_SOLVER32_THREADS
-#define HELM_SOLVER32_THREADS HELM_SOLVER_THREADS
-#endif
-#ifndef HELM_SOLVER32_BPS
-#define HELM_SOLVER32_BPS HELM_SOLVER_BPS
-#endif
-
-// Grid of the solver's kernels; the kernels (and `extra` ones: the tail, the
-// persistent kernel) must fit HELM_SOLVER_BPS such blocks per SM.
+// Grid of the solver's kernels: one wave.
 template <class V>
-inline helm_status krylov_shapes(helm_csr A, KShapes<V>* sh, std::initializer_list<const void*> extra = {}) {
-  std::vector<const void*> fns = {reinterpret_cast<const void*>(&k_init<V>), reinterpret_cast<const void*>(&k_p<V>),
-                                  reinterpret_cast<const void*>(&k_v<V>),    reinterpret_cast<const void*>(&k_s<V>),
-                                  reinterpret_cast<const void*>(&k_t<V>),    reinterpret_cast<const void*>(&k_xr<V>)};
-  for (const void* f : extra) fns.push_back(f);
+inline helm_status krylov_shapes(helm_csr A, KShapes<V>* sh) {
+  const int64_t nsl = (static_cast<int64_t>(A->n) + 31) / 32, sms = A->num_sms;
   const bool c64 = std::is_same<V, float2>::value;
-  const int bps = c64 ? HELM_SOLVER32_BPS : HELM_SOLVER_BPS;
-  const SliceShape ss = slice_shape(A->n, A->num_sms, c64 ? HELM_SOLVER32_THREADS : HELM_SOLVER_THREADS, bps);
-  for (const void* fn : fns) {
-    int b = 0;
-    HELM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, ss.threads, 0));
-    if (b < bps) return HELM_ERR_CUDA;
-  }
+  sh->shape = nsl > sms * kMidSlices                                                    ? SHAPE_LARGE
+              : !c64 && nsl <= sms * (SolverBounds<SHAPE_SMALL>::threads / 32 / kParts) ? SHAPE_SMALL
+                                                                                        : SHAPE_MID;
+  sh->bps = sh->shape == SHAPE_LARGE ? SolverBounds<SHAPE_LARGE>::blocks : 1;
+  const SliceShape ss = slice_shape(A->n, A->num_sms, sh->shape == SHAPE_MID ? SolverBounds<SHAPE_MID>::threads : 512, sh->bps);
   sh->grid = ss.grid;
   sh->threads = ss.threads;
   return HELM_OK;

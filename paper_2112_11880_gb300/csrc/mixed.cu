@@ -437,6 +437,14 @@ __global__ void __launch_bounds__(R128, kSolverMinBlocks) k_mx_tail(RuArgs a) {
   if (bnorm != 0.0) st->spmv_count += 1;
 }
 
+// The inner solve as one cooperative kernel, from its start to the next
+// refinement step (persist_loop, krylov.cuh): the same bits as the loop's five
+// kernels.
+template <int S>
+HELM_SOLVER_KERNEL k_mx_inner(const __grid_constant__ KArgs<float2> k, const __grid_constant__ PLayout L) {
+  persist_loop<float2, S>(k, L);
+}
+
 struct MxShapes {
   KShapes<float2> k;
   int grid128;
@@ -544,7 +552,6 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   helm_status st = ensure_vals32(A, s);
   if (st == HELM_OK) st = ensure_vectors(A, kNumVec > 3 + 2 * kGcr ? kNumVec : 3 + 2 * kGcr);
   if (st == HELM_OK) st = ensure_vectors32(A, 8);
-  if (st == HELM_OK) st = prepare_krylov_kernels<float2>();
   if (st != HELM_OK) return st;
   for (const void* fn : {reinterpret_cast<const void*>(&k_mx_init), reinterpret_cast<const void*>(&k_mx_residual),
                          reinterpret_cast<const void*>(&k_gcr_project), reinterpret_cast<const void*>(&k_mx_tail)})
@@ -602,11 +609,19 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   a.tickets = A->tickets;
   a.dev_err = A->dev_err;
 
+  // HELM_LAUNCH_AUTO: persistent inner solves where the device can launch them
+  PShape ps;
+  const void* inner = nullptr;
+  with_shape(sh.k, [&](auto S) { inner = reinterpret_cast<const void*>(&k_mx_inner<S.value>); });
+  const bool persistent = o.launch == HELM_LAUNCH_AUTO && persist_fit(inner, n, sh.k.grid, sh.k.threads, sh.k.bps, 1,
+                                                                 Phases<float2>::kOwn, sizeof(float2), &ps);
+  (void)cudaGetLastError();
+
   // the inner-loop graph and the step graph per (b, x), tagged as mixed in
   // the cache key
   GraphEntry* gi = nullptr;
   GraphEntry* gs = nullptr;
-  if (o.launch != HELM_LAUNCH_HOST) {
+  if (o.launch != HELM_LAUNCH_HOST && !persistent) {
     auto ki = graph_key(b, x, 2, o), ks = graph_key(b, x, 3, o);
     auto ii = A->graphs.find(ki), is = A->graphs.find(ks);
     if (ii != A->graphs.end() && is != A->graphs.end()) {
@@ -640,9 +655,17 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   k_mx_configure<<<1, 1, 0, s>>>(A->state, o.inner_tol);
   HELM_CUDA_TRY(cudaGetLastError());
   SolverState* hs = A->state_host;
+  unsigned int herr = 0;
   mx_init(a, sh, s);
   for (;;) {
-    if (gi) {
+    if (persistent) {
+      HELM_CUDA_TRY(cudaMemsetAsync(A->tickets + TK_BAR_COUNT, 0, 2 * sizeof(unsigned int), s));  // count, abort
+      void* args[] = {&k, &ps.L};
+      HELM_CUDA_TRY(cudaLaunchCooperativeKernel(inner, dim3(ps.grid), dim3(ps.threads), args, ps.smem, s));
+      mx_step(a, sh, s);
+      HELM_CUDA_TRY(cudaGetLastError());
+      HELM_CUDA_TRY(cudaMemcpyAsync(&herr, A->dev_err, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
+    } else if (gi) {
       HELM_CUDA_TRY(cudaGraphLaunch(gi->exec, s));
       HELM_CUDA_TRY(cudaGraphLaunch(gs->exec, s));
     } else {
@@ -651,11 +674,11 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
     }
     HELM_CUDA_TRY(cudaMemcpyAsync(hs, A->state, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
     HELM_CUDA_TRY(cudaStreamSynchronize(s));
+    if (herr) return HELM_ERR_CUDA;
     if (hs->status != ST_RUNNING) break;
   }
   mx_tail(a, sh, s);
   HELM_CUDA_TRY(cudaGetLastError());
-  unsigned int herr = 0;
   HELM_CUDA_TRY(cudaMemcpyAsync(hs, A->state, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
   HELM_CUDA_TRY(cudaMemcpyAsync(&herr, A->dev_err, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
   HELM_CUDA_TRY(cudaStreamSynchronize(s));

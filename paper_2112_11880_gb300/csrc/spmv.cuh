@@ -110,27 +110,36 @@ __device__ __forceinline__ float2 mac_imag(float b, float2 x, float2 acc) {
 
 // How the gathered vector is loaded.  Kernels that only read x take the
 // read-only path; a kernel that writes the vector it later gathers (the
-// persistent solver, across its grid barriers) must use coherent loads.
+// persistent solvers, across their grid barriers) must use coherent loads.
 struct GatherReadOnly {
   template <class V> __device__ __forceinline__ static V ld(const V* p) { return __ldg(p); }
 };
 struct GatherCoherent {
-  // ld.global.cg: served by L2, the point of coherence of the GPU (an SM's
-  // L1 may still hold a line another SM has since rewritten)
-  template <class V> __device__ __forceinline__ static V ld(const V* p) { return __ldcg(p); }
+  // an ordinary load: the acquire fence of the grid barrier before it orders
+  // it after the other blocks' stores (and drops this SM's L1 lines), and
+  // within a phase neighbouring rows share the lines in L1
+  template <class V> __device__ __forceinline__ static V ld(const V* p) { return *p; }
 };
 
-// Sum of row r = 32 s + lane (len entries) of slice s: real parts in CSR
-// order (U-entry pipeline), then the row's imaginary entries.
-template <class V, class G = GatherReadOnly, int U = kSpmvUnroll>
-__device__ __forceinline__ V sell_row(const CsrDev<V>& A, int32_t s, int lane, int32_t r, int32_t len,
-                                      const V* x) {
+// Where a slice lies: its first entry and width, and those of its imaginary
+// entries.
+struct SlicePos {
+  int32_t base, w, ib, iw;
+};
+template <class V>
+__device__ __forceinline__ SlicePos slice_pos(const CsrDev<V>& A, int32_t s) {
+  const int32_t base = A.soff[s], ib = A.isoff[s];
+  return SlicePos{base, (A.soff[s + 1] - base) >> 5, ib, (A.isoff[s + 1] - ib) >> 5};
+}
+
+// acc + sum over the row's `len` entries of (IMAG ? i : 1) v_k x[c_k], entry k
+// at stride 32 from v and c, at most w entries in the slice: a U-entry
+// software pipeline (the next stage's entries are loaded before this one's
+// products; the gathers of a stage are in flight together).
+template <class V, class G, int U, bool IMAG>
+__device__ __forceinline__ V sell_acc(const typename RealOf<V>::T* v, const int32_t* c, int32_t w, int32_t len,
+                                      const V* x, V acc) {
   using R = typename RealOf<V>::T;
-  const int32_t base = A.soff[s];
-  const int32_t w = (A.soff[s + 1] - base) >> 5;
-  const R* v = A.sval + base + lane;
-  const int32_t* c = A.scol + base + lane;
-  V acc = vzero<V>();
   R a[U];
   int32_t cc[U];
 #pragma unroll
@@ -142,6 +151,7 @@ __device__ __forceinline__ V sell_row(const CsrDev<V>& A, int32_t s, int lane, i
       cc[u] = __ldcs(c + u * 32);
     }
   }
+#pragma unroll 1
   for (int32_t k = 0; k < w; k += U) {
     V xv[U];
 #pragma unroll
@@ -160,24 +170,55 @@ __device__ __forceinline__ V sell_row(const CsrDev<V>& A, int32_t s, int lane, i
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (k + u < len) acc = mac_real(a[u], xv[u], acc);
+      if (k + u < len) acc = IMAG ? mac_imag(a[u], xv[u], acc) : mac_real(a[u], xv[u], acc);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       a[u] = an[u];
       cc[u] = cn[u];
     }
   }
-  const int32_t ib = A.isoff[s];
-  const int32_t iw = (A.isoff[s + 1] - ib) >> 5;
+  return acc;
+}
+
+// acc + the row's imaginary entries (iw in its slice at most, from ib).
+template <class V, class G>
+__device__ __forceinline__ V imag_row(const CsrDev<V>& A, int32_t ib, int32_t iw, int lane, int32_t r, const V* x,
+                                      V acc) {
   if (iw > 0) {
     const int32_t il = r < A.n ? A.ilen[r] : 0;
     for (int32_t q = 0; q < iw; ++q) {
       if (q < il) {
-        const R b = A.ival[ib + q * 32 + lane];
+        const typename RealOf<V>::T b = A.ival[ib + q * 32 + lane];
         acc = mac_imag(b, G::ld(x + A.icol[ib + q * 32 + lane]), acc);
       }
     }
   }
+  return acc;
+}
+
+// Sum of row r = 32 s + lane (len entries) of the slice at `sp`: real parts in
+// CSR order, then the row's imaginary entries.
+template <class V, class G = GatherReadOnly, int U = kSpmvUnroll>
+__device__ __forceinline__ V sell_row(const CsrDev<V>& A, const SlicePos& sp, int lane, int32_t r, int32_t len,
+                                      const V* x) {
+  const V acc = sell_acc<V, G, U, false>(A.sval + sp.base + lane, A.scol + sp.base + lane, sp.w, len, x, vzero<V>());
+  return imag_row<V, G>(A, sp.ib, sp.iw, lane, r, x, acc);
+}
+
+// A row's sum in kParts parts, for solvers that share it out to as many warps
+// (and then, in every form, take it as the parts added in order): part p is
+// entries [p w', (p + 1) w') with w' = ceil(w / kParts) for slice width w, real
+// parts, then imaginary ones likewise.
+constexpr int kParts = 3;
+__host__ __device__ __forceinline__ int32_t part_width(int32_t w) { return (w + kParts - 1) / kParts; }
+template <class V, class G, int U>
+__device__ __forceinline__ V sell_row_part(const CsrDev<V>& A, const SlicePos& sp, int lane, int32_t r, int32_t len,
+                                           int32_t p, const V* x) {
+  const int32_t ch = part_width(sp.w), ci = part_width(sp.iw);
+  const int32_t il = sp.iw > 0 && r < A.n ? A.ilen[r] : 0;
+  const int32_t at = sp.base + p * ch * 32 + lane, ai = sp.ib + p * ci * 32 + lane;
+  V acc = sell_acc<V, G, U, false>(A.sval + at, A.scol + at, ch, max(min(len - p * ch, ch), 0), x, vzero<V>());
+  if (sp.iw > 0) acc = sell_acc<V, G, 2, true>(A.ival + ai, A.icol + ai, ci, max(min(il - p * ci, ci), 0), x, acc);
   return acc;
 }
 
@@ -203,12 +244,18 @@ struct SliceRows {
   // Move to this warp's slice of the next round that gives it one; s = nsl
   // when there is none.
   __device__ __forceinline__ bool advance() {
-    const int64_t G = gridDim.x, WB = blockDim.x >> 5, W = G * WB;
-    const int64_t b = blockIdx.x, w = threadIdx.x >> 5;
-    for (++k; static_cast<int64_t>(k) * W < nsl; ++k) {
-      const int64_t base = static_cast<int64_t>(k) * W;
-      const int64_t R = nsl - base < W ? nsl - base : W;
-      const int64_t lo = base + (b * R) / G, hi = base + ((b + 1) * R) / G;
+    // 32-bit arithmetic: nsl < 2^26, W <= 2^17 warps and b R < 2^31 on this
+    // GPU's grids; a full round (R = W) gives block b its WB slices without a
+    // division
+    const uint32_t G = gridDim.x, WB = blockDim.x >> 5, W = G * WB, m = static_cast<uint32_t>(nsl);
+    const uint32_t b = blockIdx.x, w = threadIdx.x >> 5;
+    uint32_t base = static_cast<uint32_t>(++k) * W;
+    for (; base < m; base += W, ++k) {
+      uint32_t lo = base + b * WB, hi = lo + WB;
+      if (m - base < W) {
+        lo = base + b * (m - base) / G;
+        hi = base + (b + 1) * (m - base) / G;
+      }
       if (lo + w < hi) {
         s = static_cast<int32_t>(lo + w);
         return true;
@@ -248,17 +295,7 @@ __device__ __forceinline__ float2 dia_row(const CsrDev<float2>& A, int32_t s, in
     }
   }
   const int32_t ib = A.isoff[s];
-  const int32_t iw = (A.isoff[s + 1] - ib) >> 5;
-  if (iw > 0) {
-    const int32_t il = r < A.n ? A.ilen[r] : 0;
-    for (int32_t q = 0; q < iw; ++q) {
-      if (q < il) {
-        const float b = A.ival[ib + q * 32 + lane];
-        acc = mac_imag(b, G::ld(x + A.icol[ib + q * 32 + lane]), acc);
-      }
-    }
-  }
-  return acc;
+  return imag_row<float2, G>(A, ib, (A.isoff[s + 1] - ib) >> 5, lane, r, x, acc);
 }
 
 struct NoGate {
@@ -286,9 +323,9 @@ __device__ __forceinline__ bool spmv_run(const CsrDev<V>& A, const V* __restrict
     V acc;
     if constexpr (std::is_same<V, float2>::value) {
       if (A.ndia > 0) acc = dia_row<G>(A, q.s, q.lane, r, x);
-      else acc = sell_row<V, G, U>(A, q.s, q.lane, r, len, x);
+      else acc = sell_row<V, G, U>(A, slice_pos(A, q.s), q.lane, r, len, x);
     } else {
-      acc = sell_row<V, G, U>(A, q.s, q.lane, r, len, x);
+      acc = sell_row<V, G, U>(A, slice_pos(A, q.s), q.lane, r, len, x);
     }
     if (r < A.n) epi.row(r, acc);
   }

@@ -14,6 +14,7 @@
 #include <utility>
 #include <vector>
 
+#include "blas1.cuh"
 #include "common.cuh"
 #include "internal.hpp"
 #include "krylov.cuh"
@@ -1023,6 +1024,14 @@ helm_status helm_dot(int64_t n, helm_dtype dt, const void* d_x, const void* d_y,
   const size_t esz = dt == HELM_C128 ? 16 : 8;
   if (!aligned(d_x, esz) || !aligned(d_y, esz) || !aligned(d_out, 16)) return HELM_ERR_INVALID;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  if (n <= kShortMax) {
+    if (dt == HELM_C128)
+      launch_short_dot(n, (const double2*)d_x, (const double2*)d_y, conj_x != 0, static_cast<double*>(d_out), s);
+    else
+      launch_short_dot(n, (const float2*)d_x, (const float2*)d_y, conj_x != 0, static_cast<double*>(d_out), s);
+    HELM_CUDA_TRY(cudaGetLastError());
+    return HELM_OK;
+  }
   const int grid = vec_grid_for(n);
   double* part = nullptr;
   HELM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&part), sizeof(double) * 2 * grid, s));
@@ -1050,6 +1059,12 @@ helm_status helm_nrm2(int64_t n, helm_dtype dt, const void* d_x, double* d_out, 
   const size_t esz = dt == HELM_C128 ? 16 : 8;
   if (!aligned(d_x, esz) || !aligned(d_out, 8)) return HELM_ERR_INVALID;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  if (n <= kShortMax) {
+    if (dt == HELM_C128) launch_short_norm(n, (const double2*)d_x, d_out, s);
+    else launch_short_norm(n, (const float2*)d_x, d_out, s);
+    HELM_CUDA_TRY(cudaGetLastError());
+    return HELM_OK;
+  }
   const int grid = vec_grid_for(n);
   double* part = nullptr;
   HELM_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&part), sizeof(double) * grid, s));

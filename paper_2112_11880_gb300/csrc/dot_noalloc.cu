@@ -17,6 +17,7 @@
 // cudaGetSymbolAddress and passes it to the kernels.  Nothing is cached: after
 // a device reset the library's device code is loaded again (possibly at a new
 // address), and the next call sees that address.
+#include "blas1.cuh"
 #include "common.cuh"
 #include "internal.hpp"
 #include "spmv.cuh"
@@ -87,10 +88,16 @@ extern "C" helm_status helm_dot_noalloc(int64_t n, helm_dtype dt, const void* d_
   if (n > 0 && (!d_x || !d_y)) return HELM_ERR_INVALID;
   const size_t esz = dt == HELM_C128 ? 16 : 8;
   if (!aligned(d_x, esz) || !aligned(d_y, esz) || !aligned(d_out, 16)) return HELM_ERR_INVALID;
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  if (n <= kShortMax) {  // no scratch at all
+    double* out = static_cast<double*>(d_out);
+    if (dt == HELM_C128) launch_short_dot(n, (const double2*)d_x, (const double2*)d_y, conj_x != 0, out, s);
+    else launch_short_dot(n, (const float2*)d_x, (const float2*)d_y, conj_x != 0, out, s);
+    return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_ERR_CUDA;
+  }
   double* scratch = nullptr;
   helm_status st = scratch_address(&scratch);
   if (st != HELM_OK) return st;
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   // The grid never exceeds the scratch capacity; the grid-stride loop covers
   // any n below 2^31 with it.
   int64_t want = (n + kNoallocThreads - 1) / kNoallocThreads;

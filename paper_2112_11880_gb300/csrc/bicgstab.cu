@@ -116,25 +116,10 @@ helm_status bicgstab_fp64(helm_csr A, const double2* b, double2* x, const helm_o
     });
     PShape ps;
     if (persist_fit(fn, n, sh.grid, sh.threads, sh.bps, split, Phases<V>::kOwn, sizeof(V), &ps)) {
-      k_configure<<<1, 1, 0, s>>>(A->state, o.tol, o.maxit, use_x0_first, o.deadline_s, 1);
-      HELM_CUDA_TRY(cudaGetLastError());
-      HELM_CUDA_TRY(cudaMemsetAsync(A->tickets + TK_BAR_COUNT, 0, 2 * sizeof(unsigned int), s));  // count, abort
       void* args[] = {&a, &ps.L};
-      const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(ps.grid), dim3(ps.threads), args, ps.smem, s);
-      if (e == cudaSuccess) {
-        HELM_CUDA_TRY(cudaMemcpyAsync(hs, A->state, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
-        HELM_CUDA_TRY(cudaMemcpyAsync(&herr, A->dev_err, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
-        HELM_CUDA_TRY(cudaStreamSynchronize(s));
-        if (herr) return HELM_ERR_CUDA;
-        done = true;
-      } else {
-        debug_cuda_error(e, __FILE__, __LINE__);
-      }
+      HELM_TRY(run_persistent(A, fn, args, ps, o, s, &done));
     }
-    if (!done) {
-      (void)cudaGetLastError();
-      if (o.launch == HELM_LAUNCH_PERSISTENT) return HELM_ERR_CUDA;
-    }
+    if (!done && o.launch == HELM_LAUNCH_PERSISTENT) return HELM_ERR_CUDA;
   }
 
   if (!done) {

@@ -226,10 +226,32 @@ __device__ __forceinline__ void put_block_partials(double (&v)[K], double* red, 
   }
 }
 
-// Fixed-order totals of all blocks' partials, valid in thread 0: one warp per
+// out[k] = sum over the blocks of component k's partials, k < K: one warp per
 // component, lane j adds blocks j, j + 32, j + 64, ... (five loaded at a time) in
-// that order, then the lanes' tree; or thread j adds blocks j, j + T, ..., then
-// the block tree.
+// that order, then the lanes' tree.  Whole block; ends with its barrier.
+__device__ __forceinline__ void sum_components(const double* partials, int G, int K, double* out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = static_cast<int>(blockDim.x >> 5);
+#pragma unroll 1
+  for (int k = warp; k < K; k += nwarps) {
+    double acc = 0.0;
+#pragma unroll 1
+    for (int j0 = lane; j0 < G; j0 += 5 * 32) {
+      double w[5];
+#pragma unroll
+      for (int u = 0; u < 5; ++u)
+        w[u] = j0 + 32 * u < G ? ld_cg(&partials[static_cast<size_t>(k) * G + j0 + 32 * u]) : 0.0;
+#pragma unroll
+      for (int u = 0; u < 5; ++u)
+        if (j0 + 32 * u < G) acc += w[u];
+    }
+    acc = lanes_sum(acc, 32);
+    if (lane == 0) out[k] = acc;
+  }
+  __syncthreads();
+}
+
+// Fixed-order totals of all blocks' partials, valid in thread 0: sum_components,
+// or thread j adds blocks j, j + T, ..., then the block tree.
 template <class V, int S, int K>
 __device__ __forceinline__ void sum_block_partials(const double* partials, int G, double* red, double (&tot)[K]) {
   if constexpr (kOrderedSums<V, S>) {
@@ -243,25 +265,8 @@ __device__ __forceinline__ void sum_block_partials(const double* partials, int G
 #pragma unroll
     for (int k = 0; k < K; ++k) tot[k] = acc[k];
   } else {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = static_cast<int>(blockDim.x >> 5);
     __shared__ double out[K];
-#pragma unroll 1
-    for (int k = warp; k < K; k += nwarps) {
-      double acc = 0.0;
-#pragma unroll 1
-      for (int j0 = lane; j0 < G; j0 += 5 * 32) {
-        double w[5];
-#pragma unroll
-        for (int u = 0; u < 5; ++u)
-          w[u] = j0 + 32 * u < G ? ld_cg(&partials[static_cast<size_t>(k) * G + j0 + 32 * u]) : 0.0;
-#pragma unroll
-        for (int u = 0; u < 5; ++u)
-          if (j0 + 32 * u < G) acc += w[u];
-      }
-      acc = lanes_sum(acc, 32);
-      if (lane == 0) out[k] = acc;
-    }
-    __syncthreads();
+    sum_components(partials, G, K, out);
     if (threadIdx.x == 0) {
 #pragma unroll
       for (int k = 0; k < K; ++k) tot[k] = out[k];
@@ -497,6 +502,21 @@ __host__ __device__ __forceinline__ bool restart_due(SolverState* st) {
   if (st->status == ST_RESTART && st->relres_true <= st->tol) st->status = HELM_OK;
   if (st->status == ST_RESTART && st->iter >= st->maxit) st->status = HELM_ERR_NOT_CONVERGED;
   return st->status == ST_RESTART || (st->status == HELM_OK && st->relres_true > st->tol && st->iter < st->maxit);
+}
+
+// The state of a solve that starts again from x (k_configure with fresh = 0).
+__device__ __forceinline__ void restart_state(SolverState* st) {
+  const double2 one = make_double2(1.0, 0.0);
+  st->restarts += 1;
+  st->use_x0 = 1;
+  st->status = ST_RUNNING;
+  st->phase = PH_RUN;
+  st->relres = 0.0;
+  st->relres_true = 0.0;
+  st->rho = one;
+  st->alpha = one;
+  st->omega = one;
+  st->beta = make_double2(0.0, 0.0);
 }
 
 // ---------------------------------------------------------------- phases
@@ -834,17 +854,7 @@ __device__ __forceinline__ void persist_loop(const KArgs<V>& a, const PLayout& L
         // (as the host does for the graph)
         if (restart_due(&sst)) {
           next = STEP_INIT_X0;
-          sst.restarts += 1;
-          sst.use_x0 = 1;
-          sst.status = ST_RUNNING;
-          sst.phase = PH_RUN;
-          sst.relres = 0.0;
-          sst.relres_true = 0.0;
-          const double2 one = make_double2(1.0, 0.0);
-          sst.rho = one;
-          sst.alpha = one;
-          sst.omega = one;
-          sst.beta = make_double2(0.0, 0.0);
+          restart_state(&sst);
         }
       }
       s_step = next;
@@ -882,6 +892,28 @@ struct KShapes {
   int bps;      // blocks per SM the grid is sized for
   int shape;    // SHAPE_*
 };
+
+// A whole solve as one cooperative launch of `fn` on the shape that persist_fit
+// gave it; the final state is in A->state_host.  *done stays false (and nothing
+// has run) when the device did not take the launch.
+inline helm_status run_persistent(helm_csr A, const void* fn, void** args, const PShape& ps, const helm_opts& o,
+                                  cudaStream_t s, bool* done) {
+  k_configure<<<1, 1, 0, s>>>(A->state, o.tol, o.maxit, o.use_x0 ? 1 : 0, o.deadline_s, 1);
+  HELM_CUDA_TRY(cudaGetLastError());
+  HELM_CUDA_TRY(cudaMemsetAsync(A->tickets + TK_BAR_COUNT, 0, 2 * sizeof(unsigned int), s));  // count, abort
+  const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(ps.grid), dim3(ps.threads), args, ps.smem, s);
+  if (e != cudaSuccess) {
+    debug_cuda_error(e, __FILE__, __LINE__);
+    (void)cudaGetLastError();
+    return HELM_OK;
+  }
+  unsigned int herr = 0;
+  HELM_CUDA_TRY(cudaMemcpyAsync(A->state_host, A->state, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
+  HELM_CUDA_TRY(cudaMemcpyAsync(&herr, A->dev_err, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
+  HELM_CUDA_TRY(cudaStreamSynchronize(s));
+  *done = true;
+  return herr ? HELM_ERR_CUDA : HELM_OK;
+}
 
 // A loop kernel launched with programmatic stream serialization (a
 // programmatic edge from the kernel before it when captured into a graph);

@@ -908,7 +908,7 @@ helm_status helm_csr_create(helm_csr* out, int32_t n, int64_t nnz, const int32_t
   A->dt = dt;
 
   // workspace: partials for the largest grid, tickets, error flags, state
-  const size_t nparts = static_cast<size_t>(A->num_sms) * 32 * 8;  // <= 32 blocks/SM x 8 sums
+  const size_t nparts = static_cast<size_t>(A->num_sms) * kPartialsPerSm;
   if (cudaMalloc(&A->partials, nparts * sizeof(double)) != cudaSuccess) return fail(HELM_ERR_NOMEM);
   if (cudaMalloc(&A->tickets, (TK_COUNT + 2) * sizeof(unsigned int)) != cudaSuccess) return fail(HELM_ERR_NOMEM);
   if (cudaMemsetAsync(A->tickets, 0, (TK_COUNT + 2) * sizeof(unsigned int), s) != cudaSuccess)

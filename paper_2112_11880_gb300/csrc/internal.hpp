@@ -148,6 +148,9 @@ inline bool overlaps(const void* p, size_t pn, const void* q, size_t qn) {
 // Launch-shape helpers (api.cu).
 cudaError_t set_smem_attr(const void* fn, size_t bytes);
 int sm_count();
+// Doubles of a handle's partial sums per SM: 32 blocks of 8 sums.
+constexpr size_t kPartialsPerSm = 32 * 8;
+
 int vec_grid_for(int64_t n);
 
 // Allocate the complex128 Krylov vectors (and FP32 ones) on first use.

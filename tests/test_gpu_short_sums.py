@@ -1,4 +1,4 @@
-"""Dot products and norms of vectors up to 65,536 elements (one cluster of
+"""Dot products and norms of vectors up to 32,768 elements (one cluster of
 eight blocks) and one past it: against FP64 sums on the host.
 
 Bounds: a complex128 sum is a tree of at most 40 roundings above products of
@@ -21,7 +21,8 @@ DEV = torch.device("cuda:0")
 
 
 @pytest.mark.parametrize("dtype", [torch.complex128, torch.complex64])
-@pytest.mark.parametrize("n", [0, 1, 33, 256, 257, 1023, 8193, 33_000, 65_535, 65_536, 65_537])
+@pytest.mark.parametrize("n", [0, 1, 33, 256, 257, 2047, 2049, 8193, 9261, 32_767, 32_768, 32_769,
+                               65_537])
 def test_short_dot_and_norm(n, dtype):
     x = torch.as_tensor(g.complex_vector(n + 1, 7), device=DEV).to(dtype)[1:]  # aligned to an element only
     y = torch.as_tensor(g.complex_vector(n + 1, 8), device=DEV).to(dtype)[1:]

@@ -112,6 +112,8 @@ _lock = threading.Lock()
 def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     """Load libhelm.so (built by build.py / __graft_entry__.build())."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(path):
@@ -131,9 +133,12 @@ def _check(status: int, what: str):
 
 
 def _stream(stream=None) -> int:
-    import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the current stream's handle: torch.cuda.current_stream().cuda_stream
+        # without the Stream object that it makes for it (a tenth of a vector
+        # call of 9,261 elements)
+        import torch
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return int(getattr(stream, "cuda_stream", stream) or 0)
 
 
@@ -141,9 +146,12 @@ def _ptr(t) -> Optional[int]:
     return None if t is None else int(t.data_ptr())
 
 
+_C2 = ctypes.c_double * 2
+
+
 def _c2(z) -> ctypes.Array:
     z = complex(z)
-    return (ctypes.c_double * 2)(z.real, z.imag)
+    return _C2(z.real, z.imag)
 
 
 def _dtype_code(t) -> int:

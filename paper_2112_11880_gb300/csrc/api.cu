@@ -54,6 +54,65 @@ __global__ void __launch_bounds__(Engine<V>::kThreads, Engine<V>::kMinBlocks) k_
   (void)spmv_run<V, AxpbyEpi<V>, NoGate, GatherReadOnly, U>(A, x, epi, nullptr, nullptr);
 }
 
+// The complex64 product of a matrix with a diagonal copy, two neighbouring rows a
+// thread.  The values are read once and are what bounds it (HBM); to stream them a
+// thread has to have enough of them in flight without waiting on the gathers.  Of
+// up to three neighbouring diagonals two rows need four neighbours of x, not six,
+// and two values of a diagonal are one load.  Each row as dia_row sums it: the same
+// bits.  Bound by HBM and by how many loads an SM has in flight.
+// Measured (27 diagonals, us; one row a thread in blocks of 1,024 -> this):
+// 1,644,381 rows 40.3 -> 32.9 (6.2 TB/s of matrix and vectors), 847,665 23.2 ->
+// 19.7, 376,431 12.4 -> 10.9; 109,593 5.2 -> 5.7, 9,261 3.9 -> 4.3: from 200,000
+// rows on.
+constexpr int kDiaThreads = 128, kDiaBlocks = 10, kDiaUnroll = 2;
+constexpr int32_t kDiaRows = 200000;
+__global__ void __launch_bounds__(kDiaThreads, kDiaBlocks) k_spmv_dia(CsrDev<float2> A, const __grid_constant__ DiaPieces P,
+                                                 const float2* __restrict__ x, float2* y, float2 alpha, float2 beta,
+                                                 int mode) {
+  const uint32_t r = 2 * (blockIdx.x * static_cast<uint32_t>(kDiaThreads) + threadIdx.x), n = static_cast<uint32_t>(A.n);
+  if (r >= n) return;
+  const int32_t s = static_cast<int32_t>(r >> 5), lane = static_cast<int32_t>(r & 31);
+  const int32_t ib = A.isoff[s], ie = A.isoff[s + 1];
+  const float* dv = A.dval + r;
+  float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+  auto add = [](float a, float2 xv, float2& acc) {  // a zero leaves the sum untouched
+    const float sx = fmaf(a, xv.x, acc.x), sy = fmaf(a, xv.y, acc.y);
+    const bool nz = a != 0.f;
+    acc.x = nz ? sx : acc.x;
+    acc.y = nz ? sy : acc.y;
+  };
+#pragma unroll kDiaUnroll
+  for (int32_t p = 0; p < P.n; ++p) {
+    const int32_t d0 = P.d0[p], len = P.len[p];
+    float2 a[3], w[4];
+#pragma unroll
+    for (int32_t u = 0; u < 3; ++u)
+      a[u] = u < len ? __ldcs(reinterpret_cast<const float2*>(dv + (d0 + u) * A.dld)) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int32_t u = 0; u < 4; ++u) {
+      const uint32_t j = r + static_cast<uint32_t>(P.off[p] + u);
+      w[u] = u <= len && j < n ? __ldg(x + j) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int32_t u = 0; u < 3; ++u) {
+      add(a[u].x, w[u], s0);
+      add(a[u].y, w[u + 1], s1);
+    }
+  }
+  if (ie > ib) {
+    const int32_t iw = (ie - ib) >> 5;
+    s0 = imag_row<float2, GatherReadOnly>(A, ib, iw, lane, static_cast<int32_t>(r), x, s0);
+    s1 = imag_row<float2, GatherReadOnly>(A, ib, iw, lane + 1, static_cast<int32_t>(r + 1), x, s1);
+  }
+  AxpbyEpi<float2> epi{y, alpha, beta, mode, vzero<float2>()};
+  epi.prefetch(static_cast<int32_t>(r));
+  epi.row(static_cast<int32_t>(r), s0);
+  if (r + 1 < n) {
+    epi.prefetch(static_cast<int32_t>(r + 1));
+    epi.row(static_cast<int32_t>(r + 1), s1);
+  }
+}
+
 // ---------------------------------------------------------------- SELL-32 layout
 
 // Slice widths: w[s] = longest row of rows [32 s, 32 s + 32).
@@ -395,7 +454,7 @@ __global__ void k_dia_fill(int32_t n, const int32_t* __restrict__ rowptr, const 
       const int32_t d = colind[k] - i;
       int q = 0;
       while (q < D.nd - 1 && D.off[q] != d) ++q;
-      dval[static_cast<size_t>(q) * n + i] = static_cast<float>(vals[k].x);
+      dval[static_cast<size_t>(q) * dia_ld(n) + i] = static_cast<float>(vals[k].x);
     }
   }
 }
@@ -552,6 +611,12 @@ helm_status launch_spmv128(helm_csr A, const double2* x, double2* y, double2 alp
 helm_status launch_spmv64(helm_csr A, const float2* x, float2* y, float2 alpha, float2 beta, cudaStream_t s) {
   if (A->n == 0) return HELM_OK;
   const CsrDev<float2> d = csr_dev<float2>(A, static_cast<const float2*>(A->vals), A->sv);
+  if (d.ndia > 0 && A->n >= kDiaRows) {
+    const int64_t blocks = (static_cast<int64_t>(A->n) + 2 * kDiaThreads - 1) / (2 * kDiaThreads);
+    k_spmv_dia<<<static_cast<unsigned>(blocks), kDiaThreads, 0, s>>>(d, A->dia, x, y, alpha, beta, spmv_mode(alpha, beta));
+    HELM_CUDA_TRY(cudaGetLastError());
+    return HELM_OK;
+  }
   spmv_enqueue<float2>(A->spmv_variant, A->spmv_grid, A->spmv_threads, d, x, y, alpha, beta, spmv_mode(alpha, beta), s);
   HELM_CUDA_TRY(cudaGetLastError());
   return HELM_OK;
@@ -677,6 +742,19 @@ static helm_status analyze_diagonals(helm_csr A, cudaStream_t s) {
       break;
     }
     A->ndia = len;
+    DiaPieces& P = A->dia;
+    P.n = 0;
+    for (int q = 0; q < len; ++q) {
+      const int32_t last = P.n - 1;
+      if (last >= 0 && P.len[last] < 3 && D.off[q] == P.off[last] + P.len[last]) {
+        P.len[last] += 1;
+      } else {
+        P.off[P.n] = D.off[q];
+        P.d0[P.n] = static_cast<int16_t>(q);
+        P.len[P.n] = 1;
+        P.n += 1;
+      }
+    }
   } while (false);
   cudaFree(d_key);
   cudaFree(d_bad);
@@ -692,7 +770,7 @@ static helm_status build_dia_vals(helm_csr A, const float2* vals, SellVals* out,
   D.nd = A->ndia;
   HELM_CUDA_TRY(cudaMemcpyAsync(D.off, A->dia_off, sizeof(int32_t) * A->ndia, cudaMemcpyDeviceToHost, s));
   HELM_CUDA_TRY(cudaStreamSynchronize(s));
-  const size_t slots = static_cast<size_t>(A->ndia) * A->n;
+  const size_t slots = static_cast<size_t>(A->ndia) * dia_ld(A->n);
   HELM_CUDA_TRY(cudaMalloc(&out->dval, sizeof(float) * slots));
   HELM_CUDA_TRY(cudaMemsetAsync(out->dval, 0, sizeof(float) * slots, s));
   k_dia_fill<float2><<<vec_grid_for(A->n), 256, 0, s>>>(A->n, A->rowptr, A->colind, vals, D,

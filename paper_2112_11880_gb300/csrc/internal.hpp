@@ -43,6 +43,14 @@ enum : int { TK_INIT = 0, TK_V, TK_S, TK_T, TK_XR, TK_TAIL, TK_AUX0, TK_AUX1, TK
 // Group counters per two-level reduction (groups of blockDim blocks).
 constexpr int kGroupTickets = 256;
 
+// The diagonals of a handle as pieces of up to three neighbours: diagonals d0[p],
+// ..., d0[p] + len[p] - 1 with offsets off[p], off[p] + 1, ...
+struct DiaPieces {
+  int32_t n = 0;
+  int32_t off[32] = {};
+  int16_t d0[32] = {}, len[32] = {};
+};
+
 // Values of a matrix in the SELL-32 layout of the SpMV engine (spmv.cuh);
 // the slice offsets and columns are the handle's (shared by every value
 // array of one pattern).  Arrays are double for complex128 values, float for
@@ -53,7 +61,7 @@ struct SellVals {
   int32_t* icol = nullptr;   // columns of the imaginary entries
   void* ival = nullptr;      // imaginary parts
   int32_t* ilen = nullptr;   // [n] imaginary entries per row
-  void* dval = nullptr;      // complex64 sets of a handle with a diagonal copy: real parts [ndia][n]
+  void* dval = nullptr;      // complex64 sets of a handle with a diagonal copy: real parts [ndia][dia_ld(n)]
 };
 
 // complex128 Krylov vectors per handle (BiCGStab uses 6, TFQMR 8)
@@ -102,6 +110,7 @@ struct helm_csr_s {
   // one of ndia <= 32 diagonals col - row = dia_off[d] (ascending)
   int32_t ndia = 0;
   int32_t* dia_off = nullptr;
+  helm::DiaPieces dia;  // the same, neighbouring diagonals together
   helm::SellVals sv;                   // the caller's values (complex128 or complex64)
   helm::SellVals sv32;                 // the complex64 copy (mixed precision, complex128 handles)
   helm::SellVals svjac;                // A D^-1 (right Jacobi)

@@ -74,8 +74,10 @@ struct CsrDev {
   const int32_t* ilen;    // [n] imaginary entries per row (read only in slices that have some)
   int32_t ndia;           // complex64 with a diagonal copy: the real parts on ndia diagonals, else 0
   const int32_t* doff;    // [ndia] ascending offsets col - row
-  const R* dval;          // [ndia][n] real part of entry (r, r + doff[d]), 0 where none
+  int64_t dld;            // row length of dval: n rounded up to a multiple of 4
+  const R* dval;          // [ndia][dld] real part of entry (r, r + doff[d]), 0 where none
 };
+__host__ __device__ __forceinline__ int64_t dia_ld(int32_t n) { return (static_cast<int64_t>(n) + 3) & ~int64_t(3); }
 
 template <class V> __device__ __forceinline__ V vzero();
 template <> __device__ __forceinline__ double2 vzero<double2>() { return make_double2(0.0, 0.0); }
@@ -285,7 +287,7 @@ __device__ __forceinline__ float2 dia_row(const CsrDev<float2>& A, int32_t s, in
 #pragma unroll 9
     for (int32_t d = 0; d < A.ndia; ++d) {
       const int32_t j = r + __ldg(A.doff + d);
-      const float a = __ldcs(dv + static_cast<size_t>(d) * A.n);
+      const float a = __ldcs(dv + static_cast<size_t>(d) * A.dld);
       float2 xv = make_float2(0.f, 0.f);
       if (static_cast<uint32_t>(j) < static_cast<uint32_t>(A.n)) xv = G::ld(x + j);
       const float sx = fmaf(a, xv.x, acc.x), sy = fmaf(a, xv.y, acc.y);
@@ -354,7 +356,7 @@ inline CsrDev<V> csr_dev(const helm_csr_s* A, const V* vals, const SellVals& sv)
                    A->colind,   vals,     A->nsl,
                    A->sell_off, A->sell_col, static_cast<const R*>(sv.sval),
                    sv.isoff,    sv.icol,  static_cast<const R*>(sv.ival),
-                   sv.ilen,     dia ? A->ndia : 0, dia ? A->dia_off : nullptr,
+                   sv.ilen,     dia ? A->ndia : 0, dia ? A->dia_off : nullptr, dia_ld(A->n),
                    dia ? static_cast<const R*>(sv.dval) : nullptr};
 }
 

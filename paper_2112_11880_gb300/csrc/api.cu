@@ -54,6 +54,35 @@ __global__ void __launch_bounds__(Engine<V>::kThreads, Engine<V>::kMinBlocks) k_
   (void)spmv_run<V, AxpbyEpi<V>, NoGate, GatherReadOnly, U>(A, x, epi, nullptr, nullptr);
 }
 
+// The same for a matrix of few slices: P warps take a part of a slice's
+// rows each (sell_row_part), the first adds the parts in order.  At a few warps
+// per SM nothing is bound by bytes or FP64 but by a row's chain of loads, one
+// gather after the other.
+// Measured (us, a warp a slice -> this): ragged rows of up to 60 complex entries,
+// 20,011 rows 21.3 -> 12.7 (then the FP64 pipe: 240 instructions a slot of the
+// widest row), 5,000 18.5 -> 6.8, 1,000 18.0 -> 4.6; meshes of 27 entries a row,
+// 20x20x20 6.4 -> 3.8, 40x20x16 6.2 -> 4.4; ten slices per SM (60x30x25) 7.9 ->
+// 10.4.  Eight parts up to one slice per SM (1,000 rows: four 6.2), four up to five.
+constexpr int kSplitUnroll = 4;
+constexpr int kSplitSlices = 5;  // per SM, at most
+template <class V, int P>
+__global__ void __launch_bounds__(32 * P) k_spmv_split(CsrDev<V> A, const V* __restrict__ x, V* y, V alpha, V beta,
+                                                       int mode) {
+  __shared__ V part[P - 1][32];
+  const int lane = threadIdx.x & 31, p = threadIdx.x >> 5;
+  const int32_t s = blockIdx.x, r = s * 32 + lane;
+  const int32_t len = r < A.n ? A.rowptr[r + 1] - A.rowptr[r] : 0;
+  V acc = sell_row_part<V, GatherReadOnly, kSplitUnroll, P, kSplitUnroll>(A, slice_pos(A, s), lane, r, len, p, x);
+  if (p > 0) part[p - 1][lane] = acc;
+  __syncthreads();
+  if (p > 0 || r >= A.n) return;
+#pragma unroll
+  for (int q = 0; q < P - 1; ++q) acc = cadd(acc, part[q][lane]);
+  AxpbyEpi<V> epi{y, alpha, beta, mode, vzero<V>()};
+  epi.prefetch(r);
+  epi.row(r, acc);
+}
+
 // The complex64 product of a matrix with a diagonal copy, two neighbouring rows a
 // thread.  The values are read once and are what bounds it (HBM); to stream them a
 // thread has to have enough of them in flight without waiting on the gathers.  Of
@@ -599,10 +628,24 @@ static int spmv_mode(V alpha, V beta) {
   return (a1 && b0) ? 0 : (b0 ? 1 : 2);
 }
 
+// Launches k_spmv_split where a matrix has few enough slices for it.
+template <class V>
+static bool spmv_split(helm_csr A, const CsrDev<V>& d, const V* x, V* y, V alpha, V beta, cudaStream_t s) {
+  if (A->nsl > static_cast<int64_t>(A->num_sms) * kSplitSlices) return false;
+  const int mode = spmv_mode(alpha, beta);
+  if (A->nsl <= A->num_sms) k_spmv_split<V, 8><<<A->nsl, 256, 0, s>>>(d, x, y, alpha, beta, mode);
+  else k_spmv_split<V, 4><<<A->nsl, 128, 0, s>>>(d, x, y, alpha, beta, mode);
+  return true;
+}
+
 helm_status launch_spmv128(helm_csr A, const double2* x, double2* y, double2 alpha, double2 beta,
                            cudaStream_t s) {
   if (A->n == 0) return HELM_OK;
   const CsrDev<double2> d = csr_dev<double2>(A, static_cast<const double2*>(A->vals), A->sv);
+  if (spmv_split(A, d, x, y, alpha, beta, s)) {
+    HELM_CUDA_TRY(cudaGetLastError());
+    return HELM_OK;
+  }
   spmv_enqueue<double2>(A->spmv_variant, A->spmv_grid, A->spmv_threads, d, x, y, alpha, beta, spmv_mode(alpha, beta), s);
   HELM_CUDA_TRY(cudaGetLastError());
   return HELM_OK;
@@ -611,6 +654,11 @@ helm_status launch_spmv128(helm_csr A, const double2* x, double2* y, double2 alp
 helm_status launch_spmv64(helm_csr A, const float2* x, float2* y, float2 alpha, float2 beta, cudaStream_t s) {
   if (A->n == 0) return HELM_OK;
   const CsrDev<float2> d = csr_dev<float2>(A, static_cast<const float2*>(A->vals), A->sv);
+  // (a sliced-only handle takes the rows as a diagonal copy does: the same bits)
+  if (d.ndia == 0 && !A->sliced_only && spmv_split(A, d, x, y, alpha, beta, s)) {
+    HELM_CUDA_TRY(cudaGetLastError());
+    return HELM_OK;
+  }
   if (d.ndia > 0 && A->n >= kDiaRows) {
     const int64_t blocks = (static_cast<int64_t>(A->n) + 2 * kDiaThreads - 1) / (2 * kDiaThreads);
     k_spmv_dia<<<static_cast<unsigned>(blocks), kDiaThreads, 0, s>>>(d, A->dia, x, y, alpha, beta, spmv_mode(alpha, beta));
@@ -1028,7 +1076,8 @@ helm_status helm_csr_create(helm_csr* out, int32_t n, int64_t nnz, const int32_t
   // entries), then the stand-alone SpMV variant for this matrix
   helm_status st = build_sell_pattern(A, s);
   // complex64 products read the diagonal copy when the pattern has one
-  if (st == HELM_OK && !(flags & HELM_CSR_SLICED_ONLY)) st = analyze_diagonals(A, s);
+  A->sliced_only = (flags & HELM_CSR_SLICED_ONLY) != 0;
+  if (st == HELM_OK && !A->sliced_only) st = analyze_diagonals(A, s);
   if (st == HELM_OK) st = build_sell_vals(A, d_vals, dt, &A->sv, s);
   if (st == HELM_OK)
     st = dt == HELM_C128 ? autotune_spmv<double2>(A, csr_dev<double2>(A, static_cast<const double2*>(d_vals), A->sv), s)

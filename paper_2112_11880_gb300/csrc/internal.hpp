@@ -108,6 +108,7 @@ struct helm_csr_s {
   int32_t* sell_col = nullptr;         // [sell_entries]
   // diagonal copy of the pattern (complex64 products): every entry lies on
   // one of ndia <= 32 diagonals col - row = dia_off[d] (ascending)
+  bool sliced_only = false;  // created without it (HELM_CSR_SLICED_ONLY)
   int32_t ndia = 0;
   int32_t* dia_off = nullptr;
   helm::DiaPieces dia;  // the same, neighbouring diagonals together

@@ -207,20 +207,23 @@ __device__ __forceinline__ V sell_row(const CsrDev<V>& A, const SlicePos& sp, in
   return imag_row<V, G>(A, sp.ib, sp.iw, lane, r, x, acc);
 }
 
-// A row's sum in kParts parts, for solvers that share it out to as many warps
-// (and then, in every form, take it as the parts added in order): part p is
-// entries [p w', (p + 1) w') with w' = ceil(w / kParts) for slice width w, real
+// A row's sum in PARTS parts, for kernels that share it out to as many warps and
+// add the parts in order (solvers: kParts, in every form of the solve): part p is
+// entries [p w', (p + 1) w') with w' = ceil(w / PARTS) for slice width w, real
 // parts, then imaginary ones likewise.
 constexpr int kParts = 3;
-__host__ __device__ __forceinline__ int32_t part_width(int32_t w) { return (w + kParts - 1) / kParts; }
-template <class V, class G, int U>
+template <int PARTS = kParts>
+__host__ __device__ __forceinline__ int32_t part_width(int32_t w) {
+  return (w + PARTS - 1) / PARTS;
+}
+template <class V, class G, int U, int PARTS = kParts, int UI = 2>
 __device__ __forceinline__ V sell_row_part(const CsrDev<V>& A, const SlicePos& sp, int lane, int32_t r, int32_t len,
                                            int32_t p, const V* x) {
-  const int32_t ch = part_width(sp.w), ci = part_width(sp.iw);
+  const int32_t ch = part_width<PARTS>(sp.w), ci = part_width<PARTS>(sp.iw);
   const int32_t il = sp.iw > 0 && r < A.n ? A.ilen[r] : 0;
   const int32_t at = sp.base + p * ch * 32 + lane, ai = sp.ib + p * ci * 32 + lane;
   V acc = sell_acc<V, G, U, false>(A.sval + at, A.scol + at, ch, max(min(len - p * ch, ch), 0), x, vzero<V>());
-  if (sp.iw > 0) acc = sell_acc<V, G, 2, true>(A.ival + ai, A.icol + ai, ci, max(min(il - p * ci, ci), 0), x, acc);
+  if (sp.iw > 0) acc = sell_acc<V, G, UI, true>(A.ival + ai, A.icol + ai, ci, max(min(il - p * ci, ci), 0), x, acc);
   return acc;
 }
 

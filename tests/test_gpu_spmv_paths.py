@@ -1,5 +1,6 @@
-"""Stand-alone products at the sizes where their path changes: complex64 matrices
-on diagonals from 200,000 rows on."""
+"""Stand-alone products at the sizes where their path changes: matrices whose few
+slices are shared out to several warps, complex64 matrices on
+diagonals from 200,000 rows on."""
 import numpy as np
 import pytest
 
@@ -14,7 +15,49 @@ if not torch.cuda.is_available():
 import paper_2112_11880_gb300 as helm  # noqa: E402
 
 DEV = torch.device("cuda:0")
+SMS = torch.cuda.get_device_properties(0).multi_processor_count
 AXPBY = [(1.0, 0.0), (0.5 - 2.0j, 0.0), (1.5 + 0.5j, -0.25 + 1.0j)]
+
+
+def _ragged(n, most, complex_part, seed):
+    rng = np.random.default_rng(seed)
+    lens = rng.integers(0, most + 1, n)
+    lens[rng.random(n) < 0.1] = 0
+    lens = np.minimum(lens, n)
+    lens[0] = min(most, n)
+    rp = np.zeros(n + 1, np.int32)
+    rp[1:] = lens.cumsum()
+    start = rng.integers(0, np.maximum(n - lens + 1, 1))
+    ci = np.concatenate([np.arange(s, s + k) for s, k in zip(start, lens)] or [np.zeros(0)]).astype(np.int32)
+    v = rng.uniform(-1, 1, ci.size) + 1j * rng.uniform(-1, 1, ci.size) * (rng.random(ci.size) < complex_part)
+    return rp, ci, v
+
+
+@pytest.mark.parametrize("slices,extra", [(1, -31), (1, 0), (SMS, 0), (SMS, 1), (5 * SMS, -7), (5 * SMS, 1)])
+@pytest.mark.parametrize("most,complex_part", [(1, 1.0), (3, 0.0), (27, 0.05), (61, 1.0)])
+@pytest.mark.parametrize("dtype", [np.complex128, np.complex64])
+def test_slices_shared_out(slices, extra, most, complex_part, dtype):
+    """A row of m entries: 2 m products and sums of parts, m + 12 roundings a
+    component at most, and six of alpha and beta."""
+    n = 32 * slices + extra
+    rp, ci, v = _ragged(n, most, complex_part, 3)
+    v, x, y0 = v.astype(dtype), g.complex_vector(n, 4).astype(dtype), g.complex_vector(n, 5).astype(dtype)
+    eps = 2.0 ** -53 if dtype == np.complex128 else 2.0 ** -24
+    A = helm.CsrMatrix.from_host(rp, ci, v, device=DEV)
+    xd = torch.as_tensor(x, device=DEV)
+    rows = np.repeat(np.arange(n), np.diff(rp))
+
+    def rowsum(t):
+        return np.bincount(rows, weights=t, minlength=n)
+    t = v.astype(np.complex128) * x[ci]
+    ax = rowsum(t.real) + 1j * rowsum(t.imag)
+    ab = rowsum(np.abs(v).astype(np.float64) * np.abs(x[ci]))
+    for al, be in AXPBY:
+        y = torch.as_tensor(y0, device=DEV)
+        A.matvec(xd, y, alpha=al, beta=be)
+        bound = 4 * (most + 18) * eps * (abs(al) * ab + abs(be) * np.abs(y0).astype(np.float64))
+        assert np.all(np.abs(y.cpu().numpy() - (al * ax + be * y0)) <= bound)
+    A.close()
 
 
 @pytest.mark.parametrize("n", [200_000, 200_001, 200_003, 262_147])

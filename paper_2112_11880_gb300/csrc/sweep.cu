@@ -5,24 +5,25 @@
 // complex64 inner solves.
 //
 // Layout: every Krylov vector is node-major, frequency-minor: V[i * Fp + j],
-// Fp = F rounded up to a multiple of 32.  A warp owns one row and 32
-// frequencies: the row's K, M, B values and column indices are warp-uniform
-// loads (one transaction serves 32 frequencies), each gathered V[col][j..j+31]
-// is one 512-byte coalesced access, and every FP64 instruction does useful
-// work in all 32 lanes.  Per stored entry and frequency the work is 1 FMA to
+// Fp = F rounded up to a multiple of 32.  A warp takes a row of 32 running
+// frequencies, or as many rows as it takes to fill its lanes (SweepWalk): a row's
+// K, M, B values and column indices are loads that its lanes share, each gathered
+// V[col][j] is coalesced over the frequencies, and every FP64 instruction does
+// useful work in all 32 lanes.  Per stored entry and frequency the work is 1 FMA to
 // form Re(A_j) = K - w_j^2 M and 2 FMA for the real x complex product (rows
 // whose 32-row block has B = 0), or the complex product where B != 0.
 //
 // All per-frequency scalars (rho, alpha, omega, beta, norms, status, counts)
 // live on the device; each dot product is a per-frequency partial sum per
 // block, added in block order by the last block to arrive.  A frequency that
-// has converged (or failed) is frozen: its lanes do no arithmetic and write
-// nothing, and a 32-frequency group whose frequencies have all stopped is
-// skipped by every kernel.  The loop is one CUDA graph (conditional WHILE
+// has converged (or failed) is frozen: it leaves the list of running ones, and
+// no lane works on it any more.  The loop is one CUDA graph (conditional WHILE
 // node), as for the single solve.
 //
-// Tile shape autotuning: at creation the sweep times the batched SpMV with
-// 4, 8 and 16 warps per block on the actual matrix and keeps the fastest.
+// Blocks have 16 warps: few, large blocks leave few partial sums per frequency for
+// the last block to add (the sweep measured below, before its last change: 16 warps 905
+// ms, 8 warps 1050, 4 warps 1448); 8 or 4 where 16 would leave SMs without a block (80 rows, 32
+// frequencies: 16 warps 97 us an iteration, 4 warps 73).
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -38,6 +39,7 @@ namespace helm {
 
 namespace {
 
+constexpr int kSweepWarps = 16, kSweepMinWarps = 4;  // per block
 constexpr int kMaxF = 128;  // frequencies per sweep (<= threads per block: one thread per frequency)
 #ifndef HELM_SWEEP_FORM_MAX
 #define HELM_SWEEP_FORM_MAX (size_t(8) << 30)
@@ -79,14 +81,14 @@ struct SweepArgsT {
   double2 *rho, *alpha, *omg, *beta;    // [Fp]
   double *bnorm, *relres, *relres_true; // [Fp]
   int32_t *status, *iters, *phase;      // [Fp]
-  int32_t* gactive;                     // [G]: a frequency of the group is running
+  int32_t *act, *pos, *nact;            // the running frequencies: list [Fp], place in it (-1: stopped) [Fp], count
   // batched TFQMR only (null otherwise): A un and d [n][Fp]; gamma and
-  // (theta, tau) [Fp]; the true-residual check flags per frequency, per group
+  // (theta, tau) [Fp]; the true-residual check flags per frequency
   // and for the whole sweep; the iteration at which each frequency's
   // current (re)start began
   V *q1, *q2;
   double2 *gam, *tt;
-  int32_t *chk, *gcheck, *anychk, *start;
+  int32_t *chk, *anychk, *start;
   // batched BiCGStab(l) only: r_0..r_l and u_0..u_l (r_0 = r, u_0 = p, the
   // shadow r~ = rh), rho1 [Fp], the minimal-residual coefficients [Fp][8],
   // the Gram matrices [Fp][45] and the Gram step's block partials
@@ -128,31 +130,88 @@ template <class V> __device__ __forceinline__ V sw_zero();
 template <> __device__ __forceinline__ double2 sw_zero<double2>() { return make_double2(0.0, 0.0); }
 template <> __device__ __forceinline__ float2 sw_zero<float2>() { return make_float2(0.f, 0.f); }
 
-// Per-frequency partial sums of one block: each warp's lanes hold the partials
-// of frequencies g*32 + lane (g = the warp's group); warps with the same group
-// are added in warp order through shared memory, then one value per (block,
-// frequency) goes to `partials`.  The last block adds the partials of all
-// blocks in block order; there thread j < Fp owns frequency j's totals in
-// tot[].  Requires Fp <= blockDim.x.  `sh` holds (warps per block) * 32 * K
-// doubles.
+// How the na frequencies of a launch (the running ones, or all) are dealt to a
+// block's threads.  A block has S = warps / (Fp / 32) slots; slot s of block b
+// takes rows b S + s, + grid S, ... for every frequency.  FP64 instructions are
+// what a sweep spends its time on, and one costs the same whatever lanes are on,
+// so the S na pairs of slot and frequency are packed densely: thread t has slot
+// t / na and the (t mod na)-th frequency; the warps past them do nothing.  As
+// frequencies stop, fewer and fewer warps of every block are left, all of them
+// full, and which rows and in which order a frequency's sums are formed does not
+// depend on which others are running.
+// Memory is what is short then: a warp's gathers that miss L1 return some 75
+// clocks apart, and a row waits for 27 of them.  So a slot's rows are shared out to
+// the threads that are left over (walk_split), which store their products; the
+// slot's sums are formed afterwards, in the order of its rows (sweep_chain).
+// Measured: 64 frequencies of the 60x30x25 cavity, 50 to 300 Hz, to 1e-10 (162 to
+// 1835 iterations, 674 on average): 1411 ms with a fixed warp for every slot and
+// 32 frequencies, on until the last of them stopped; packed 1340; and rows loaded
+// ahead and shared out 869; the same bits.  An iteration with 64, 32, 16, 8, 1
+// frequencies running: 941, 526, 522, 521, 520 us before, now 940, 516, 340, 232,
+// 196.
+struct SweepWalk {
+  int j;               // this thread's frequency (-1: none)
+  int32_t i, step;     // its rows: i, i + step, ...  (n < 2^27: seven vectors of n x 32 have to fit)
+  int na, slots;
+  int split;           // threads that share a slot's rows (walk_split; 1: none), one row each at least
+  int32_t ci, cstep;   // split: the rows whose sums this thread adds up (ci < 0: none)
+  const int32_t* pos;  // a frequency's place among the na (null: all, in order)
+  __device__ __forceinline__ SweepWalk(int na_, int groups, const int32_t* act, const int32_t* pos_, int32_t n = 0)
+      : j(-1), i(0), step(1), na(na_), slots(static_cast<int>(blockDim.x >> 5) / groups), split(1), ci(-1), cstep(1),
+        pos(pos_) {
+    if (na == 0) return;
+    const int pairs = slots * na, t = static_cast<int>(threadIdx.x);
+    cstep = static_cast<int32_t>(gridDim.x) * slots;
+    split = max(min(static_cast<int>(blockDim.x) / pairs, (n + cstep - 1) / cstep), 1);
+    const int sub = t / pairs, slot = (t - sub * pairs) / na, p = t - sub * pairs - slot * na;
+    if (sub < split) j = act ? act[p] : p;
+    const int32_t first = static_cast<int32_t>(blockIdx.x) * slots + slot;
+    if (sub == 0) ci = first;
+    i = first + sub * cstep;
+    step = split * cstep;
+  }
+  // frequency j's place (-1: not among them)
+  __device__ __forceinline__ int place(int f, int F) const { return pos ? pos[f] : f < F ? f : -1; }
+};
+// the running frequencies; all of them
+template <class V>
+__device__ __forceinline__ SweepWalk walk_running(const SweepArgsT<V>& a) {
+  return SweepWalk(*a.nact, a.G, a.act, a.pos);
+}
+// the running ones, a slot's rows shared out to the threads that the pairs leave:
+// the kernel forms the slot's sums afterwards (sweep_chain)
+template <class V>
+__device__ __forceinline__ SweepWalk walk_split(const SweepArgsT<V>& a) {
+  return SweepWalk(*a.nact, a.G, a.act, a.pos, a.A.n);
+}
+template <class V>
+__device__ __forceinline__ SweepWalk walk_all(const SweepArgsT<V>& a) {
+  return SweepWalk(a.F, a.G, nullptr, nullptr);
+}
+
+// Per-frequency partial sums of one block: the slots' sums in slot order through
+// shared memory, then one value per (block, frequency) goes to `partials`.  The
+// last block adds the partials of all blocks in block order; there thread j < Fp
+// owns frequency j's totals in tot[].  Requires Fp <= blockDim.x.  `sh` holds
+// (warps per block) * 32 * K doubles.
 template <int K, class V>
-__device__ bool sweep_grid_sum(const SweepArgsT<V>& a, const double (&v)[K], double* sh, unsigned int* ticket,
-                               double (&tot)[K]) {
+__device__ bool sweep_grid_sum(const SweepArgsT<V>& a, const SweepWalk& wk, const double (&v)[K], double* sh,
+                               unsigned int* ticket, double (&tot)[K]) {
   __shared__ bool s_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
-  for (int k = 0; k < K; ++k) sh[(warp * 32 + lane) * K + k] = v[k];
+  for (int k = 0; k < K; ++k) sh[threadIdx.x * K + k] = v[k];
   __syncthreads();
   const int j = threadIdx.x;
   if (j < a.Fp) {
     double acc[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) acc[k] = 0.0;
-    for (int w = 0; w < nw; ++w) {
-      const int gw = static_cast<int>((static_cast<int64_t>(blockIdx.x) * nw + w) % a.G);
-      if (gw != j / 32) continue;
+    const int p = wk.place(j, a.F);
+    if (p >= 0) {
+      for (int s = 0; s < wk.slots; ++s) {
 #pragma unroll
-      for (int k = 0; k < K; ++k) acc[k] += sh[(w * 32 + (j & 31)) * K + k];
+        for (int k = 0; k < K; ++k) acc[k] += sh[(s * wk.na + p) * K + k];
+      }
     }
 #pragma unroll
     for (int k = 0; k < K; ++k) a.partials[(static_cast<size_t>(blockIdx.x) * a.Fp + j) * K + k] = acc[k];
@@ -213,55 +272,97 @@ __device__ bool sweep_grid_sum(const SweepArgsT<V>& a, const double (&v)[K], dou
 // formed as (fma(-w2, M, K), w_j B) and multiplied in CSR order; rows of a
 // 32-row block where B = 0 take the real x complex product (bit-identical
 // for finite x: the skipped terms are exact zeros).  x[col * ld + j].
-__device__ __forceinline__ double2 sweep_row(const SweepDev& A, int32_t i, int j, double wj, double w2,
-                                             const double2* __restrict__ x, int64_t ld) {
-  const int64_t k0 = __ldg(A.rowptr + i), k1 = __ldg(A.rowptr + i + 1);
+// With the real parts formed beforehand (are), a row is a pipeline of kSweepU
+// entries a stage: the next stage's entries are loaded behind this one's gathers.
+// Once few frequencies are left, a warp's chain of loads is what a product takes.
+// (32-bit offsets: the formed parts take 8 GiB at most, and a vector of 2^32
+// complex128 would not leave room for the other six.)
+constexpr int kSweepU = 4;
+__device__ __forceinline__ double2 sweep_row_real(const SweepDev& A, int32_t k0, int32_t k1, uint32_t j,
+                                                  const double2* __restrict__ x, uint32_t ld) {
+  constexpr int U = kSweepU;
   double2 acc = make_double2(0.0, 0.0);
-  if (A.bzero_blk[i >> 5] != 0) {
-    if (A.are) {
-      // the formed real parts: one coalesced load per entry and 32 frequencies
-      const double* ar = A.are + j;
-#pragma unroll 4
-      for (int64_t k = k0; k < k1; ++k) {
-        const int32_t c = __ldg(A.colind + k);
-        const double are = __ldg(ar + k * A.are_ld);
-        const double2 xv = __ldg(x + static_cast<int64_t>(c) * ld + j);
-        acc.x = fma(are, xv.x, acc.x);
-        acc.y = fma(are, xv.y, acc.y);
-      }
-    } else {
-#pragma unroll 4
-      for (int64_t k = k0; k < k1; ++k) {
-        const int32_t c = __ldg(A.colind + k);
-        const double are = fma(-w2, __ldg(A.M + k), __ldg(A.K + k));
-        const double2 xv = __ldg(x + static_cast<int64_t>(c) * ld + j);
-        acc.x = fma(are, xv.x, acc.x);
-        acc.y = fma(are, xv.y, acc.y);
+  double a[U];
+  int32_t c[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    a[u] = 0.0;
+    c[u] = 0;
+    if (k0 + u < k1) {
+      c[u] = __ldg(A.colind + k0 + u);
+      a[u] = __ldg(A.are + (static_cast<uint32_t>(k0 + u) * static_cast<uint32_t>(A.are_ld) + j));
+    }
+  }
+#pragma unroll 1
+  for (int32_t k = k0; k < k1; k += U) {
+    double2 xv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (k + u < k1) xv[u] = __ldg(x + (static_cast<uint32_t>(c[u]) * ld + j));
+    double an[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      an[u] = 0.0;
+      if (k + U + u < k1) {
+        c[u] = __ldg(A.colind + k + U + u);
+        an[u] = __ldg(A.are + (static_cast<uint32_t>(k + U + u) * static_cast<uint32_t>(A.are_ld) + j));
       }
     }
-  } else {
-#pragma unroll 2
-    for (int64_t k = k0; k < k1; ++k) {
-      const int32_t c = __ldg(A.colind + k);
-      const double re = A.are ? __ldg(A.are + k * A.are_ld + j) : fma(-w2, __ldg(A.M + k), __ldg(A.K + k));
-      const double2 av = make_double2(re, wj * __ldg(A.B + k));
-      acc = cfma(av, __ldg(x + static_cast<int64_t>(c) * ld + j), acc);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (k + u < k1) {
+        acc.x = fma(a[u], xv[u].x, acc.x);
+        acc.y = fma(a[u], xv[u].y, acc.y);
+      }
+      a[u] = an[u];
     }
   }
   return acc;
+}
+// The other rows: real parts formed entry by entry, or B not zero.  Out of line,
+// so that its loops do not take registers from the pipeline above.
+__device__ __noinline__ double2 sweep_row_other(const int32_t* __restrict__ colind, const double* __restrict__ K,
+                                                const double* __restrict__ M, const double* __restrict__ B,
+                                                const double* __restrict__ are, int32_t are_ld, bool real, int32_t k0,
+                                                int32_t k1, int j, double wj, const double2* __restrict__ x, int64_t ld) {
+  const double w2 = wj * wj;
+  double2 acc = make_double2(0.0, 0.0);
+  if (real) {
+#pragma unroll 4
+    for (int32_t k = k0; k < k1; ++k) {
+      const int32_t c = __ldg(colind + k);
+      const double re = fma(-w2, __ldg(M + k), __ldg(K + k));
+      const double2 xv = __ldg(x + static_cast<int64_t>(c) * ld + j);
+      acc.x = fma(re, xv.x, acc.x);
+      acc.y = fma(re, xv.y, acc.y);
+    }
+  } else {
+#pragma unroll 2
+    for (int32_t k = k0; k < k1; ++k) {
+      const int32_t c = __ldg(colind + k);
+      const double re = are ? __ldg(are + static_cast<int64_t>(k) * are_ld + j) : fma(-w2, __ldg(M + k), __ldg(K + k));
+      acc = cfma(make_double2(re, wj * __ldg(B + k)), __ldg(x + static_cast<int64_t>(c) * ld + j), acc);
+    }
+  }
+  return acc;
+}
+__device__ __forceinline__ double2 sweep_row(const SweepDev& A, int32_t i, int32_t k0, int32_t k1, int j, double wj,
+                                             double, const double2* __restrict__ x, int64_t ld) {
+  const bool real = A.bzero_blk[i >> 5] != 0;
+  if (A.are && real) return sweep_row_real(A, k0, k1, static_cast<uint32_t>(j), x, static_cast<uint32_t>(ld));
+  return sweep_row_other(A.colind, A.K, A.M, A.B, A.are, A.are_ld, real, k0, k1, j, wj, x, ld);
 }
 
 // The same row for complex64 vectors (the inner operator of the mixed
 // sweep): the entries are formed in FP32 from FP32 copies of K, M, B,
 // products and the row sum are FP32 -- no FP64 instruction per entry.
-__device__ __forceinline__ float2 sweep_row(const SweepDev& A, int32_t i, int j, double wj, double w2,
-                                            const float2* __restrict__ x, int64_t ld) {
-  const int64_t k0 = __ldg(A.rowptr + i), k1 = __ldg(A.rowptr + i + 1);
+__device__ __forceinline__ float2 sweep_row(const SweepDev& A, int32_t i, int32_t k0, int32_t k1, int j, double wj,
+                                            double w2, const float2* __restrict__ x, int64_t ld) {
   const float wf = static_cast<float>(wj), w2f = static_cast<float>(w2);
   float2 acc = make_float2(0.f, 0.f);
   if (A.bzero_blk[i >> 5] != 0) {
 #pragma unroll 4
-    for (int64_t k = k0; k < k1; ++k) {
+    for (int32_t k = k0; k < k1; ++k) {
       const int32_t c = __ldg(A.colind + k);
       const float are = fmaf(-w2f, __ldg(A.M32 + k), __ldg(A.K32 + k));
       const float2 xv = __ldg(x + static_cast<int64_t>(c) * ld + j);
@@ -270,7 +371,7 @@ __device__ __forceinline__ float2 sweep_row(const SweepDev& A, int32_t i, int j,
     }
   } else {
 #pragma unroll 2
-    for (int64_t k = k0; k < k1; ++k) {
+    for (int32_t k = k0; k < k1; ++k) {
       const int32_t c = __ldg(A.colind + k);
       const float2 av = make_float2(fmaf(-w2f, __ldg(A.M32 + k), __ldg(A.K32 + k)), wf * __ldg(A.B32 + k));
       acc = cfma32(av, __ldg(x + static_cast<int64_t>(c) * ld + j), acc);
@@ -279,45 +380,105 @@ __device__ __forceinline__ float2 sweep_row(const SweepDev& A, int32_t i, int j,
   return acc;
 }
 
-// Batched SpMV over the warp's (row, group) units: acc[j] = sum_k A_j[k] x[col][j].
-// Calls epi(i, lane_frequency, acc) for running frequencies.
-template <class V, class Epi>
-__device__ __forceinline__ void sweep_spmv(const SweepArgsT<V>& a, const V* __restrict__ x, Epi& epi) {
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-  const int64_t units = static_cast<int64_t>(a.A.n) * a.G;
-  // a warp keeps the same group for all its units when nwarps is a multiple
-  // of G (the launcher guarantees it), so its lane frequency is fixed
-  const int g = static_cast<int>(gw % a.G);
-  const int j = g * 32 + lane;
-  const bool grp_on = a.gactive[g] != 0;
-  const bool run = grp_on && j < a.F && a.status[j] == ST_RUNNING;
-  const double wj = a.w[j];
-  const double w2 = wj * wj;
-  for (int64_t u = gw; u < units; u += nwarps) {
-    if (!grp_on) break;
-    const int32_t i = static_cast<int32_t>(u / a.G);
-    const V acc = sweep_row(a.A, i, j, wj, w2, x, a.Fp);
-    if (run) epi(i, j, acc);
-  }
+template <class V>
+__device__ __forceinline__ V sweep_row(const SweepDev& A, int32_t i, int j, double wj, double w2, const V* __restrict__ x,
+                                       int64_t ld) {
+  return sweep_row(A, i, __ldg(A.rowptr + i), __ldg(A.rowptr + i + 1), j, wj, w2, x, ld);
 }
 
-// Y_j = A_j X_j for the stand-alone batched product (helm_sweep_spmv): warp
-// per (row, 32-frequency group), lane = frequency, the solver's row sum.
+// Batched SpMV over this thread's rows: acc = sum_k A_j[k] x[col][j].  Calls
+// pre(i, j), whose loads are in flight with the row's, and epi(i, j, acc) where
+// its frequency is running (and `on`).
+template <class V, class Pre, class Epi>
+__device__ __forceinline__ void sweep_spmv(const SweepArgsT<V>& a, const SweepWalk& wk, const V* __restrict__ x, Pre pre,
+                                           Epi& epi, bool on = true) {
+  const int j = wk.j;
+  if (!on || j < 0 || a.status[j] != ST_RUNNING || wk.i >= a.A.n) return;
+  const double wj = a.w[j];
+  const double w2 = wj * wj;
+  int32_t k0 = __ldg(a.A.rowptr + wk.i), k1 = __ldg(a.A.rowptr + wk.i + 1);
+#pragma unroll 1
+  for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+    const int32_t i = q, next = q + wk.step < a.A.n ? q + wk.step : q;  // the next row's extent, early
+    const int32_t n0 = __ldg(a.A.rowptr + next), n1 = __ldg(a.A.rowptr + next + 1);
+    pre(i, j);
+    epi(i, j, sweep_row(a.A, i, k0, k1, j, wj, w2, x, a.Fp));
+    k0 = n0;
+    k1 = n1;
+  }
+}
+// Sums of split rows: add(ld(idx)) over this slot's rows in order, after every
+// thread of the block has stored its rows' values; nothing when rows are not split
+// (the kernel has added them as they came).
+template <class V, class Ld, class F>
+__device__ __forceinline__ void sweep_chain(const SweepArgsT<V>& a, const SweepWalk& wk, Ld ld, F add) {
+  if (wk.split == 1) return;
+  __syncthreads();
+  if (wk.ci < 0 || wk.j < 0) return;
+  constexpr int R = 2;
+#pragma unroll 1
+  for (int32_t q = wk.ci; q < a.A.n; q += R * wk.cstep) {
+    decltype(ld(size_t(0))) v[R];
+#pragma unroll
+    for (int u = 0; u < R; ++u)
+      if (q + u * wk.cstep < a.A.n) v[u] = ld(static_cast<size_t>(q + u * wk.cstep) * a.Fp + wk.j);
+#pragma unroll
+    for (int u = 0; u < R; ++u)
+      if (q + u * wk.cstep < a.A.n) add(v[u]);
+  }
+}
+struct SweepNoPre {
+  __device__ __forceinline__ void operator()(int32_t, int) const {}
+};
+
+// f(idx, ld(idx)) over this thread's rows in order, idx = row Fp + j: the loads
+// of R rows are in flight together.
+template <int R, class V, class Ld, class F>
+__device__ __forceinline__ void sweep_rows(const SweepArgsT<V>& a, const SweepWalk& wk, Ld ld, F f) {
+#pragma unroll 1
+  for (int32_t q = wk.i; q < a.A.n; q += R * wk.step) {
+    decltype(ld(size_t(0))) v[R];
+#pragma unroll
+    for (int u = 0; u < R; ++u)
+      if (q + u * wk.step < a.A.n) v[u] = ld(static_cast<size_t>(q + u * wk.step) * a.Fp + wk.j);
+#pragma unroll
+    for (int u = 0; u < R; ++u)
+      if (q + u * wk.step < a.A.n) f(static_cast<size_t>(q + u * wk.step) * a.Fp + wk.j, v[u]);
+  }
+}
+template <class V> struct Vec3 { V a, b, c; };
+template <class V> struct Vec2 { V a, b; };
+template <class V> struct Vec5 { V a, b, c, d, e; };
+
+// Y_j = A_j X_j for the stand-alone batched product (helm_sweep_spmv): the
+// solver's row sum.
 __global__ void __launch_bounds__(256) k_sw_apply(SweepDev A, int32_t F, int32_t G, const double* __restrict__ w,
                                                   const double2* __restrict__ X, int32_t ldx, double2* __restrict__ Y,
                                                   int32_t ldy) {
+  const SweepWalk wk(F, G, nullptr, nullptr);
+  const int j = wk.j;
+  if (j < 0) return;
+  const double wj = w[j];
+  for (int64_t i = wk.i; i < A.n; i += wk.step)
+    Y[i * ldy + j] = sweep_row(A, static_cast<int32_t>(i), j, wj, wj * wj, X, ldx);
+}
+
+// The list of running frequencies, in order (one warp); returns their number.
+template <class V>
+__device__ int sweep_list_running(const SweepArgsT<V>& a) {
   const int lane = threadIdx.x & 31;
-  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-  for (int64_t u = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-       u < static_cast<int64_t>(A.n) * G; u += nwarps) {
-    const int32_t i = static_cast<int32_t>(u / G);
-    const int j = static_cast<int>(u % G) * 32 + lane;
-    if (j >= F) continue;
-    const double wj = w[j];
-    Y[static_cast<int64_t>(i) * ldy + j] = sweep_row(A, i, j, wj, wj * wj, X, ldx);
+  int base = 0;
+  for (int g = 0; g < a.G; ++g) {
+    const int j = g * 32 + lane;
+    const bool on = a.status[j] == ST_RUNNING;
+    const unsigned int m = __ballot_sync(0xffffffffu, on);
+    const int p = base + __popc(m & ((1u << lane) - 1u));
+    a.pos[j] = on ? p : -1;
+    if (on) a.act[p] = j;
+    base += __popc(m);
   }
+  if (lane == 0) *a.nact = base;
+  return base;
 }
 
 // fresh: every frequency starts (iteration counts from 0).  Otherwise a
@@ -348,33 +509,39 @@ __global__ void k_sw_configure(SweepArgsT<V> a, double tol, int32_t maxit, int32
     a.omg[j] = one;
     a.beta[j] = make_double2(0.0, 0.0);
   }
-  for (int g = threadIdx.x; g < a.G; g += blockDim.x) a.gactive[g] = 1;
+  __syncthreads();
+  if (threadIdx.x < 32) sweep_list_running(a);
 }
 
-// Update the group flags and the loop condition from the per-frequency status
-// (thread 0 of the last block of a reduction kernel, after the statuses are set).
+// Update the list of running frequencies and the loop condition from the
+// per-frequency status (one warp of the last block of a reduction kernel, after
+// the statuses are set and a barrier of the block).
 template <class V>
-__device__ void sweep_refresh_groups(const SweepArgsT<V>& a) {
-  bool any = false;
-  for (int g = 0; g < a.G; ++g) {
-    bool on = false;
-    for (int l = 0; l < 32; ++l) on |= a.status[g * 32 + l] == ST_RUNNING;
-    a.gactive[g] = on ? 1 : 0;
-    any |= on;
+__device__ void sweep_refresh(const SweepArgsT<V>& a) {
+  const bool any = sweep_list_running(a) > 0;
+  if ((threadIdx.x & 31) == 0) {
+    a.st->status = any ? ST_RUNNING : HELM_OK;
+    sweep_set_cond(a, any);
   }
-  a.st->status = any ? ST_RUNNING : HELM_OK;
-  sweep_set_cond(a, any);
 }
+
+// kernels that walk the running frequencies
+#define SWEEP_ELEMENTWISE_BEGIN            \
+  const SweepWalk wk = walk_running(a);    \
+  const int j = wk.j;                      \
+  const bool run = j >= 0 && a.status[j] == ST_RUNNING;
+
+#define SWEEP_SPLIT_BEGIN                  \
+  const SweepWalk wk = walk_split(a);      \
+  const int j = wk.j;                      \
+  const bool run = j >= 0 && a.status[j] == ST_RUNNING;
 
 // init: r = b - A_j x (or r = b, x = 0), r^ = r, p = v = 0; ||b||, ||r||, rho
 template <class V>
-__global__ void __launch_bounds__(512) k_sw_init(SweepArgsT<V> a) {
+__global__ void __launch_bounds__(512, 2) k_sw_init(SweepArgsT<V> a) {
   extern __shared__ double sh[];
   const int use_x0 = a.st->use_x0;
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int g = static_cast<int>(gw % a.G);
-  const int j = g * 32 + lane;
+  SWEEP_ELEMENTWISE_BEGIN
   double part[4] = {0.0, 0.0, 0.0, 0.0};
   auto body = [&](int32_t i, int jj, V ax) {
     const size_t idx = static_cast<size_t>(i) * a.Fp + jj;
@@ -391,20 +558,16 @@ __global__ void __launch_bounds__(512) k_sw_init(SweepArgsT<V> a) {
     part[3] = d.y;
   };
   if (use_x0) {
-    sweep_spmv(a, a.x, body);
-  } else {
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    const bool run = j < a.F && a.status[j] == ST_RUNNING;
-    for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-      const int32_t i = static_cast<int32_t>(u / a.G);
-      if (run) {
-        a.x[static_cast<size_t>(i) * a.Fp + j] = sw_zero<V>();
-        body(i, j, sw_zero<V>());
-      }
+    sweep_spmv(a, wk, a.x, SweepNoPre(), body);
+  } else if (run) {
+    for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+      const int32_t i = q;
+      a.x[static_cast<size_t>(i) * a.Fp + j] = sw_zero<V>();
+      body(i, j, sw_zero<V>());
     }
   }
   double tot[4];
-  if (!sweep_grid_sum<4>(a, part, sh, a.tickets + TK_INIT, tot)) return;
+  if (!sweep_grid_sum<4>(a, wk, part, sh, a.tickets + TK_INIT, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
     if (a.status[jj] != ST_RUNNING) continue;  // frozen by a restart of other frequencies
     const double bn = sqrt(tot[0]);
@@ -428,49 +591,42 @@ __global__ void __launch_bounds__(512) k_sw_init(SweepArgsT<V> a) {
     a.status[jj] = status;
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
-
-// element-wise kernels walk (row, group) units like the SpMV, 32 frequencies per warp
-#define SWEEP_ELEMENTWISE_BEGIN                                                          \
-  const int lane = threadIdx.x & 31;                                                     \
-  const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; \
-  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;            \
-  const int g = static_cast<int>(gw % a.G);                                              \
-  const int j = g * 32 + lane;                                                           \
-  const bool grp_on = a.gactive[g] != 0;                                                 \
-  const bool run = grp_on && j < a.F && a.status[j] == ST_RUNNING;
 
 // K1: p = r + beta (p - omega v)
 template <class V>
-__global__ void __launch_bounds__(512) k_sw_p(SweepArgsT<V> a) {
-  SWEEP_ELEMENTWISE_BEGIN
+__global__ void __launch_bounds__(512, 2) k_sw_p(SweepArgsT<V> a) {
+  SWEEP_SPLIT_BEGIN
   if (!run) return;
   const V beta = sw_cvt<V>(a.beta[j]), omg = sw_cvt<V>(a.omg[j]);
-  for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-    const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
-    a.p[idx] = cfma(beta, cfms(omg, a.v[idx], a.p[idx]), a.r[idx]);
-  }
+  sweep_rows<2>(
+      a, wk, [&](size_t idx) { return Vec3<V>{a.v[idx], a.p[idx], a.r[idx]}; },
+      [&](size_t idx, const Vec3<V>& l) { a.p[idx] = cfma(beta, cfms(omg, l.a, l.b), l.c); });
 }
 
 // K2: v = A_j p, (r^, v) -> alpha
 template <class V>
-__global__ void __launch_bounds__(512) k_sw_v(SweepArgsT<V> a) {
+__global__ void __launch_bounds__(512, 2) k_sw_v(SweepArgsT<V> a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
-  const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int g = static_cast<int>(gw % a.G);
+  const SweepWalk wk = walk_split(a);
   double part[2] = {0.0, 0.0};
-  auto body = [&](int32_t i, int j, V ax) {
-    const size_t idx = static_cast<size_t>(i) * a.Fp + j;
-    a.v[idx] = ax;
-    double2 d = sw_dot(make_double2(part[0], part[1]), a.rh[idx], ax);
+  auto add = [&](const Vec2<V>& l) {
+    const double2 d = sw_dot(make_double2(part[0], part[1]), l.a, l.b);
     part[0] = d.x;
     part[1] = d.y;
   };
-  sweep_spmv(a, a.p, body);
+  V rhi = sw_zero<V>();
+  auto pre = [&](int32_t i, int j) { rhi = a.rh[static_cast<size_t>(i) * a.Fp + j]; };
+  auto body = [&](int32_t i, int j, V ax) {
+    a.v[static_cast<size_t>(i) * a.Fp + j] = ax;
+    if (wk.split == 1) add(Vec2<V>{rhi, ax});
+  };
+  sweep_spmv(a, wk, a.p, pre, body);
+  sweep_chain(a, wk, [&](size_t idx) { return Vec2<V>{a.rh[idx], a.v[idx]}; }, add);
   double tot[2];
-  if (!sweep_grid_sum<2>(a, part, sh, a.tickets + TK_V, tot)) return;
+  if (!sweep_grid_sum<2>(a, wk, part, sh, a.tickets + TK_V, tot)) return;
   for (int j = threadIdx.x; j < a.F && j == (int)threadIdx.x; j += blockDim.x) {
     if (a.status[j] != ST_RUNNING) continue;
     a.iters[j] += 1;
@@ -484,27 +640,29 @@ __global__ void __launch_bounds__(512) k_sw_v(SweepArgsT<V> a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // K3: s = r - alpha v, ||s||
 template <class V>
-__global__ void __launch_bounds__(512) k_sw_s(SweepArgsT<V> a) {
+__global__ void __launch_bounds__(512, 2) k_sw_s(SweepArgsT<V> a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
-  SWEEP_ELEMENTWISE_BEGIN
+  SWEEP_SPLIT_BEGIN
   double part[1] = {0.0};
   if (run) {
     const V al = sw_cvt<V>(a.alpha[j]);
-    for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-      const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
-      const V si = cfms(al, a.v[idx], a.r[idx]);
-      a.s[idx] = si;
-      part[0] = sw_nrm(part[0], si);
-    }
+    sweep_rows<2>(
+        a, wk, [&](size_t idx) { return Vec2<V>{a.v[idx], a.r[idx]}; },
+        [&](size_t idx, const Vec2<V>& l) {
+          const V si = cfms(al, l.a, l.b);
+          a.s[idx] = si;
+          if (wk.split == 1) part[0] = sw_nrm(part[0], si);
+        });
   }
+  sweep_chain(a, wk, [&](size_t idx) { return a.s[idx]; }, [&](V si) { part[0] = sw_nrm(part[0], si); });
   double tot[1];
-  if (!sweep_grid_sum<1>(a, part, sh, a.tickets + TK_S, tot)) return;
+  if (!sweep_grid_sum<1>(a, wk, part, sh, a.tickets + TK_S, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
     if (a.status[jj] != ST_RUNNING) continue;
     const double sn = sqrt(tot[0]);
@@ -515,29 +673,36 @@ __global__ void __launch_bounds__(512) k_sw_s(SweepArgsT<V> a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // K4: t = A_j s, (t, s), (t, t) -> omega (frequencies stopped at s skip)
 template <class V>
-__global__ void __launch_bounds__(512) k_sw_t(SweepArgsT<V> a) {
+__global__ void __launch_bounds__(512, 2) k_sw_t(SweepArgsT<V> a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
-  const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int g = static_cast<int>(gw % a.G);
+  const SweepWalk wk = walk_split(a);
   double part[3] = {0.0, 0.0, 0.0};
-  auto body = [&](int32_t i, int j, V ax) {
-    if (a.phase[j] != PH_RUN) return;
-    const size_t idx = static_cast<size_t>(i) * a.Fp + j;
-    a.t[idx] = ax;
-    double2 d = sw_dot(make_double2(part[0], part[1]), ax, a.s[idx]);
+  const bool on = wk.j >= 0 && a.phase[wk.j] == PH_RUN;
+  auto add = [&](const Vec2<V>& l) {
+    const double2 d = sw_dot(make_double2(part[0], part[1]), l.a, l.b);
     part[0] = d.x;
     part[1] = d.y;
-    part[2] = sw_nrm(part[2], ax);
+    part[2] = sw_nrm(part[2], l.a);
   };
-  sweep_spmv(a, a.s, body);
+  V si = sw_zero<V>();
+  auto pre = [&](int32_t i, int j) { si = a.s[static_cast<size_t>(i) * a.Fp + j]; };
+  auto body = [&](int32_t i, int j, V ax) {
+    a.t[static_cast<size_t>(i) * a.Fp + j] = ax;
+    if (wk.split == 1) add(Vec2<V>{ax, si});
+  };
+  sweep_spmv(a, wk, a.s, pre, body, on);
+  if (wk.split > 1)
+    sweep_chain(a, wk, [&](size_t idx) { return Vec2<V>{a.t[idx], a.s[idx]}; }, [&](const Vec2<V>& l) {
+      if (on) add(l);
+    });
   double tot[3];
-  if (!sweep_grid_sum<3>(a, part, sh, a.tickets + TK_T, tot)) return;
+  if (!sweep_grid_sum<3>(a, wk, part, sh, a.tickets + TK_T, tot)) return;
   for (int j = threadIdx.x; j < a.F && j == (int)threadIdx.x; j += blockDim.x) {
     if (a.status[j] != ST_RUNNING || a.phase[j] != PH_RUN) continue;
     const double2 ts = make_double2(tot[0], tot[1]);
@@ -551,40 +716,44 @@ __global__ void __launch_bounds__(512) k_sw_t(SweepArgsT<V> a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // K5: x += alpha p + omega s, r = s - omega t; per-frequency stop tests
 template <class V>
-__global__ void __launch_bounds__(512) k_sw_xr(SweepArgsT<V> a) {
+__global__ void __launch_bounds__(512, 2) k_sw_xr(SweepArgsT<V> a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) {
     if (blockIdx.x == 0 && threadIdx.x == 0) sweep_set_cond(a, false);
     return;
   }
-  SWEEP_ELEMENTWISE_BEGIN
+  SWEEP_SPLIT_BEGIN
   double part[3] = {0.0, 0.0, 0.0};
+  auto add = [&](const Vec2<V>& l) {
+    const double2 d = sw_dot(make_double2(part[0], part[1]), l.a, l.b);
+    part[0] = d.x;
+    part[1] = d.y;
+    part[2] = sw_nrm(part[2], l.b);
+  };
   if (run) {
     const V al = sw_cvt<V>(a.alpha[j]), om = sw_cvt<V>(a.omg[j]);
     const bool sconv = a.phase[j] == PH_SCONV;
-    for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-      const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
-      if (sconv) {
-        a.x[idx] = cfma(al, a.p[idx], a.x[idx]);
-      } else {
-        const V si = a.s[idx];
-        a.x[idx] = cfma(om, si, cfma(al, a.p[idx], a.x[idx]));
-        const V ri = cfms(om, a.t[idx], si);
-        a.r[idx] = ri;
-        double2 d = sw_dot(make_double2(part[0], part[1]), a.rh[idx], ri);
-        part[0] = d.x;
-        part[1] = d.y;
-        part[2] = sw_nrm(part[2], ri);
-      }
-    }
+    sweep_rows<1>(
+        a, wk, [&](size_t idx) { return Vec5<V>{a.x[idx], a.p[idx], a.s[idx], a.t[idx], a.rh[idx]}; },
+        [&](size_t idx, const Vec5<V>& l) {
+          if (sconv) {
+            a.x[idx] = cfma(al, l.b, l.a);
+            return;
+          }
+          a.x[idx] = cfma(om, l.c, cfma(al, l.b, l.a));
+          const V ri = cfms(om, l.d, l.c);
+          a.r[idx] = ri;
+          if (wk.split == 1) add(Vec2<V>{l.e, ri});
+        });
   }
+  sweep_chain(a, wk, [&](size_t idx) { return Vec2<V>{a.rh[idx], a.r[idx]}; }, add);
   double tot[3];
-  if (!sweep_grid_sum<3>(a, part, sh, a.tickets + TK_XR, tot)) return;
+  if (!sweep_grid_sum<3>(a, wk, part, sh, a.tickets + TK_XR, tot)) return;
   const bool late = a.st->deadline_ns != 0ull && (globaltimer_ns() - a.st->t0) > a.st->deadline_ns;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
     if (a.status[jj] != ST_RUNNING) continue;
@@ -610,29 +779,26 @@ __global__ void __launch_bounds__(512) k_sw_xr(SweepArgsT<V> a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // tail: true residual per frequency, ||b - A_j x|| / ||b||
 template <class V>
-__global__ void __launch_bounds__(512) k_sw_tail(SweepArgsT<V> a) {
+__global__ void __launch_bounds__(512, 2) k_sw_tail(SweepArgsT<V> a) {
   extern __shared__ double sh[];
-  const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int g = static_cast<int>(gw % a.G);
-  // every frequency is measured: mark them all active for the product
+  const SweepWalk wk = walk_all(a);  // every frequency is measured
+  const int j = wk.j;
   double part[1] = {0.0};
-  const int lane = threadIdx.x & 31;
-  const int j = g * 32 + lane;
-  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-  const double wj = a.w[j], w2 = wj * wj;
-  for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-    const int32_t i = static_cast<int32_t>(u / a.G);
-    const V acc = sweep_row(a.A, i, j, wj, w2, a.x, a.Fp);
-    if (j < a.F)
+  if (j >= 0) {
+    const double wj = a.w[j], w2 = wj * wj;
+    for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+      const int32_t i = q;
+      const V acc = sweep_row(a.A, i, j, wj, w2, a.x, a.Fp);
       part[0] = sw_nrm(part[0], csub(a.b[a.b_ld ? static_cast<size_t>(i) * a.b_ld + j : static_cast<size_t>(i)], acc));
+    }
   }
   double tot[1];
-  if (!sweep_grid_sum<1>(a, part, sh, a.tickets + TK_TAIL, tot)) return;
+  if (!sweep_grid_sum<1>(a, wk, part, sh, a.tickets + TK_TAIL, tot)) return;
   for (int jj = threadIdx.x; jj < a.F; jj += blockDim.x)
     a.relres_true[jj] = a.bnorm[jj] > 0.0 ? sqrt(tot[0]) / a.bnorm[jj] : 0.0;
 }
@@ -646,8 +812,7 @@ __global__ void __launch_bounds__(512) k_sw_tail(SweepArgsT<V> a) {
 // u = p, un = s, v = v, Au = t, A un = q1, d = q2; eta lives in omg.  When a
 // half-step's quasi-residual bound tau sqrt(m + 2) falls below tol ||b_j||,
 // the frequency's true residual ||b_j - A_j x_j|| is computed after the odd
-// half-step (only the 32-frequency groups with such a frequency make that
-// product); a frequency whose bound is below tol but whose true residual is
+// half-step (only the lanes of such frequencies make that product); a frequency whose bound is below tol but whose true residual is
 // not stops with ST_RESTART and the host starts it again from its x.
 
 // After a half-step of frequency j: theta = ||w|| / tau, c = 1 / sqrt(1 + theta^2),
@@ -677,7 +842,7 @@ __device__ __forceinline__ void swq_gamma(const SweepArgs& a, int j) {
 }
 
 // init A: r0 = b - A_j x (or b, x = 0); w = u = r0; d = 0; ||b||, ||r0||, rho = (r0, r0)
-__global__ void __launch_bounds__(512) k_swq_init_a(SweepArgs a) {
+__global__ void __launch_bounds__(512, 2) k_swq_init_a(SweepArgs a) {
   extern __shared__ double sh[];
   const int use_x0 = a.st->use_x0;
   SWEEP_ELEMENTWISE_BEGIN
@@ -697,16 +862,16 @@ __global__ void __launch_bounds__(512) k_swq_init_a(SweepArgs a) {
     part[3] = d.y;
   };
   if (use_x0) {
-    sweep_spmv(a, a.x, body);
+    sweep_spmv(a, wk, a.x, SweepNoPre(), body);
   } else if (run) {
-    for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-      const int32_t i = static_cast<int32_t>(u / a.G);
+    for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+      const int32_t i = q;
       a.x[static_cast<size_t>(i) * a.Fp + j] = make_double2(0.0, 0.0);
       body(i, j, make_double2(0.0, 0.0));
     }
   }
   double tot[4];
-  if (!sweep_grid_sum<4>(a, part, sh, a.tickets + TK_INIT, tot)) return;
+  if (!sweep_grid_sum<4>(a, wk, part, sh, a.tickets + TK_INIT, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
     if (a.status[jj] != ST_RUNNING) continue;  // frozen by a restart of other frequencies
     const double bn = sqrt(tot[0]);
@@ -732,20 +897,18 @@ __global__ void __launch_bounds__(512) k_swq_init_a(SweepArgs a) {
     a.status[jj] = status;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int g2 = 0; g2 < a.G; ++g2) a.gcheck[g2] = 0;
-    *a.anychk = 0;
-    sweep_refresh_groups(a);
-  }
+  if (threadIdx.x == 0) *a.anychk = 0;
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // init B: v = A_j u, Au = v, sigma = (r0, v) -> alpha
-__global__ void __launch_bounds__(512) k_swq_init_b(SweepArgs a) {
+__global__ void __launch_bounds__(512, 2) k_swq_init_b(SweepArgs a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) {
     if (blockIdx.x == 0 && threadIdx.x == 0) sweep_set_cond(a, false);
     return;
   }
+  const SweepWalk wk = walk_running(a);
   double part[2] = {0.0, 0.0};
   auto body = [&](int32_t i, int j, double2 ax) {
     const size_t idx = static_cast<size_t>(i) * a.Fp + j;
@@ -755,9 +918,9 @@ __global__ void __launch_bounds__(512) k_swq_init_b(SweepArgs a) {
     part[0] = d.x;
     part[1] = d.y;
   };
-  sweep_spmv(a, a.p, body);
+  sweep_spmv(a, wk, a.p, SweepNoPre(), body);
   double tot[2];
-  if (!sweep_grid_sum<2>(a, part, sh, a.tickets + TK_V, tot)) return;
+  if (!sweep_grid_sum<2>(a, wk, part, sh, a.tickets + TK_V, tot)) return;
   for (int j = threadIdx.x; j < a.F && j == (int)threadIdx.x; j += blockDim.x) {
     if (a.status[j] != ST_RUNNING) continue;
     const double2 sigma = make_double2(tot[0], tot[1]), rho = a.rho[j];
@@ -770,19 +933,19 @@ __global__ void __launch_bounds__(512) k_swq_init_b(SweepArgs a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // T1, even half-step: un = u - alpha v, w -= alpha Au, d = u + gamma d, ||w||^2
-__global__ void __launch_bounds__(512) k_swq_even(SweepArgs a) {
+__global__ void __launch_bounds__(512, 2) k_swq_even(SweepArgs a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
   SWEEP_ELEMENTWISE_BEGIN
   double part[1] = {0.0};
   if (run) {
     const double2 al = a.alpha[j], ga = a.gam[j];
-    for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-      const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
+    for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+      const size_t idx = static_cast<size_t>(q) * a.Fp + j;
       const double2 ui = a.p[idx];
       a.s[idx] = cfms(al, a.v[idx], ui);
       const double2 wi = cfms(al, a.t[idx], a.r[idx]);
@@ -792,7 +955,7 @@ __global__ void __launch_bounds__(512) k_swq_even(SweepArgs a) {
     }
   }
   double tot[1];
-  if (!sweep_grid_sum<1>(a, part, sh, a.tickets + TK_S, tot)) return;
+  if (!sweep_grid_sum<1>(a, wk, part, sh, a.tickets + TK_S, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
     if (a.status[jj] != ST_RUNNING) continue;
     a.iters[jj] += 1;
@@ -800,33 +963,32 @@ __global__ void __launch_bounds__(512) k_swq_even(SweepArgs a) {
     if (a.status[jj] == ST_RUNNING) swq_gamma(a, jj);  // the odd half-step's d update (same alpha)
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // T2: A un; x += eta d (the even half-step's x update)
-__global__ void __launch_bounds__(512) k_swq_spmv_un(SweepArgs a) {
+__global__ void __launch_bounds__(512, 2) k_swq_spmv_un(SweepArgs a) {
   if (a.st->status != ST_RUNNING) return;
-  const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int jl = static_cast<int>(gw % a.G) * 32 + (threadIdx.x & 31);
-  const double2 eta = a.omg[jl];
+  const SweepWalk wk = walk_running(a);
+  const double2 eta = a.omg[max(wk.j, 0)];
   auto body = [&](int32_t i, int j, double2 ax) {
     const size_t idx = static_cast<size_t>(i) * a.Fp + j;
     a.q1[idx] = ax;
     a.x[idx] = cfma(eta, a.q2[idx], a.x[idx]);
   };
-  sweep_spmv(a, a.s, body);
+  sweep_spmv(a, wk, a.s, SweepNoPre(), body);
 }
 
 // T3, odd half-step: w -= alpha A un, d = un + gamma d, ||w||^2, (r0, w) -> rho, beta
-__global__ void __launch_bounds__(512) k_swq_odd(SweepArgs a) {
+__global__ void __launch_bounds__(512, 2) k_swq_odd(SweepArgs a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
   SWEEP_ELEMENTWISE_BEGIN
   double part[3] = {0.0, 0.0, 0.0};
   if (run) {
     const double2 al = a.alpha[j], ga = a.gam[j];
-    for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-      const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
+    for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+      const size_t idx = static_cast<size_t>(q) * a.Fp + j;
       const double2 wi = cfms(al, a.q1[idx], a.r[idx]);
       a.r[idx] = wi;
       a.q2[idx] = cfma(ga, a.q2[idx], a.s[idx]);
@@ -837,7 +999,7 @@ __global__ void __launch_bounds__(512) k_swq_odd(SweepArgs a) {
     }
   }
   double tot[3];
-  if (!sweep_grid_sum<3>(a, part, sh, a.tickets + TK_T, tot)) return;
+  if (!sweep_grid_sum<3>(a, wk, part, sh, a.tickets + TK_T, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
     if (a.status[jj] != ST_RUNNING) continue;
     swq_half(a, jj, tot[0], 2 * (a.iters[jj] - 1 - a.start[jj]) + 1);
@@ -851,39 +1013,34 @@ __global__ void __launch_bounds__(512) k_swq_odd(SweepArgs a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int any = 0;
-    for (int g2 = 0; g2 < a.G; ++g2) {
-      int on = 0;
-      for (int l = 0; l < 32; ++l) on |= a.status[g2 * 32 + l] == ST_RUNNING && a.chk[g2 * 32 + l] != 0;
-      a.gcheck[g2] = on;
-      any |= on;
-    }
-    *a.anychk = any;
-    sweep_refresh_groups(a);
+  if (threadIdx.x < 32) {
+    bool chk = false;
+    for (int f = threadIdx.x; f < a.F; f += 32) chk |= a.status[f] == ST_RUNNING && a.chk[f] != 0;
+    const int any = __any_sync(0xffffffffu, chk);
+    if (threadIdx.x == 0) *a.anychk = any;
+    sweep_refresh(a);
   }
 }
 
 // T4: u = w + beta un; x += eta d
-__global__ void __launch_bounds__(512) k_swq_u(SweepArgs a) {
+__global__ void __launch_bounds__(512, 2) k_swq_u(SweepArgs a) {
   if (a.st->status != ST_RUNNING) return;
   SWEEP_ELEMENTWISE_BEGIN
   if (!run) return;
   const double2 be = a.beta[j], eta = a.omg[j];
-  for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-    const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
+  for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+    const size_t idx = static_cast<size_t>(q) * a.Fp + j;
     a.p[idx] = cfma(be, a.s[idx], a.r[idx]);
     a.x[idx] = cfma(eta, a.q2[idx], a.x[idx]);
   }
 }
 
 // T5: Au = A_j u; v = Au + beta (A un + beta v); sigma = (r0, v) -> alpha, gamma
-__global__ void __launch_bounds__(512) k_swq_spmv_u(SweepArgs a) {
+__global__ void __launch_bounds__(512, 2) k_swq_spmv_u(SweepArgs a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
-  const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int jl = static_cast<int>(gw % a.G) * 32 + (threadIdx.x & 31);
-  const double2 be = a.beta[jl];
+  const SweepWalk wk = walk_running(a);
+  const double2 be = a.beta[max(wk.j, 0)];
   double part[2] = {0.0, 0.0};
   auto body = [&](int32_t i, int j, double2 ax) {
     const size_t idx = static_cast<size_t>(i) * a.Fp + j;
@@ -894,9 +1051,9 @@ __global__ void __launch_bounds__(512) k_swq_spmv_u(SweepArgs a) {
     part[0] = d.x;
     part[1] = d.y;
   };
-  sweep_spmv(a, a.p, body);
+  sweep_spmv(a, wk, a.p, SweepNoPre(), body);
   double tot[2];
-  if (!sweep_grid_sum<2>(a, part, sh, a.tickets + TK_AUX1, tot)) return;
+  if (!sweep_grid_sum<2>(a, wk, part, sh, a.tickets + TK_AUX1, tot)) return;
   for (int j = threadIdx.x; j < a.F && j == (int)threadIdx.x; j += blockDim.x) {
     if (a.status[j] != ST_RUNNING) continue;
     const double2 sigma = make_double2(tot[0], tot[1]);
@@ -912,13 +1069,13 @@ __global__ void __launch_bounds__(512) k_swq_spmv_u(SweepArgs a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // T6: the true residual of the frequencies whose bound fell below tol (only
-// their groups make the product); iteration cap and deadline for every
+// their lanes make the product); iteration cap and deadline for every
 // running frequency; the loop condition.
-__global__ void __launch_bounds__(512) k_swq_check(SweepArgs a) {
+__global__ void __launch_bounds__(512, 2) k_swq_check(SweepArgs a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) {
     if (blockIdx.x == 0 && threadIdx.x == 0) sweep_set_cond(a, false);
@@ -926,27 +1083,26 @@ __global__ void __launch_bounds__(512) k_swq_check(SweepArgs a) {
   }
   const bool late = a.st->deadline_ns != 0ull && (globaltimer_ns() - a.st->t0) > a.st->deadline_ns;
   if (*a.anychk == 0) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      for (int j = 0; j < a.F; ++j) {
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+      for (int j = threadIdx.x; j < a.F; j += 32) {
         if (a.status[j] != ST_RUNNING) continue;
         if (a.iters[j] >= a.st->maxit) a.status[j] = HELM_ERR_NOT_CONVERGED;
         else if (late) a.status[j] = HELM_ERR_TIMEOUT;
       }
-      sweep_refresh_groups(a);
+      __syncwarp();
+      sweep_refresh(a);
     }
     return;
   }
-  SweepArgs ac = a;
-  ac.gactive = a.gcheck;  // only the groups with a frequency to check
+  const SweepWalk wk = walk_running(a);
   double part[1] = {0.0};
   auto body = [&](int32_t i, int j, double2 ax) {
-    if (a.chk[j] == 0) return;
     const double2 bi = a.b[a.b_ld ? static_cast<size_t>(i) * a.b_ld + j : static_cast<size_t>(i)];
     part[0] = sw_nrm(part[0], csub(bi, ax));
   };
-  sweep_spmv(ac, a.x, body);
+  sweep_spmv(a, wk, a.x, SweepNoPre(), body, wk.j >= 0 && a.chk[wk.j] != 0);
   double tot[1];
-  if (!sweep_grid_sum<1>(a, part, sh, a.tickets + TK_AUX2, tot)) return;
+  if (!sweep_grid_sum<1>(a, wk, part, sh, a.tickets + TK_AUX2, tot)) return;
   for (int j = threadIdx.x; j < a.F && j == (int)threadIdx.x; j += blockDim.x) {
     if (a.status[j] != ST_RUNNING) continue;
     int status = ST_RUNNING;
@@ -968,11 +1124,8 @@ __global__ void __launch_bounds__(512) k_swq_check(SweepArgs a) {
     a.status[j] = status;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int g2 = 0; g2 < a.G; ++g2) a.gcheck[g2] = 0;
-    *a.anychk = 0;
-    sweep_refresh_groups(a);
-  }
+  if (threadIdx.x == 0) *a.anychk = 0;
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // ---------------------------------------------------------------- batched BiCGStab(l)
@@ -1012,7 +1165,7 @@ __device__ __forceinline__ void swl_beta(const SweepArgs& a, int f, bool first) 
 
 // init: r_0 = b - A_j x (or b, x = 0), r~ = r_0, u_0 = 0; ||b||, ||r_0||,
 // rho1 = (r~, r_0); rho0 = 1, alpha = 0, omega = 1; the first scalar step
-__global__ void __launch_bounds__(512) k_swl_init(SweepArgs a) {
+__global__ void __launch_bounds__(512, 2) k_swl_init(SweepArgs a) {
   extern __shared__ double sh[];
   const int use_x0 = a.st->use_x0;
   SWEEP_ELEMENTWISE_BEGIN
@@ -1031,16 +1184,16 @@ __global__ void __launch_bounds__(512) k_swl_init(SweepArgs a) {
     part[3] = d.y;
   };
   if (use_x0) {
-    sweep_spmv(a, a.x, body);
+    sweep_spmv(a, wk, a.x, SweepNoPre(), body);
   } else if (run) {
-    for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-      const int32_t i = static_cast<int32_t>(u / a.G);
+    for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+      const int32_t i = q;
       a.x[static_cast<size_t>(i) * a.Fp + j] = make_double2(0.0, 0.0);
       body(i, j, make_double2(0.0, 0.0));
     }
   }
   double tot[4];
-  if (!sweep_grid_sum<4>(a, part, sh, a.tickets + TK_INIT, tot)) return;
+  if (!sweep_grid_sum<4>(a, wk, part, sh, a.tickets + TK_INIT, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
     if (a.status[jj] != ST_RUNNING) continue;  // frozen by a restart of other frequencies
     const double bn = sqrt(tot[0]);
@@ -1060,25 +1213,26 @@ __global__ void __launch_bounds__(512) k_swl_init(SweepArgs a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // B1: u_i = r_i - beta u_i, i <= js
-__global__ void __launch_bounds__(512) k_swl_u(SweepArgs a, int js) {
+__global__ void __launch_bounds__(512, 2) k_swl_u(SweepArgs a, int js) {
   if (a.st->status != ST_RUNNING) return;
   SWEEP_ELEMENTWISE_BEGIN
   if (!run) return;
   const double2 be = a.beta[j];
-  for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-    const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
+  for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+    const size_t idx = static_cast<size_t>(q) * a.Fp + j;
     for (int i = 0; i <= js; ++i) a.ul[i][idx] = cfms(be, a.ul[i][idx], a.rl[i][idx]);
   }
 }
 
 // B2: u_{js+1} = A_j u_js, gamma = (r~, u_{js+1}) -> alpha = rho0 / gamma
-__global__ void __launch_bounds__(512) k_swl_au(SweepArgs a, int js) {
+__global__ void __launch_bounds__(512, 2) k_swl_au(SweepArgs a, int js) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
+  const SweepWalk wk = walk_running(a);
   double part[2] = {0.0, 0.0};
   double2* out = a.ul[js + 1];
   auto body = [&](int32_t i, int j, double2 ax) {
@@ -1088,9 +1242,9 @@ __global__ void __launch_bounds__(512) k_swl_au(SweepArgs a, int js) {
     part[0] = d.x;
     part[1] = d.y;
   };
-  sweep_spmv(a, a.ul[js], body);
+  sweep_spmv(a, wk, a.ul[js], SweepNoPre(), body);
   double tot[2];
-  if (!sweep_grid_sum<2>(a, part, sh, a.tickets + TK_V, tot)) return;
+  if (!sweep_grid_sum<2>(a, wk, part, sh, a.tickets + TK_V, tot)) return;
   for (int j = threadIdx.x; j < a.F && j == (int)threadIdx.x; j += blockDim.x) {
     if (a.status[j] != ST_RUNNING) continue;
     const double2 gm = make_double2(tot[0], tot[1]);
@@ -1103,19 +1257,19 @@ __global__ void __launch_bounds__(512) k_swl_au(SweepArgs a, int js) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // B3: r_i -= alpha u_{i+1} (i <= js), x += alpha u_0; ||r_0||^2 -> stop test
-__global__ void __launch_bounds__(512) k_swl_r(SweepArgs a, int js) {
+__global__ void __launch_bounds__(512, 2) k_swl_r(SweepArgs a, int js) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
   SWEEP_ELEMENTWISE_BEGIN
   double part[1] = {0.0};
   if (run) {
     const double2 al = a.alpha[j];
-    for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-      const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
+    for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+      const size_t idx = static_cast<size_t>(q) * a.Fp + j;
       for (int i = 0; i <= js; ++i) {
         const double2 ri = cfms(al, a.ul[i + 1][idx], a.rl[i][idx]);
         a.rl[i][idx] = ri;
@@ -1125,17 +1279,18 @@ __global__ void __launch_bounds__(512) k_swl_r(SweepArgs a, int js) {
     }
   }
   double tot[1];
-  if (!sweep_grid_sum<1>(a, part, sh, a.tickets + TK_S, tot)) return;
+  if (!sweep_grid_sum<1>(a, wk, part, sh, a.tickets + TK_S, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x)
     if (a.status[jj] == ST_RUNNING) swl_stop(a, jj, tot[0]);
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // B4: r_{js+1} = A_j r_js, rho1 = (r~, r_{js+1}); the scalar step of BiCG step js + 1
-__global__ void __launch_bounds__(512) k_swl_ar(SweepArgs a, int js) {
+__global__ void __launch_bounds__(512, 2) k_swl_ar(SweepArgs a, int js) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
+  const SweepWalk wk = walk_running(a);
   double part[2] = {0.0, 0.0};
   double2* out = a.rl[js + 1];
   auto body = [&](int32_t i, int j, double2 ax) {
@@ -1145,16 +1300,16 @@ __global__ void __launch_bounds__(512) k_swl_ar(SweepArgs a, int js) {
     part[0] = d.x;
     part[1] = d.y;
   };
-  sweep_spmv(a, a.rl[js], body);
+  sweep_spmv(a, wk, a.rl[js], SweepNoPre(), body);
   double tot[2];
-  if (!sweep_grid_sum<2>(a, part, sh, a.tickets + TK_T, tot)) return;
+  if (!sweep_grid_sum<2>(a, wk, part, sh, a.tickets + TK_T, tot)) return;
   for (int j = threadIdx.x; j < a.F && j == (int)threadIdx.x; j += blockDim.x) {
     if (a.status[j] != ST_RUNNING) continue;
     a.rho1[j] = make_double2(tot[0], tot[1]);
     if (js + 1 < a.ell) swl_beta(a, j, false);
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // M1: per-frequency Gram matrix G_ik = (r_i, r_k), 0 <= i <= k <= L, one fused
@@ -1172,8 +1327,8 @@ __global__ void __launch_bounds__(512) k_swl_gram(SweepArgs a) {
 #pragma unroll
   for (int e = 0; e < 2 * NG; ++e) acc[e] = 0.0;
   if (run) {
-    for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-      const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
+    for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+      const size_t idx = static_cast<size_t>(q) * a.Fp + j;
       double2 rv[L + 1];
 #pragma unroll
       for (int i = 0; i <= L; ++i) rv[i] = a.rl[i][idx];
@@ -1188,20 +1343,18 @@ __global__ void __launch_bounds__(512) k_swl_gram(SweepArgs a) {
         }
     }
   }
-  // block partials, entry by entry: the warps of a frequency's group in warp order
-  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  // block partials, entry by entry, in slot order
+  const int jt = threadIdx.x;
+  const int place = jt < a.Fp ? wk.place(jt, a.F) : -1;
   for (int e = 0; e < NG; ++e) {
-    sh[(warp * 32 + lane) * 2] = acc[2 * e];
-    sh[(warp * 32 + lane) * 2 + 1] = acc[2 * e + 1];
+    sh[jt * 2] = acc[2 * e];
+    sh[jt * 2 + 1] = acc[2 * e + 1];
     __syncthreads();
-    const int jt = threadIdx.x;
     if (jt < a.Fp) {
       double s0 = 0.0, s1 = 0.0;
-      for (int w = 0; w < nw; ++w) {
-        const int gg = static_cast<int>((static_cast<int64_t>(blockIdx.x) * nw + w) % a.G);
-        if (gg != jt / 32) continue;
-        s0 += sh[(w * 32 + (jt & 31)) * 2];
-        s1 += sh[(w * 32 + (jt & 31)) * 2 + 1];
+      for (int q = 0; place >= 0 && q < wk.slots; ++q) {
+        s0 += sh[(q * wk.na + place) * 2];
+        s1 += sh[(q * wk.na + place) * 2 + 1];
       }
       const size_t o = (static_cast<size_t>(blockIdx.x) * a.Fp + jt) * (2 * NG) + 2 * e;
       a.gpart[o] = s0;
@@ -1299,7 +1452,7 @@ __global__ void __launch_bounds__(512) k_swl_gram(SweepArgs a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // M2: x += sum g_k r_{k-1}; r_0 -= sum g_k r_k; u_0 -= sum g_k u_k;
@@ -1318,8 +1471,8 @@ __global__ void __launch_bounds__(512) k_swl_mr(SweepArgs a) {
     double2 gk[L];
 #pragma unroll
     for (int k = 0; k < L; ++k) gk[k] = a.gcoef[static_cast<size_t>(j) * kSwMaxEll + k];
-    for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-      const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
+    for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+      const size_t idx = static_cast<size_t>(q) * a.Fp + j;
       double2 xq = a.x[idx], r0 = a.rl[0][idx], u0 = a.ul[0][idx];
       double2 rprev = r0;
 #pragma unroll
@@ -1340,7 +1493,7 @@ __global__ void __launch_bounds__(512) k_swl_mr(SweepArgs a) {
     }
   }
   double tot[3];
-  if (!sweep_grid_sum<3>(a, part, sh, a.tickets + TK_XR, tot)) return;
+  if (!sweep_grid_sum<3>(a, wk, part, sh, a.tickets + TK_XR, tot)) return;
   const bool late = a.st->deadline_ns != 0ull && (globaltimer_ns() - a.st->t0) > a.st->deadline_ns;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
     if (a.status[jj] != ST_RUNNING) continue;
@@ -1352,7 +1505,7 @@ __global__ void __launch_bounds__(512) k_swl_mr(SweepArgs a) {
     else swl_beta(a, jj, true);
   }
   __syncthreads();
-  if (threadIdx.x == 0) sweep_refresh_groups(a);
+  if (threadIdx.x < 32) sweep_refresh(a);
 }
 
 // X_user[i * ldx + j] <-> x[i * Fp + j]
@@ -1406,13 +1559,6 @@ __global__ void k_sw_to_f32(int64_t nnz, const double* __restrict__ K, const dou
   }
 }
 
-// SpMV-only kernel for the tile-shape autotuner (x = y = internal buffers).
-template <class V>
-__global__ void __launch_bounds__(512) k_sw_spmv_probe(SweepArgsT<V> a) {
-  auto body = [&](int32_t i, int j, V ax) { a.v[static_cast<size_t>(i) * a.Fp + j] = ax; };
-  sweep_spmv(a, a.p, body);
-}
-
 // ---------------------------------------------------------------- mixed precision
 // The mixed-precision sweep: FP64 refinement per frequency around complex64
 // inner sweeps (the kernels above instantiated for complex64 vectors).  One
@@ -1433,24 +1579,20 @@ struct MxsArgs {
   double* out;          // [Fp][4] per-frequency sums of the last reduction
 };
 
-#define MXS_UNITS_BEGIN                                                                  \
-  const SweepArgs& a = m.a;                                                              \
-  const int lane = threadIdx.x & 31;                                                     \
-  const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; \
-  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;            \
-  const int g = static_cast<int>(gw % a.G);                                              \
-  const int j = g * 32 + lane;                                                           \
-  const bool on = j < a.F && m.act[j] == 1;
+#define MXS_UNITS_BEGIN                \
+  const SweepArgs& a = m.a;            \
+  const SweepWalk wk = walk_all(a);    \
+  const int j = wk.j;                  \
+  const bool on = j >= 0 && m.act[j] == 1;
 
 // r = b - A x (or b when zero_x), out[j][0] = ||r_j||^2
 __global__ void __launch_bounds__(512) k_mxs_residual(MxsArgs m, int zero_x) {
   extern __shared__ double sh[];
   MXS_UNITS_BEGIN
   double part[1] = {0.0};
-  const double wj = a.w[j], w2 = wj * wj;
-  for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-    const int32_t i = static_cast<int32_t>(u / a.G);
-    if (!on) continue;
+  const double wj = a.w[max(j, 0)], w2 = wj * wj;
+  for (int32_t q = wk.i; on && q < a.A.n; q += wk.step) {
+    const int32_t i = q;
     const size_t idx = static_cast<size_t>(i) * a.Fp + j;
     const double2 bi = a.b[a.b_ld ? static_cast<size_t>(i) * a.b_ld + j : static_cast<size_t>(i)];
     const double2 ri = zero_x ? bi : csub(bi, sweep_row(a.A, i, j, wj, w2, a.x, a.Fp));
@@ -1458,17 +1600,17 @@ __global__ void __launch_bounds__(512) k_mxs_residual(MxsArgs m, int zero_x) {
     part[0] = cabs2_acc(ri, part[0]);
   }
   double tot[1];
-  if (!sweep_grid_sum<1>(a, part, sh, a.tickets + TK_AUX0, tot)) return;
+  if (!sweep_grid_sum<1>(a, wk, part, sh, a.tickets + TK_AUX0, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) m.out[4 * jj] = tot[0];
 }
 
 // f_j = complex64(r_j / sigma_j) for running frequencies, 0 for the others
 __global__ void __launch_bounds__(512) k_mxs_down(MxsArgs m) {
   MXS_UNITS_BEGIN
-  if (j >= a.Fp) return;
+  if (j < 0) return;
   const double inv = on ? 1.0 / m.sigma[j] : 0.0;
-  for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-    const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
+  for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+    const size_t idx = static_cast<size_t>(q) * a.Fp + j;
     float2 f = make_float2(0.f, 0.f);
     if (on) {
       const double2 ri = a.r[idx];
@@ -1483,8 +1625,8 @@ __global__ void __launch_bounds__(512) k_mxs_lift(MxsArgs m) {
   MXS_UNITS_BEGIN
   if (!on) return;
   const double sc = m.sigma[j];
-  for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-    const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
+  for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+    const size_t idx = static_cast<size_t>(q) * a.Fp + j;
     const float2 d = m.x32[idx];
     a.p[idx] = make_double2(sc * static_cast<double>(d.x), sc * static_cast<double>(d.y));
   }
@@ -1495,10 +1637,9 @@ __global__ void __launch_bounds__(512) k_mxs_apply(MxsArgs m) {
   extern __shared__ double sh[];
   MXS_UNITS_BEGIN
   double part[3] = {0.0, 0.0, 0.0};
-  const double wj = a.w[j], w2 = wj * wj;
-  for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-    const int32_t i = static_cast<int32_t>(u / a.G);
-    if (!on) continue;
+  const double wj = a.w[max(j, 0)], w2 = wj * wj;
+  for (int32_t q = wk.i; on && q < a.A.n; q += wk.step) {
+    const int32_t i = q;
     const size_t idx = static_cast<size_t>(i) * a.Fp + j;
     const double2 wi = sweep_row(a.A, i, j, wj, w2, a.p, a.Fp);
     a.v[idx] = wi;
@@ -1508,7 +1649,7 @@ __global__ void __launch_bounds__(512) k_mxs_apply(MxsArgs m) {
     part[2] = cabs2_acc(wi, part[2]);
   }
   double tot[3];
-  if (!sweep_grid_sum<3>(a, part, sh, a.tickets + TK_AUX1, tot)) return;
+  if (!sweep_grid_sum<3>(a, wk, part, sh, a.tickets + TK_AUX1, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
     m.out[4 * jj] = tot[0];
     m.out[4 * jj + 1] = tot[1];
@@ -1519,16 +1660,14 @@ __global__ void __launch_bounds__(512) k_mxs_apply(MxsArgs m) {
 // x_j += gamma_j z_j (running frequencies); x_j = 0 where b_j = 0
 __global__ void __launch_bounds__(512) k_mxs_update(MxsArgs m) {
   const SweepArgs& a = m.a;
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-  const int j = static_cast<int>(gw % a.G) * 32 + lane;
-  if (j >= a.F) return;
+  const SweepWalk wk = walk_all(a);
+  const int j = wk.j;
+  if (j < 0) return;
   const int act = m.act[j];
   const double2 gm = m.gamma[j];
   if (act == 0 || (act == 1 && czero(gm))) return;
-  for (int64_t u = gw; u < static_cast<int64_t>(a.A.n) * a.G; u += nwarps) {
-    const size_t idx = static_cast<size_t>(u / a.G) * a.Fp + j;
+  for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
+    const size_t idx = static_cast<size_t>(q) * a.Fp + j;
     a.x[idx] = act == 2 ? make_double2(0.0, 0.0) : cfma(gm, a.p[idx], a.x[idx]);
   }
 }
@@ -1554,7 +1693,7 @@ struct helm_sweep_s {
   double2* vec = nullptr;         // 7 vectors [n][Fcap]
   double2* scal = nullptr;        // 4 [Fcap]
   double* dscal = nullptr;        // 3 [Fcap] + w [Fcap]
-  int32_t* iscal = nullptr;       // 3 [Fcap] + groups [Fcap / 32] + restart flags [Fcap]
+  int32_t* iscal = nullptr;       // 3 [Fcap] + restart flags [Fcap] + list and places of the running [2 Fcap] + their number
   SolverState* state = nullptr;
   double* partials = nullptr;
   size_t partials_cap = 0;
@@ -1569,8 +1708,8 @@ struct helm_sweep_s {
   double* oscal = nullptr;
   int32_t* oact = nullptr;
   // batched TFQMR: 2 vectors [n][Fcapq] (A un, d), gamma and (theta, tau)
-  // [2 Fcapq], check flags and start iterations [2 Fcapq], group check flags
-  // [Fcapq / 32] and one sweep-wide flag
+  // [2 Fcapq], check flags and start iterations [2 Fcapq] and one
+  // sweep-wide flag
   double2* vecq = nullptr;
   double2* tqscal = nullptr;
   int32_t* tqint = nullptr;
@@ -1588,8 +1727,6 @@ struct helm_sweep_s {
   double* are = nullptr;
   size_t are_cap = 0;
   std::vector<double> are_w;      // the frequencies they were formed for
-  int warps_per_block = 8;        // autotuned
-  bool tuned = false;
   std::mutex mu;
   struct G {
     int32_t F = -1, b_ld = -1;
@@ -1626,7 +1763,7 @@ helm_status sweep_alloc(helm_sweep S, int32_t Fp, size_t blocks) {
     HELM_CUDA_TRY(cudaMalloc(&S->vec, 7 * nf * sizeof(double2)));
     HELM_CUDA_TRY(cudaMalloc(&S->scal, 4 * static_cast<size_t>(Fp) * sizeof(double2)));
     HELM_CUDA_TRY(cudaMalloc(&S->dscal, 4 * static_cast<size_t>(Fp) * sizeof(double)));
-    HELM_CUDA_TRY(cudaMalloc(&S->iscal, (4 * static_cast<size_t>(Fp) + Fp / 32) * sizeof(int32_t)));
+    HELM_CUDA_TRY(cudaMalloc(&S->iscal, (6 * static_cast<size_t>(Fp) + 1) * sizeof(int32_t)));
     S->Fcap = Fp;
     drop_sweep_graphs(S);
   }
@@ -1671,7 +1808,9 @@ SweepArgs make_args(helm_sweep S, int32_t F, int32_t Fp, const double2* b, int32
   a.status = S->iscal;
   a.iters = S->iscal + Fp;
   a.phase = S->iscal + 2 * Fp;
-  a.gactive = S->iscal + 3 * Fp;
+  a.act = S->iscal + 4 * Fp;
+  a.pos = S->iscal + 5 * Fp;
+  a.nact = S->iscal + 6 * Fp;
   a.st = S->state;
   a.partials = S->partials;
   a.tickets = S->tickets;
@@ -1713,7 +1852,9 @@ SweepArgsT<float2> make_args32(helm_sweep S, const SweepArgs& a64) {
   a.status = a64.status;
   a.iters = a64.iters;
   a.phase = a64.phase;
-  a.gactive = a64.gactive;
+  a.act = a64.act;
+  a.pos = a64.pos;
+  a.nact = a64.nact;
   a.st = a64.st;
   a.partials = a64.partials;
   a.tickets = a64.tickets;
@@ -1763,7 +1904,7 @@ helm_status sweep_alloc_tfqmr(helm_sweep S, int32_t Fp) {
   const size_t nf = static_cast<size_t>(std::max<int32_t>(S->n, 1)) * Fp;
   HELM_CUDA_TRY(cudaMalloc(&S->vecq, 2 * nf * sizeof(double2)));
   HELM_CUDA_TRY(cudaMalloc(&S->tqscal, 2 * static_cast<size_t>(Fp) * sizeof(double2)));
-  HELM_CUDA_TRY(cudaMalloc(&S->tqint, (2 * static_cast<size_t>(Fp) + Fp / 32 + 1) * sizeof(int32_t)));
+  HELM_CUDA_TRY(cudaMalloc(&S->tqint, (2 * static_cast<size_t>(Fp) + 1) * sizeof(int32_t)));
   S->Fcapq = Fp;
   if (S->graphq.exec) {
     cudaGraphExecDestroy(S->graphq.exec);
@@ -1781,8 +1922,7 @@ void set_tfqmr_args(helm_sweep S, SweepArgs& a) {
   a.tt = S->tqscal + a.Fp;
   a.chk = S->tqint;
   a.start = S->tqint + a.Fp;
-  a.gcheck = S->tqint + 2 * static_cast<size_t>(a.Fp);
-  a.anychk = S->tqint + 2 * static_cast<size_t>(a.Fp) + a.Fp / 32;
+  a.anychk = S->tqint + 2 * static_cast<size_t>(a.Fp);
 }
 
 // Buffers of the batched BiCGStab(l) (allocated at its first use, grown
@@ -1845,10 +1985,11 @@ struct SweepShape {
 
 SweepShape sweep_shape(helm_sweep S, int G) {
   SweepShape sh;
-  sh.threads = 32 * S->warps_per_block;
-  // each warp keeps one group: the number of warps must be a multiple of G
-  const int warps_per_block = S->warps_per_block;
-  sh.smem = static_cast<size_t>(warps_per_block) * 32 * 4 * sizeof(double);
+  const int64_t units = static_cast<int64_t>(S->n) * G;
+  int warps = kSweepWarps;
+  while (warps > kSweepMinWarps && units < static_cast<int64_t>(warps) * S->num_sms) warps /= 2;
+  sh.threads = 32 * warps;
+  sh.smem = static_cast<size_t>(warps) * 32 * 4 * sizeof(double);
   // up to 1024 resident threads per SM (enough warps to hide latency, few
   // block partials for the per-frequency reductions), and no more blocks
   // than every sweep kernel fits on an SM at once: one wave
@@ -1871,17 +2012,8 @@ SweepShape sweep_shape(helm_sweep S, int G) {
   }
   (void)cudaGetLastError();
   int64_t blocks = static_cast<int64_t>(S->num_sms) * per_sm;
-  int64_t units = static_cast<int64_t>(S->n) * G;
-  int64_t want = (units + warps_per_block - 1) / warps_per_block;
+  const int64_t want = (units + warps - 1) / warps;
   if (want < blocks) blocks = want < 1 ? 1 : want;
-  // warps in the grid = blocks * warps_per_block: make it a multiple of G
-  // (rounding down keeps one wave; up only when that leaves no block)
-  const int64_t b0 = blocks;
-  while (blocks > 1 && (blocks * warps_per_block) % G != 0) --blocks;
-  if ((blocks * warps_per_block) % G != 0) {
-    blocks = b0;
-    while ((blocks * warps_per_block) % G != 0) ++blocks;
-  }
   sh.grid = static_cast<int>(blocks);
   return sh;
 }
@@ -2018,47 +2150,6 @@ helm_status build_bicgstabl_graph(const SweepArgs& base, const SweepShape& sh, c
       [&](const SweepArgs& a, cudaStream_t cs) { swl_body(a, sh, cs); },
       [&](const SweepArgs& a, cudaStream_t cs) { k_sw_tail<double2><<<sh.grid, sh.threads, sh.smem, cs>>>(a); },
       gout, eout);
-}
-
-// Time the batched SpMV with 4, 8 and 16 warps per block; keep the fastest.
-helm_status autotune(helm_sweep S, int32_t F, int32_t Fp, cudaStream_t s) {
-  const int candidates[3] = {4, 8, 16};  // 128..512 threads: at least kMaxF
-  float best = 1e30f;
-  int best_w = 8;
-  cudaEvent_t e0, e1;
-  HELM_CUDA_TRY(cudaEventCreate(&e0));
-  HELM_CUDA_TRY(cudaEventCreate(&e1));
-  helm_status result = HELM_OK;
-  for (int c : candidates) {
-    S->warps_per_block = c;
-    const SweepShape sh = sweep_shape(S, Fp / 32);
-    result = sweep_alloc(S, Fp, sh.grid);
-    if (result != HELM_OK) break;
-    SweepArgs a = make_args(S, F, Fp, nullptr, 0);
-    // every group active, every frequency running, p = 0 (timing only)
-    k_sw_configure<double2><<<1, 256, 0, s>>>(a, 0.0, 1, 0, 0.0, 1, nullptr);
-    cudaMemsetAsync(a.p, 0, static_cast<size_t>(S->n) * Fp * sizeof(double2), s);
-    k_sw_spmv_probe<double2><<<sh.grid, sh.threads, 0, s>>>(a);
-    cudaEventRecord(e0, s);
-    for (int rep = 0; rep < 3; ++rep) k_sw_spmv_probe<double2><<<sh.grid, sh.threads, 0, s>>>(a);
-    cudaEventRecord(e1, s);
-    if (cudaEventSynchronize(e1) != cudaSuccess) {
-      result = HELM_ERR_CUDA;
-      break;
-    }
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    if (ms < best) {
-      best = ms;
-      best_w = c;
-    }
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  (void)cudaGetLastError();
-  S->warps_per_block = best_w;
-  S->tuned = true;
-  return result;
 }
 
 // The mixed-precision sweep (precision HELM_PREC_MIXED): refinement steps as
@@ -2317,10 +2408,6 @@ helm_status helm_sweep_solve(helm_sweep S, int32_t nfreq, const double* h_omega,
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   std::lock_guard<std::mutex> lk(S->mu);
   const int32_t Fp = (nfreq + 31) / 32 * 32;
-  if (!S->tuned) {
-    helm_status st = autotune(S, nfreq, Fp, s);
-    if (st != HELM_OK) return st;
-  }
   const SweepShape sh = sweep_shape(S, Fp / 32);
   helm_status st = sweep_alloc(S, Fp, sh.grid);
   if (st != HELM_OK) return st;
@@ -2414,7 +2501,7 @@ helm_status helm_sweep_solve(helm_sweep S, int32_t nfreq, const double* h_omega,
     }
   }
   // restart flags of the frequencies that run again from their x
-  int32_t* d_restart = S->iscal + 3 * static_cast<size_t>(Fp) + Fp / 32;
+  int32_t* d_restart = S->iscal + 3 * static_cast<size_t>(Fp);
   std::vector<int32_t> status(Fp), iters(Fp), restart(Fp, 0), restarts(nfreq, 0);
   std::vector<double> relres(Fp), relres_true(Fp);
   for (int32_t fresh = 1, use_x0 = opts.use_x0 ? 1 : 0;; fresh = 0, use_x0 = 1) {

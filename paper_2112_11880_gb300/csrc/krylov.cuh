@@ -106,22 +106,24 @@ __device__ __forceinline__ double nrm_acc(double acc, float2 a) {
 // every run.
 //   small: one block per SM; a row is summed in kParts parts, which the
 //          persistent kernel gives to three warps;
-//   mid:   one block per SM of at most 640 threads (96 registers a thread);
+//   mid:   one block per SM of at most 768 threads (80 registers a thread);
 //   large: two blocks per SM of at most 512 threads (64 registers).
 // complex64 (the inner solves of mixed precision): mid or large (us per inner
-// iteration, persistent / before: 20^3 29.9 / 44.5, 60x30x25 29.7 / 37.1,
-// 80x40x32 38.4 / 47, 120x60x50 70.2 / 77.9, 200x100x80 192.7 / 204.8).
+// iteration, persistent / graph / before: 20^3 29.7 / 33.9 / 44.5, 60x30x25 29.4 /
+// 34.5 / 37.1, 80x40x32 37.6 / 44.9 / 47, 120x60x50 68.4 / 73.8 / 77.9, 200x100x80
+// 191 / 184 / 205: on the large shape the default is the graph).
 // Measured (BiCGStab, us per iteration: persistent / graph kernels; before, on
 // one shape with graph kernels):
-//   20^3 box      (2 slices per SM)  small 25.7 / 42.8                       (39.7)
-//   60x30x25      (10)               mid   37.7 / 39.0, large 50.1 / 47.6    (43.6)
-//   80x40x32      (23)               mid   57.1 / 59.4, large 60.0 / 67.0    (65.1)
-//   120x60x50     (77)               mid  122.0 / 136.2, large 135.4 / 140.2 (134.0)
-//   200x100x80    (338)              mid  504 (512 threads), large 470 / 500 (478)
+//   20^3 box      (2 slices per SM)  small 25.7 / 43.7                       (39.7)
+//   60x30x25      (10)               mid   37.2 / 39.1, large 50.1 / 47.6    (43.6)
+//   80x40x32      (23)               mid   54.0 / 61.6, large 60.0 / 67.0    (65.1)
+//   120x60x50     (77)               mid  121.1 / 136.9, large 135.4 / 140.2 (134.0)
+//   200x100x80    (338)              mid  504 (512 threads), large 475 / 498 (478)
+// (mid of 640 threads: 37.3, 55.1, 121.5; 704: 40.5, 61.0, 124.1; more spill.)
 enum : int { SHAPE_SMALL = 0, SHAPE_MID = 1, SHAPE_LARGE = 2 };
 constexpr int kMidSlices = 150;  // slices per SM from which the shape is large
 template <int S> struct SolverBounds {
-  static constexpr int threads = S == SHAPE_SMALL ? 384 : S == SHAPE_MID ? 640 : 512;  // warps of a split persistent kernel included
+  static constexpr int threads = S == SHAPE_SMALL ? 384 : S == SHAPE_MID ? 768 : 512;  // warps of a split persistent kernel included
   static constexpr int blocks = S == SHAPE_LARGE ? 2 : 1;
   static constexpr int parts = S == SHAPE_SMALL ? kParts : 1;
   // entries per pipeline stage of the persistent kernel's products

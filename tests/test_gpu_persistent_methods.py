@@ -14,7 +14,7 @@ if not torch.cuda.is_available():
     pytest.skip("needs a GPU", allow_module_level=True)
 
 import paper_2112_11880_gb300 as helm  # noqa: E402
-from test_gpu_solver_shapes import SMS, _banded  # noqa: E402
+from test_gpu_solver_shapes import SMS, _banded, _check  # noqa: E402
 
 DEV = torch.device("cuda:0")
 METHODS = [(helm.HELM_TFQMR, 2)] + [(helm.HELM_BICGSTABL, ell) for ell in (1, 2, 3, 4, 5, 8)]
@@ -71,3 +71,9 @@ def test_zero_right_hand_side(method, ell):
     assert info["status"] == "ok" and info["relres_true"] == 0.0
     assert not x.any()
     A.close()
+
+
+@pytest.mark.parametrize("extra", [0, 1, 32 * SMS])
+def test_bicgstab_at_a_full_round_of_the_mid_shape(extra):
+    """24 slices per SM are one round of its warps."""
+    _check(*_banded(32 * 24 * SMS + extra, [-70, -1, 0, 1, 70], lambda r: (r % 97 == 0) * 1.0, 3), seed=11)

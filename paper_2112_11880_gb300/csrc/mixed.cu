@@ -609,11 +609,14 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   a.tickets = A->tickets;
   a.dev_err = A->dev_err;
 
-  // HELM_LAUNCH_AUTO: persistent inner solves where the device can launch them
+  // HELM_LAUNCH_AUTO: persistent inner solves where the device can launch them,
+  // but the graph on the large shape (us per inner iteration on the 200x100x80
+  // cavity: 184 against 191; below, the persistent kernel is ahead by 5 to 6)
   PShape ps;
   const void* inner = nullptr;
   with_shape(sh.k, [&](auto S) { inner = reinterpret_cast<const void*>(&k_mx_inner<S.value>); });
-  const bool persistent = o.launch == HELM_LAUNCH_AUTO && persist_fit(inner, n, sh.k.grid, sh.k.threads, sh.k.bps, 1,
+  const bool persistent = o.launch == HELM_LAUNCH_AUTO && sh.k.shape != SHAPE_LARGE &&
+                          persist_fit(inner, n, sh.k.grid, sh.k.threads, sh.k.bps, 1,
                                                                  Phases<float2>::kOwn, sizeof(float2), &ps);
   (void)cudaGetLastError();
 

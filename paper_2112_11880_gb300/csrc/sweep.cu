@@ -141,14 +141,15 @@ template <> __device__ __forceinline__ float2 sw_zero<float2>() { return make_fl
 // depend on which others are running.
 // Memory is what is short then: a warp's gathers that miss L1 return some 75
 // clocks apart, and a row waits for 27 of them.  So a slot's rows are shared out to
-// the threads that are left over (walk_split), which store their products; the
+// the threads that are left over (walk_split), which store their results; the
 // slot's sums are formed afterwards, in the order of its rows (sweep_chain).
 // Measured: 64 frequencies of the 60x30x25 cavity, 50 to 300 Hz, to 1e-10 (162 to
 // 1835 iterations, 674 on average): 1411 ms with a fixed warp for every slot and
 // 32 frequencies, on until the last of them stopped; packed 1340; and rows loaded
 // ahead and shared out 869; the same bits.  An iteration with 64, 32, 16, 8, 1
 // frequencies running: 941, 526, 522, 521, 520 us before, now 940, 516, 340, 232,
-// 196.
+// 196.  (Five frequencies, 200 iterations: BiCGStab 109 -> 42 ms, TFQMR 109 -> 40,
+// BiCGStab(2), 200 cycles, 244 -> 91.)
 struct SweepWalk {
   int j;               // this thread's frequency (-1: none)
   int32_t i, step;     // its rows: i, i + step, ...  (n < 2^27: seven vectors of n x 32 have to fit)
@@ -940,7 +941,7 @@ __global__ void __launch_bounds__(512, 2) k_swq_init_b(SweepArgs a) {
 __global__ void __launch_bounds__(512, 2) k_swq_even(SweepArgs a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
-  SWEEP_ELEMENTWISE_BEGIN
+  SWEEP_SPLIT_BEGIN
   double part[1] = {0.0};
   if (run) {
     const double2 al = a.alpha[j], ga = a.gam[j];
@@ -951,9 +952,10 @@ __global__ void __launch_bounds__(512, 2) k_swq_even(SweepArgs a) {
       const double2 wi = cfms(al, a.t[idx], a.r[idx]);
       a.r[idx] = wi;
       a.q2[idx] = cfma(ga, a.q2[idx], ui);
-      part[0] = sw_nrm(part[0], wi);
+      if (wk.split == 1) part[0] = sw_nrm(part[0], wi);
     }
   }
+  sweep_chain(a, wk, [&](size_t idx) { return a.r[idx]; }, [&](double2 wi) { part[0] = sw_nrm(part[0], wi); });
   double tot[1];
   if (!sweep_grid_sum<1>(a, wk, part, sh, a.tickets + TK_S, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
@@ -969,7 +971,7 @@ __global__ void __launch_bounds__(512, 2) k_swq_even(SweepArgs a) {
 // T2: A un; x += eta d (the even half-step's x update)
 __global__ void __launch_bounds__(512, 2) k_swq_spmv_un(SweepArgs a) {
   if (a.st->status != ST_RUNNING) return;
-  const SweepWalk wk = walk_running(a);
+  const SweepWalk wk = walk_split(a);
   const double2 eta = a.omg[max(wk.j, 0)];
   auto body = [&](int32_t i, int j, double2 ax) {
     const size_t idx = static_cast<size_t>(i) * a.Fp + j;
@@ -983,8 +985,14 @@ __global__ void __launch_bounds__(512, 2) k_swq_spmv_un(SweepArgs a) {
 __global__ void __launch_bounds__(512, 2) k_swq_odd(SweepArgs a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
-  SWEEP_ELEMENTWISE_BEGIN
+  SWEEP_SPLIT_BEGIN
   double part[3] = {0.0, 0.0, 0.0};
+  auto add = [&](const Vec2<double2>& l) {
+    part[0] = sw_nrm(part[0], l.b);
+    const double2 d = sw_dot(make_double2(part[1], part[2]), l.a, l.b);
+    part[1] = d.x;
+    part[2] = d.y;
+  };
   if (run) {
     const double2 al = a.alpha[j], ga = a.gam[j];
     for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
@@ -992,12 +1000,10 @@ __global__ void __launch_bounds__(512, 2) k_swq_odd(SweepArgs a) {
       const double2 wi = cfms(al, a.q1[idx], a.r[idx]);
       a.r[idx] = wi;
       a.q2[idx] = cfma(ga, a.q2[idx], a.s[idx]);
-      part[0] = sw_nrm(part[0], wi);
-      const double2 d = sw_dot(make_double2(part[1], part[2]), a.rh[idx], wi);
-      part[1] = d.x;
-      part[2] = d.y;
+      if (wk.split == 1) add(Vec2<double2>{a.rh[idx], wi});
     }
   }
+  sweep_chain(a, wk, [&](size_t idx) { return Vec2<double2>{a.rh[idx], a.r[idx]}; }, add);
   double tot[3];
   if (!sweep_grid_sum<3>(a, wk, part, sh, a.tickets + TK_T, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x) {
@@ -1025,7 +1031,7 @@ __global__ void __launch_bounds__(512, 2) k_swq_odd(SweepArgs a) {
 // T4: u = w + beta un; x += eta d
 __global__ void __launch_bounds__(512, 2) k_swq_u(SweepArgs a) {
   if (a.st->status != ST_RUNNING) return;
-  SWEEP_ELEMENTWISE_BEGIN
+  SWEEP_SPLIT_BEGIN
   if (!run) return;
   const double2 be = a.beta[j], eta = a.omg[j];
   for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
@@ -1039,19 +1045,23 @@ __global__ void __launch_bounds__(512, 2) k_swq_u(SweepArgs a) {
 __global__ void __launch_bounds__(512, 2) k_swq_spmv_u(SweepArgs a) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
-  const SweepWalk wk = walk_running(a);
+  const SweepWalk wk = walk_split(a);
   const double2 be = a.beta[max(wk.j, 0)];
   double part[2] = {0.0, 0.0};
+  auto add = [&](const Vec2<double2>& l) {
+    const double2 d = sw_dot(make_double2(part[0], part[1]), l.a, l.b);
+    part[0] = d.x;
+    part[1] = d.y;
+  };
   auto body = [&](int32_t i, int j, double2 ax) {
     const size_t idx = static_cast<size_t>(i) * a.Fp + j;
     a.t[idx] = ax;
     const double2 vn = cfma(be, cfma(be, a.v[idx], a.q1[idx]), ax);
     a.v[idx] = vn;
-    const double2 d = sw_dot(make_double2(part[0], part[1]), a.rh[idx], vn);
-    part[0] = d.x;
-    part[1] = d.y;
+    if (wk.split == 1) add(Vec2<double2>{a.rh[idx], vn});
   };
   sweep_spmv(a, wk, a.p, SweepNoPre(), body);
+  sweep_chain(a, wk, [&](size_t idx) { return Vec2<double2>{a.rh[idx], a.v[idx]}; }, add);
   double tot[2];
   if (!sweep_grid_sum<2>(a, wk, part, sh, a.tickets + TK_AUX1, tot)) return;
   for (int j = threadIdx.x; j < a.F && j == (int)threadIdx.x; j += blockDim.x) {
@@ -1219,7 +1229,7 @@ __global__ void __launch_bounds__(512, 2) k_swl_init(SweepArgs a) {
 // B1: u_i = r_i - beta u_i, i <= js
 __global__ void __launch_bounds__(512, 2) k_swl_u(SweepArgs a, int js) {
   if (a.st->status != ST_RUNNING) return;
-  SWEEP_ELEMENTWISE_BEGIN
+  SWEEP_SPLIT_BEGIN
   if (!run) return;
   const double2 be = a.beta[j];
   for (int32_t q = wk.i; q < a.A.n; q += wk.step) {
@@ -1232,17 +1242,21 @@ __global__ void __launch_bounds__(512, 2) k_swl_u(SweepArgs a, int js) {
 __global__ void __launch_bounds__(512, 2) k_swl_au(SweepArgs a, int js) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
-  const SweepWalk wk = walk_running(a);
+  const SweepWalk wk = walk_split(a);
   double part[2] = {0.0, 0.0};
   double2* out = a.ul[js + 1];
-  auto body = [&](int32_t i, int j, double2 ax) {
-    const size_t idx = static_cast<size_t>(i) * a.Fp + j;
-    out[idx] = ax;
-    const double2 d = sw_dot(make_double2(part[0], part[1]), a.rh[idx], ax);
+  auto add = [&](const Vec2<double2>& l) {
+    const double2 d = sw_dot(make_double2(part[0], part[1]), l.a, l.b);
     part[0] = d.x;
     part[1] = d.y;
   };
+  auto body = [&](int32_t i, int j, double2 ax) {
+    const size_t idx = static_cast<size_t>(i) * a.Fp + j;
+    out[idx] = ax;
+    if (wk.split == 1) add(Vec2<double2>{a.rh[idx], ax});
+  };
   sweep_spmv(a, wk, a.ul[js], SweepNoPre(), body);
+  sweep_chain(a, wk, [&](size_t idx) { return Vec2<double2>{a.rh[idx], out[idx]}; }, add);
   double tot[2];
   if (!sweep_grid_sum<2>(a, wk, part, sh, a.tickets + TK_V, tot)) return;
   for (int j = threadIdx.x; j < a.F && j == (int)threadIdx.x; j += blockDim.x) {
@@ -1264,7 +1278,7 @@ __global__ void __launch_bounds__(512, 2) k_swl_au(SweepArgs a, int js) {
 __global__ void __launch_bounds__(512, 2) k_swl_r(SweepArgs a, int js) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
-  SWEEP_ELEMENTWISE_BEGIN
+  SWEEP_SPLIT_BEGIN
   double part[1] = {0.0};
   if (run) {
     const double2 al = a.alpha[j];
@@ -1273,11 +1287,12 @@ __global__ void __launch_bounds__(512, 2) k_swl_r(SweepArgs a, int js) {
       for (int i = 0; i <= js; ++i) {
         const double2 ri = cfms(al, a.ul[i + 1][idx], a.rl[i][idx]);
         a.rl[i][idx] = ri;
-        if (i == 0) part[0] = sw_nrm(part[0], ri);
+        if (i == 0 && wk.split == 1) part[0] = sw_nrm(part[0], ri);
       }
       a.x[idx] = cfma(al, a.ul[0][idx], a.x[idx]);
     }
   }
+  sweep_chain(a, wk, [&](size_t idx) { return a.rl[0][idx]; }, [&](double2 r0) { part[0] = sw_nrm(part[0], r0); });
   double tot[1];
   if (!sweep_grid_sum<1>(a, wk, part, sh, a.tickets + TK_S, tot)) return;
   for (int jj = threadIdx.x; jj < a.F && jj == (int)threadIdx.x; jj += blockDim.x)
@@ -1290,17 +1305,21 @@ __global__ void __launch_bounds__(512, 2) k_swl_r(SweepArgs a, int js) {
 __global__ void __launch_bounds__(512, 2) k_swl_ar(SweepArgs a, int js) {
   extern __shared__ double sh[];
   if (a.st->status != ST_RUNNING) return;
-  const SweepWalk wk = walk_running(a);
+  const SweepWalk wk = walk_split(a);
   double part[2] = {0.0, 0.0};
   double2* out = a.rl[js + 1];
-  auto body = [&](int32_t i, int j, double2 ax) {
-    const size_t idx = static_cast<size_t>(i) * a.Fp + j;
-    out[idx] = ax;
-    const double2 d = sw_dot(make_double2(part[0], part[1]), a.rh[idx], ax);
+  auto add = [&](const Vec2<double2>& l) {
+    const double2 d = sw_dot(make_double2(part[0], part[1]), l.a, l.b);
     part[0] = d.x;
     part[1] = d.y;
   };
+  auto body = [&](int32_t i, int j, double2 ax) {
+    const size_t idx = static_cast<size_t>(i) * a.Fp + j;
+    out[idx] = ax;
+    if (wk.split == 1) add(Vec2<double2>{a.rh[idx], ax});
+  };
   sweep_spmv(a, wk, a.rl[js], SweepNoPre(), body);
+  sweep_chain(a, wk, [&](size_t idx) { return Vec2<double2>{a.rh[idx], out[idx]}; }, add);
   double tot[2];
   if (!sweep_grid_sum<2>(a, wk, part, sh, a.tickets + TK_T, tot)) return;
   for (int j = threadIdx.x; j < a.F && j == (int)threadIdx.x; j += blockDim.x) {
@@ -1465,8 +1484,14 @@ __global__ void __launch_bounds__(512) k_swl_mr(SweepArgs a) {
     if (blockIdx.x == 0 && threadIdx.x == 0) sweep_set_cond(a, false);
     return;
   }
-  SWEEP_ELEMENTWISE_BEGIN
+  SWEEP_SPLIT_BEGIN
   double part[3] = {0.0, 0.0, 0.0};
+  auto add = [&](const Vec2<double2>& l) {
+    part[0] = sw_nrm(part[0], l.b);
+    const double2 d = sw_dot(make_double2(part[1], part[2]), l.a, l.b);
+    part[1] = d.x;
+    part[2] = d.y;
+  };
   if (run) {
     double2 gk[L];
 #pragma unroll
@@ -1486,12 +1511,10 @@ __global__ void __launch_bounds__(512) k_swl_mr(SweepArgs a) {
       a.x[idx] = xq;
       a.rl[0][idx] = r0;
       a.ul[0][idx] = u0;
-      part[0] = sw_nrm(part[0], r0);
-      const double2 d = sw_dot(make_double2(part[1], part[2]), a.rh[idx], r0);
-      part[1] = d.x;
-      part[2] = d.y;
+      if (wk.split == 1) add(Vec2<double2>{a.rh[idx], r0});
     }
   }
+  sweep_chain(a, wk, [&](size_t idx) { return Vec2<double2>{a.rh[idx], a.rl[0][idx]}; }, add);
   double tot[3];
   if (!sweep_grid_sum<3>(a, wk, part, sh, a.tickets + TK_XR, tot)) return;
   const bool late = a.st->deadline_ns != 0ull && (globaltimer_ns() - a.st->t0) > a.st->deadline_ns;

@@ -26,7 +26,7 @@
 // pipe (l = 4: 8 products of 39 us and some 230 FP64 instructions a row for the
 // vectors on the 120x60x50 cavity, 0.49 ms a cycle).
 // Measured, us per cycle, l = 4, persistent / graph / before (22 graph kernels,
-// four of one thread): 20^3 box 123 / 172 / 282, 60x30x25 165 / 174 / 319,
+// four of one thread): 20^3 box 123 / 158 / 282, 60x30x25 165 / 174 / 319,
 // 80x40x32 246 / 263 / 375, 120x60x50 550 / 578 / 735, 200x100x80 2164 / 2167 /
 // 2310.
 #include <cmath>

@@ -114,7 +114,7 @@ __device__ __forceinline__ double nrm_acc(double acc, float2 a) {
 // 191 / 184 / 205: on the large shape the default is the graph).
 // Measured (BiCGStab, us per iteration: persistent / graph kernels; before, on
 // one shape with graph kernels):
-//   20^3 box      (2 slices per SM)  small 25.7 / 43.7                       (39.7)
+//   20^3 box      (2 slices per SM)  small 25.7 / 39.0                       (39.7)
 //   60x30x25      (10)               mid   37.2 / 39.1, large 50.1 / 47.6    (43.6)
 //   80x40x32      (23)               mid   54.0 / 61.6, large 60.0 / 67.0    (65.1)
 //   120x60x50     (77)               mid  121.1 / 136.9, large 135.4 / 140.2 (134.0)

@@ -202,7 +202,7 @@ __device__ __forceinline__ void for_rows(const PRows& q, int32_t n, F f) {
 
 // Calls f(row, li, sum_k a_rk x_k) for every row of this thread; pre(row) first
 // (its loads are in flight with the sum's).  A split solver's rows are summed
-// in three parts (sell_row_part): here one after the other by the row's thread.
+// in three parts (sell_row_part): here by the row's thread (sell_row_parts).
 template <class V, int U, int PARTS, class G, class Pre, class F>
 __device__ __forceinline__ void spmv_rows(const PRows& q, const CsrDev<V>& A, const V* x, Pre pre, F f) {
 #pragma unroll 1
@@ -219,9 +219,8 @@ __device__ __forceinline__ void spmv_rows(const PRows& q, const CsrDev<V>& A, co
     } else if constexpr (PARTS == 1) {
       acc = sell_row<V, G, U>(A, sp, q.lane(), r, len, x);
     } else {
-      acc = sell_row_part<V, G, U>(A, sp, q.lane(), r, len, 0, x);
-#pragma unroll 1
-      for (int p = 1; p < PARTS; ++p) acc = cadd(acc, sell_row_part<V, G, U>(A, sp, q.lane(), r, len, p, x));
+      static_assert(PARTS == kParts, "as the split kernels sum them");
+      acc = sell_row_parts<V, G>(A, sp, q.lane(), r, len, x);
     }
     if (r < A.n) f(r, q.place(k), acc);
   }

@@ -227,6 +227,77 @@ __device__ __forceinline__ V sell_row_part(const CsrDev<V>& A, const SlicePos& s
   return acc;
 }
 
+// A row's kParts parts by one thread, added in order: the same sums, the parts'
+// pipelines side by side, two entries of each a stage (one part after the other: a
+// BiCGStab iteration of the 20^3 box as a graph 43.7 us, so 39.0).
+template <class V, class G>
+__device__ __forceinline__ V sell_row_parts(const CsrDev<V>& A, const SlicePos& sp, int lane, int32_t r, int32_t len,
+                                            const V* x) {
+  using R = typename RealOf<V>::T;
+  constexpr int U = 2;
+  const int32_t ch = part_width(sp.w), ci = part_width(sp.iw);
+  V acc[kParts];
+  R a[kParts][U];
+  int32_t c[kParts][U];
+  auto entry = [&](int p, int u, int32_t k) {
+    const int32_t e = p * ch + k;
+    a[p][u] = R(0);
+    c[p][u] = 0;
+    if (k < ch && e < len) {
+      a[p][u] = __ldcs(A.sval + sp.base + e * 32 + lane);
+      c[p][u] = __ldcs(A.scol + sp.base + e * 32 + lane);
+    }
+  };
+#pragma unroll
+  for (int p = 0; p < kParts; ++p) {
+    acc[p] = vzero<V>();
+#pragma unroll
+    for (int u = 0; u < U; ++u) entry(p, u, u);
+  }
+#pragma unroll 1
+  for (int32_t k = 0; k < ch; k += U) {
+    V xv[kParts][U];
+    R av[kParts][U];
+#pragma unroll
+    for (int p = 0; p < kParts; ++p)
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (k + u < ch && p * ch + k + u < len) xv[p][u] = G::ld(x + c[p][u]);
+        av[p][u] = a[p][u];
+      }
+#pragma unroll
+    for (int p = 0; p < kParts; ++p)
+#pragma unroll
+      for (int u = 0; u < U; ++u) entry(p, u, k + U + u);
+#pragma unroll
+    for (int p = 0; p < kParts; ++p)
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k + u < ch && p * ch + k + u < len) acc[p] = mac_real(av[p][u], xv[p][u], acc[p]);
+  }
+  if (sp.iw > 0) {
+    const int32_t il = r < A.n ? A.ilen[r] : 0;
+#pragma unroll 1
+    for (int32_t k = 0; k < ci; ++k) {
+      R b[kParts];
+      V xv[kParts];
+#pragma unroll
+      for (int p = 0; p < kParts; ++p)
+        if (p * ci + k < il) {
+          b[p] = A.ival[sp.ib + (p * ci + k) * 32 + lane];
+          xv[p] = G::ld(x + A.icol[sp.ib + (p * ci + k) * 32 + lane]);
+        }
+#pragma unroll
+      for (int p = 0; p < kParts; ++p)
+        if (p * ci + k < il) acc[p] = mac_imag(b[p], xv[p], acc[p]);
+    }
+  }
+  V sum = acc[0];
+#pragma unroll
+  for (int p = 1; p < kParts; ++p) sum = vadd(sum, acc[p]);
+  return sum;
+}
+
 // Rows of this thread.  The slices are taken in rounds of W = G WB
 // consecutive slices (G blocks of WB warps); in round k, whose R slices
 // start at k W, block b takes the contiguous sub-range

@@ -207,7 +207,7 @@ typedef enum {
   HELM_LAUNCH_AUTO = 0,       /* persistent where the device can launch it (the
                                  whole FP64 solve of each method; the complex64
                                  inner solves of mixed precision up to some
-                                 700,000 unknowns), else graph; the host-driven
+                                 240,000 unknowns), else graph; the host-driven
                                  loop if the graph cannot be built */
   HELM_LAUNCH_GRAPH = 1,      /* CUDA graph with a device-driven while node;
                                  HELM_ERR_CUDA if it cannot be built */

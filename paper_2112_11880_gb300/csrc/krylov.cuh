@@ -110,8 +110,8 @@ __device__ __forceinline__ double nrm_acc(double acc, float2 a) {
 //   large: two blocks per SM of at most 512 threads (64 registers).
 // complex64 (the inner solves of mixed precision): mid or large (us per inner
 // iteration, persistent / graph / before: 20^3 29.7 / 33.9 / 44.5, 60x30x25 29.4 /
-// 34.5 / 37.1, 80x40x32 37.6 / 44.9 / 47, 120x60x50 68.4 / 73.8 / 77.9, 200x100x80
-// 191 / 184 / 205: on the large shape the default is the graph).
+// 34.5 / 37.1, 80x40x32 37.6 / 44.9 / 47; large: 120x60x50 71.5 / 77.9, 200x100x80
+// 191 / 184 / 205: there the default is the graph).
 // Measured (BiCGStab, us per iteration: persistent / graph kernels; before, on
 // one shape with graph kernels):
 //   20^3 box      (2 slices per SM)  small 25.7 / 39.0                       (39.7)
@@ -121,7 +121,11 @@ __device__ __forceinline__ double nrm_acc(double acc, float2 a) {
 //   200x100x80    (338)              mid  504 (512 threads), large 475 / 498 (478)
 // (mid of 640 threads: 37.3, 55.1, 121.5; 704: 40.5, 61.0, 124.1; more spill.)
 enum : int { SHAPE_SMALL = 0, SHAPE_MID = 1, SHAPE_LARGE = 2 };
-constexpr int kMidSlices = 150;  // slices per SM from which the shape is large
+constexpr int kMidSlices = 150;    // slices per SM from which the shape is large
+// for complex64 sooner: whether its inner solves converge on an indefinite system
+// of that size hangs on the order of their sums (kOrderedSums; 120x60x50 at 10
+// points per wavelength, inner_tol 0.01: converges on the large shape, not on mid)
+constexpr int kMidSlices32 = 50;
 template <int S> struct SolverBounds {
   static constexpr int threads = S == SHAPE_SMALL ? 384 : S == SHAPE_MID ? 768 : 512;  // warps of a split persistent kernel included
   static constexpr int blocks = S == SHAPE_LARGE ? 2 : 1;
@@ -989,7 +993,7 @@ template <class V>
 inline helm_status krylov_shapes(helm_csr A, KShapes<V>* sh) {
   const int64_t nsl = (static_cast<int64_t>(A->n) + 31) / 32, sms = A->num_sms;
   const bool c64 = std::is_same<V, float2>::value;
-  sh->shape = nsl > sms * kMidSlices                                                    ? SHAPE_LARGE
+  sh->shape = nsl > sms * (c64 ? kMidSlices32 : kMidSlices)                             ? SHAPE_LARGE
               : !c64 && nsl <= sms * (SolverBounds<SHAPE_SMALL>::threads / 32 / kParts) ? SHAPE_SMALL
                                                                                         : SHAPE_MID;
   sh->bps = sh->shape == SHAPE_LARGE ? SolverBounds<SHAPE_LARGE>::blocks : 1;

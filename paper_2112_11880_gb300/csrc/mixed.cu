@@ -611,7 +611,7 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
 
   // HELM_LAUNCH_AUTO: persistent inner solves where the device can launch them,
   // but the graph on the large shape (us per inner iteration on the 200x100x80
-  // cavity: 184 against 191; below, the persistent kernel is ahead by 5 to 6)
+  // cavity: 184 against 191; on mid the persistent kernel is ahead by 4 to 7)
   PShape ps;
   const void* inner = nullptr;
   with_shape(sh.k, [&](auto S) { inner = reinterpret_cast<const void*>(&k_mx_inner<S.value>); });

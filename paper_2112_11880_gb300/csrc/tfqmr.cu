@@ -21,8 +21,8 @@
 // shapes, rows and sums as BiCGStab's (krylov.cuh), the same bits in each.
 // What bounds it up to some 100,000 unknowns is the latency between steps.
 // Measured, us per iteration, persistent / graph / before (six graph kernels on
-// a grid of 1024-thread blocks): 20^3 box 28.7 / 39.8 / 53.0, 60x30x25 40.1 /
-// 43.7 / 63.5, 80x40x32 60.2 / 64.7 / 77.4, 120x60x50 130 / 139 / 170,
+// a grid of 1024-thread blocks): 20^3 box 28.7 / 39.8 / 53.0, 60x30x25 39.9 /
+// 44.4 / 63.5, 80x40x32 57.3 / 63.4 / 77.4, 120x60x50 130 / 139 / 170,
 // 200x100x80 519 / 533 / 552.
 #include <cmath>
 #include <cstring>

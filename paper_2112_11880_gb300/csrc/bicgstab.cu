@@ -97,7 +97,6 @@ helm_status bicgstab_fp64(helm_csr A, const double2* b, double2* x, const helm_o
   a.st = A->state;
   a.partials = A->partials;
   a.tickets = A->tickets;
-  a.gtickets = A->gtickets;
   a.dev_err = A->dev_err;
   HELM_CUDA_TRY(cudaMemsetAsync(A->dev_err, 0, sizeof(unsigned int), s));
   const int32_t use_x0_first = o.use_x0 ? 1 : 0;

@@ -38,10 +38,8 @@ enum : int32_t { PH_RUN = 0, PH_SCONV = 1, PH_DONE = 2 };
 
 // Tickets (arrival counters for last-block reductions), one per kernel kind.
 enum : int { TK_INIT = 0, TK_V, TK_S, TK_T, TK_XR, TK_TAIL, TK_AUX0, TK_AUX1, TK_AUX2, TK_AUX3,
-             TK_BAR_COUNT, TK_BAR_ABORT, TK_BAR_GEN,  // grid barrier of the persistent solver (count, abort adjacent)
+             TK_BAR_COUNT, TK_BAR_ABORT,  // grid barrier of the persistent solvers (adjacent)
              TK_COUNT };
-// Group counters per two-level reduction (groups of blockDim blocks).
-constexpr int kGroupTickets = 256;
 
 // The diagonals of a handle as pieces of up to three neighbours: diagonals d0[p],
 // ..., d0[p] + len[p] - 1 with offsets off[p], off[p] + 1, ...
@@ -94,7 +92,6 @@ struct helm_csr_s {
   // workspace (owned)
   double* partials = nullptr;          // max(grid) * 8 doubles
   unsigned int* tickets = nullptr;     // TK_COUNT counters
-  unsigned int* gtickets = nullptr;    // 2 x kGroupTickets group counters (K2, K4)
   unsigned int* dev_err = nullptr;     // device error flags
   helm::SolverState* state = nullptr;  // device
   helm::SolverState* state_host = nullptr;  // pinned host mirror
@@ -158,10 +155,9 @@ inline bool overlaps(const void* p, size_t pn, const void* q, size_t qn) {
 // Launch-shape helpers (api.cu).
 cudaError_t set_smem_attr(const void* fn, size_t bytes);
 int sm_count();
+int vec_grid_for(int64_t n);
 // Doubles of a handle's partial sums per SM: 32 blocks of 8 sums.
 constexpr size_t kPartialsPerSm = 32 * 8;
-
-int vec_grid_for(int64_t n);
 
 // Allocate the complex128 Krylov vectors (and FP32 ones) on first use.
 helm_status ensure_vectors(helm_csr A, int nvec);

@@ -146,7 +146,6 @@ struct KArgs {
   SolverState* st;
   double* partials;
   unsigned int* tickets;
-  unsigned int* gtickets;
   unsigned int* dev_err;
   cudaGraphConditionalHandle cond;
   int has_cond;

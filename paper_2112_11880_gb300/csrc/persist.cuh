@@ -24,6 +24,7 @@
 
 #include "common.cuh"
 #include "internal.hpp"
+#include "persist_plan.hpp"
 #include "spmv.cuh"
 
 namespace helm {
@@ -96,28 +97,13 @@ __device__ __forceinline__ void copy_state(SolverState* to, const SolverState* f
 
 // The block's warps: unsplit, each warp owns its slices' rows; split (small
 // meshes: one slice a warp), the first third own the rows and each row's sum is
-// shared out to three warps.
-//
-// Dynamic shared memory of a persistent kernel:
-//   table (rounds <= kTabRounds): per round and owner warp its slice (-1: none)
-//     and that slice's position, per round and owner thread the row's length;
-//     longer walks compute them;
-//   exchange (split): the helper warps' partial row sums;
-//   nown vectors of rounds x owner threads elements.
-constexpr int kTabRounds = 64;
-
+// shared out to three warps.  The block's dynamic shared memory is laid out by
+// persist_plan.hpp.
 struct RoundTab {
   SlicePos pos;
   int32_t s, pad_[3];
 };
-// Layout, worked out on the host (every field a kernel parameter).
-struct PLayout {
-  int32_t rounds, split, nown;
-  int32_t warps;                     // owner warps
-  int32_t tab;                       // the table is there
-  int32_t tlen_at, xchg_at, own_at;  // bytes from the start
-  int32_t own_len;                   // elements of an own vector
-};
+static_assert(sizeof(RoundTab) == kRoundTabBytes && sizeof(double2) == kExchangeBytes, "as the host lays them out");
 
 extern __shared__ __align__(128) unsigned char persist_smem[];
 
@@ -329,19 +315,6 @@ struct PShape {
   size_t smem = 0;
 };
 
-inline size_t persist_layout(PLayout* L, size_t elem) {
-  const size_t rounds = static_cast<size_t>(L->rounds), warps = static_cast<size_t>(L->warps);
-  L->tab = L->rounds <= kTabRounds;
-  const size_t tlen = L->tab ? rounds * warps * sizeof(RoundTab) : 0;
-  const size_t xchg = tlen + (L->tab ? rounds * warps * 32 * sizeof(int32_t) : 0);
-  const size_t own = xchg + static_cast<size_t>(L->split - 1) * warps * 32 * sizeof(double2);
-  L->tlen_at = static_cast<int32_t>(tlen);
-  L->xchg_at = static_cast<int32_t>(xchg);
-  L->own_at = static_cast<int32_t>(own);
-  L->own_len = static_cast<int32_t>(rounds * warps * 32);
-  return own + static_cast<size_t>(L->nown) * rounds * warps * 32 * elem;
-}
-
 // Fit a persistent kernel on a grid of `grid` blocks (bps per SM) of `owners`
 // owner threads, times `split` warps a slice: the table and as many of `want`
 // own vectors of `elem` bytes as there is room for.  False when the kernel
@@ -357,19 +330,10 @@ inline bool persist_fit(const void* fn, int32_t n, int grid, int owners, int bps
       cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
       cudaFuncGetAttributes(&fa, fn) != cudaSuccess)
     return false;
-  const int64_t nsl = (static_cast<int64_t>(n) + 31) / 32, W = static_cast<int64_t>(grid) * (owners / 32);
   p->grid = grid;
   p->threads = owners * split;
-  PLayout& L = p->L;
-  L.rounds = static_cast<int32_t>((nsl + W - 1) / W);
-  L.split = split;
-  L.warps = owners / 32;
   const size_t room = static_cast<size_t>(std::min(per_sm / bps - reserved, optin)) - fa.sharedSizeBytes;
-  L.nown = 0;
-  if (persist_layout(&L, elem) > room) return false;
-  L.nown = want;
-  while (persist_layout(&L, elem) > room) --L.nown;
-  p->smem = persist_layout(&L, elem);
+  if (!persist_plan(n, grid, owners, split, want, elem, room, &p->L, &p->smem)) return false;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            optin - static_cast<int>(fa.sharedSizeBytes)) != cudaSuccess)
     return false;

@@ -1,0 +1,67 @@
+// Plan of a persistent solver kernel (persist.cuh): the rounds of its grid and
+// the layout of a block's dynamic shared memory.  Host arithmetic only.
+#pragma once
+
+#include <stddef.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+namespace helm {
+
+// Dynamic shared memory of a block:
+//   table (rounds <= kTabRounds): per round and owner warp its slice (-1: none)
+//     and that slice's position, per round and owner thread the row's length;
+//     longer walks compute them;
+//   exchange (split): the helper warps' partial row sums (complex128);
+//   nown vectors of rounds x owner threads elements.
+constexpr int kTabRounds = 64;
+constexpr size_t kRoundTabBytes = 32, kExchangeBytes = 16;
+
+struct PLayout {
+  int32_t rounds, split, nown;
+  int32_t warps;                     // owner warps
+  int32_t tab;                       // the table is there
+  int32_t tlen_at, xchg_at, own_at;  // bytes from the start
+  int32_t own_len;                   // elements of an own vector
+};
+
+// Rounds of `grid` blocks of `warps` owner warps over the slices of n rows.  One
+// at least: a split kernel reads the first round's entry whatever n is (without
+// rows it says that there is no slice).
+inline int32_t persist_rounds(int32_t n, int grid, int warps) {
+  const int64_t nsl = (static_cast<int64_t>(n) + 31) / 32, W = static_cast<int64_t>(grid) * warps;
+  return static_cast<int32_t>(std::max<int64_t>((nsl + W - 1) / W, 1));
+}
+
+// The offsets for L's rounds, warps, split and nown; returns the bytes in all.
+inline size_t persist_layout(PLayout* L, size_t elem) {
+  const size_t rounds = static_cast<size_t>(L->rounds), warps = static_cast<size_t>(L->warps);
+  L->tab = L->rounds <= kTabRounds;
+  const size_t tlen = L->tab ? rounds * warps * kRoundTabBytes : 0;
+  const size_t xchg = tlen + (L->tab ? rounds * warps * 32 * sizeof(int32_t) : 0);
+  const size_t own = xchg + static_cast<size_t>(L->split - 1) * warps * 32 * kExchangeBytes;
+  L->tlen_at = static_cast<int32_t>(tlen);
+  L->xchg_at = static_cast<int32_t>(xchg);
+  L->own_at = static_cast<int32_t>(own);
+  L->own_len = static_cast<int32_t>(rounds * warps * 32);
+  return own + static_cast<size_t>(L->nown) * rounds * warps * 32 * elem;
+}
+
+// The layout on a grid of `grid` blocks of `owners` owner threads, `split` warps
+// a slice: the table and as many of `want` own vectors of `elem` bytes as `room`
+// bytes hold.  *bytes is what it takes; false when it does not fit.
+inline bool persist_plan(int32_t n, int grid, int owners, int split, int want, size_t elem, size_t room, PLayout* L,
+                         size_t* bytes) {
+  L->warps = owners / 32;
+  L->rounds = persist_rounds(n, grid, L->warps);
+  L->split = split;
+  L->nown = 0;
+  if (persist_layout(L, elem) > room) return false;
+  L->nown = want;
+  while (persist_layout(L, elem) > room) --L->nown;
+  *bytes = persist_layout(L, elem);
+  return true;
+}
+
+}  // namespace helm

@@ -1,0 +1,52 @@
+// Checks of the persistent solvers' plan (persist_plan.hpp), compiled and run by
+// test_persist_plan_cpu.py: every entry that a kernel reads lies in the part of
+// its shared memory that the plan gave it, also for a system without rows.
+#include <cstdio>
+#include <cstring>
+
+#include "persist_plan.hpp"
+
+static int failures = 0;
+#define CHECK(c)                                              \
+  do {                                                        \
+    if (!(c)) {                                               \
+      std::printf("FAILED line %d: %s\n", __LINE__, #c);      \
+      ++failures;                                             \
+    }                                                         \
+  } while (0)
+
+// The parts in order, none overlapping the next, all inside `room`.
+static void check_layout(const helm::PLayout& L, size_t bytes, size_t elem, size_t room) {
+  const size_t entries = static_cast<size_t>(L.rounds) * L.warps;
+  CHECK(bytes <= room);
+  if (L.tab) {
+    CHECK(static_cast<size_t>(L.tlen_at) >= entries * helm::kRoundTabBytes);
+    CHECK(static_cast<size_t>(L.xchg_at) >= L.tlen_at + entries * 32 * sizeof(int32_t));
+  }
+  CHECK(static_cast<size_t>(L.own_at) >= L.xchg_at + static_cast<size_t>(L.split - 1) * L.warps * 32 * 16);
+  CHECK(static_cast<size_t>(L.own_len) == entries * 32);
+  CHECK(bytes >= L.own_at + static_cast<size_t>(L.nown) * L.own_len * elem);
+  CHECK(L.tlen_at % 16 == 0 && L.xchg_at % 16 == 0 && L.own_at % 16 == 0);
+}
+
+// No rows: one round all the same, whose entry (no slice) a split kernel reads
+// before anything else.
+static void empty_system() {
+  for (int split : {1, 3})
+    for (int owners : {32, 128}) {
+      helm::PLayout L;
+      size_t bytes = 0;
+      std::memset(&L, 0, sizeof(L));
+      CHECK(helm::persist_plan(0, 1, owners, split, 7, 16, 200000, &L, &bytes));
+      CHECK(L.rounds >= 1 && L.tab);
+      check_layout(L, bytes, 16, 200000);
+    }
+}
+
+int main(int argc, char** argv) {
+  const char* what = argc > 1 ? argv[1] : "";
+  if (!std::strcmp(what, "empty")) empty_system();
+  else ++failures;
+  if (failures == 0) std::printf("ok\n");
+  return failures == 0 ? 0 : 1;
+}

@@ -10,12 +10,11 @@
 namespace helm {
 
 // Dynamic shared memory of a block:
-//   table (rounds <= kTabRounds): per round and owner warp its slice (-1: none)
-//     and that slice's position, per round and owner thread the row's length;
-//     longer walks compute them;
+//   table (where it fits): per round and owner warp its slice (-1: none) and that
+//     slice's position, per round and owner thread the row's length; without it
+//     the kernel works them out at every product (unsplit kernels only);
 //   exchange (split): the helper warps' partial row sums (complex128);
 //   nown vectors of rounds x owner threads elements.
-constexpr int kTabRounds = 64;
 constexpr size_t kRoundTabBytes = 32, kExchangeBytes = 16;
 
 struct PLayout {
@@ -34,10 +33,9 @@ inline int32_t persist_rounds(int32_t n, int grid, int warps) {
   return static_cast<int32_t>(std::max<int64_t>((nsl + W - 1) / W, 1));
 }
 
-// The offsets for L's rounds, warps, split and nown; returns the bytes in all.
+// The offsets for L's rounds, warps, split, tab and nown; returns the bytes in all.
 inline size_t persist_layout(PLayout* L, size_t elem) {
   const size_t rounds = static_cast<size_t>(L->rounds), warps = static_cast<size_t>(L->warps);
-  L->tab = L->rounds <= kTabRounds;
   const size_t tlen = L->tab ? rounds * warps * kRoundTabBytes : 0;
   const size_t xchg = tlen + (L->tab ? rounds * warps * 32 * sizeof(int32_t) : 0);
   const size_t own = xchg + static_cast<size_t>(L->split - 1) * warps * 32 * kExchangeBytes;
@@ -49,14 +47,20 @@ inline size_t persist_layout(PLayout* L, size_t elem) {
 }
 
 // The layout on a grid of `grid` blocks of `owners` owner threads, `split` warps
-// a slice: the table and as many of `want` own vectors of `elem` bytes as `room`
-// bytes hold.  *bytes is what it takes; false when it does not fit.
+// a slice: the table, dropped where it does not fit (two blocks per SM of 16 warps:
+// from 45 rounds on, 6.9 million unknowns), and as many of `want` own vectors of
+// `elem` bytes as `room` bytes hold.  *bytes is what it takes; false when it does
+// not fit.  Without the table (27 entries a row, us per BiCGStab iteration, graph /
+// persistent): 7.2 million unknowns 1,997 / 1,909, 9 million 2,471 / 2,361, 10.5
+// million 2,880 / 2,758; with it, 6.5 million: 1,798 / 1,750.
 inline bool persist_plan(int32_t n, int grid, int owners, int split, int want, size_t elem, size_t room, PLayout* L,
                          size_t* bytes) {
   L->warps = owners / 32;
   L->rounds = persist_rounds(n, grid, L->warps);
   L->split = split;
   L->nown = 0;
+  L->tab = 1;
+  if (persist_layout(L, elem) > room && split == 1) L->tab = 0;
   if (persist_layout(L, elem) > room) return false;
   L->nown = want;
   while (persist_layout(L, elem) > room) --L->nown;

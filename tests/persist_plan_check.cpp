@@ -43,9 +43,36 @@ static void empty_system() {
     }
 }
 
+// Two blocks of 16 warps on each of 152 SMs, some 113 kB each: a plan for every
+// number of rounds, with the table while it fits; a split kernel never goes without.
+static void many_rounds() {
+  const int grid = 304, owners = 512;
+  const size_t room = 113000;
+  int last_tab = 0;
+  for (int rounds = 1; rounds <= 400; ++rounds)
+    for (int extra : {-31, 0}) {
+      const int32_t n = rounds * grid * owners + extra;
+      helm::PLayout L;
+      size_t bytes = 0;
+      std::memset(&L, 0, sizeof(L));
+      CHECK(helm::persist_plan(n, grid, owners, 1, 7, 16, room, &L, &bytes));
+      CHECK(L.rounds == rounds);
+      check_layout(L, bytes, 16, room);
+      if (L.tab) {
+        CHECK(last_tab >= rounds - 1);
+        last_tab = rounds;
+      }
+    }
+  CHECK(last_tab == 44);
+  helm::PLayout L;
+  size_t bytes = 0;
+  CHECK(!helm::persist_plan(100 * grid * 128, grid, 128, 3, 7, 16, 20000, &L, &bytes));
+}
+
 int main(int argc, char** argv) {
   const char* what = argc > 1 ? argv[1] : "";
   if (!std::strcmp(what, "empty")) empty_system();
+  else if (!std::strcmp(what, "rounds")) many_rounds();
   else ++failures;
   if (failures == 0) std::printf("ok\n");
   return failures == 0 ? 0 : 1;

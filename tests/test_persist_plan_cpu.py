@@ -28,3 +28,7 @@ def check(tmp_path_factory):
 
 def test_a_system_without_rows_has_a_round(check):
     check("empty")
+
+
+def test_every_number_of_rounds_has_a_plan(check):
+    check("rounds")

@@ -608,22 +608,23 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   a.tickets = A->tickets;
   a.dev_err = A->dev_err;
 
-  // HELM_LAUNCH_AUTO: persistent inner solves where the device can launch them,
+  // HELM_LAUNCH_AUTO: persistent inner solves where the device takes the launch
+  // (else the graphs: a context can have fewer SMs than the device reports),
   // but the graph on the large shape (us per inner iteration on the 200x100x80
   // cavity: 184 against 191; on mid the persistent kernel is ahead by 4 to 7)
   PShape ps;
   const void* inner = nullptr;
   with_shape(sh.k, [&](auto S) { inner = reinterpret_cast<const void*>(&k_mx_inner<S.value>); });
-  const bool persistent = o.launch == HELM_LAUNCH_AUTO && sh.k.shape != SHAPE_LARGE &&
-                          persist_fit(inner, n, sh.k.grid, sh.k.threads, sh.k.bps, 1,
-                                                                 Phases<float2>::kOwn, sizeof(float2), &ps);
+  bool persistent = o.launch == HELM_LAUNCH_AUTO && sh.k.shape != SHAPE_LARGE &&
+                    persist_fit(inner, n, sh.k.grid, sh.k.threads, sh.k.bps, 1, Phases<float2>::kOwn, sizeof(float2),
+                                &ps);
   (void)cudaGetLastError();
 
   // the inner-loop graph and the step graph per (b, x), tagged as mixed in
   // the cache key
   GraphEntry* gi = nullptr;
   GraphEntry* gs = nullptr;
-  if (o.launch != HELM_LAUNCH_HOST && !persistent) {
+  auto make_graphs = [&] {
     auto ki = graph_key(b, x, 2, o), ks = graph_key(b, x, 3, o);
     auto ii = A->graphs.find(ki), is = A->graphs.find(ks);
     if (ii != A->graphs.end() && is != A->graphs.end()) {
@@ -648,7 +649,8 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
         if (ei.graph) cudaGraphDestroy(ei.graph);
       }
     }
-  }
+  };
+  if (o.launch != HELM_LAUNCH_HOST && !persistent) make_graphs();
 
   // an explicit graph request does not fall back to the host-driven loop
   if (!gi && o.launch == HELM_LAUNCH_GRAPH) return HELM_ERR_CUDA;
@@ -663,7 +665,14 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
     if (persistent) {
       HELM_CUDA_TRY(cudaMemsetAsync(A->tickets + TK_BAR_COUNT, 0, 2 * sizeof(unsigned int), s));  // count, abort
       void* args[] = {&k, &ps.L};
-      HELM_CUDA_TRY(cudaLaunchCooperativeKernel(inner, dim3(ps.grid), dim3(ps.threads), args, ps.smem, s));
+      const cudaError_t e = cudaLaunchCooperativeKernel(inner, dim3(ps.grid), dim3(ps.threads), args, ps.smem, s);
+      if (e != cudaSuccess) {  // nothing has run: the inner solve starts from the same state
+        debug_cuda_error(e, __FILE__, __LINE__);
+        (void)cudaGetLastError();
+        persistent = false;
+        make_graphs();
+        continue;
+      }
       mx_step(a, sh, s);
       HELM_CUDA_TRY(cudaGetLastError());
       HELM_CUDA_TRY(cudaMemcpyAsync(&herr, A->dev_err, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));

@@ -332,7 +332,7 @@ inline bool persist_fit(const void* fn, int32_t n, int grid, int owners, int bps
     return false;
   p->grid = grid;
   p->threads = owners * split;
-  const size_t room = static_cast<size_t>(std::min(per_sm / bps - reserved, optin)) - fa.sharedSizeBytes;
+  const size_t room = persist_room(per_sm, optin, reserved, fa.sharedSizeBytes, bps);
   if (!persist_plan(n, grid, owners, split, want, elem, room, &p->L, &p->smem)) return false;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            optin - static_cast<int>(fa.sharedSizeBytes)) != cudaSuccess)

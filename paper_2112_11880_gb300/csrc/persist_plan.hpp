@@ -46,9 +46,24 @@ inline size_t persist_layout(PLayout* L, size_t elem) {
   return own + static_cast<size_t>(L->nown) * rounds * warps * 32 * elem;
 }
 
+// Shared memory a block may take, of `bps` blocks per SM that have `per_sm` bytes
+// between them: `reserved` and `fixed` (static) bytes go off each.  All blocks of
+// an SM stay within kPersistSmem, because what they leave of its 256 kB is L1, and
+// a warp's gathers from scattered columns each hold a line of it while they are in
+// flight: own vectors in shared memory gain next to nothing (120x60x50, us per
+// BiCGStab iteration with 16 / 48 / 112 / 227 kB per SM: 120 / 121 / 122 / 121), a
+// small L1 costs up to a factor of two where columns are scattered (27 a row, n =
+// 400,009: 141 / 141 / 143 / 251; TFQMR, 200,003: 90 / 88 / 89 / 141; BiCGStab,
+// 1,600,003: 477 / 478 / 505 / 1205).
+constexpr size_t kPersistSmem = 100 * 1024;
+inline size_t persist_room(size_t per_sm, size_t optin, size_t reserved, size_t fixed, int bps) {
+  const size_t block = std::min(std::min(per_sm, kPersistSmem) / bps - reserved, optin);
+  return block > fixed ? block - fixed : 0;
+}
+
 // The layout on a grid of `grid` blocks of `owners` owner threads, `split` warps
 // a slice: the table, dropped where it does not fit (two blocks per SM of 16 warps:
-// from 45 rounds on, 6.9 million unknowns), and as many of `want` own vectors of
+// from 20 rounds on, 3 million unknowns), and as many of `want` own vectors of
 // `elem` bytes as `room` bytes hold.  *bytes is what it takes; false when it does
 // not fit.  Without the table (27 entries a row, us per BiCGStab iteration, graph /
 // persistent): 7.2 million unknowns 1,997 / 1,909, 9 million 2,471 / 2,361, 10.5

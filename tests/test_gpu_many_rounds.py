@@ -31,7 +31,7 @@ def _banded(n, seed):
     return rowptr, cols[ok].to(torch.int32).contiguous(), torch.complex(re, im)[ok].contiguous()
 
 
-@pytest.mark.parametrize("rounds,extra", [(44, 0), (44, 1), (45, -7), (64, -31), (64, 1)])
+@pytest.mark.parametrize("rounds,extra", [(18, 0), (19, 1), (20, 0), (44, 0), (44, 1), (45, -7), (64, -31), (64, 1)])
 @pytest.mark.parametrize("method", [helm.HELM_BICGSTAB, helm.HELM_TFQMR, helm.HELM_BICGSTABL])
 def test_rounds_without_a_table(rounds, extra, method):
     n = rounds * ROUND + extra

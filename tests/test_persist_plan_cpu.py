@@ -32,3 +32,7 @@ def test_a_system_without_rows_has_a_round(check):
 
 def test_every_number_of_rounds_has_a_plan(check):
     check("rounds")
+
+
+def test_blocks_leave_an_sm_its_l1(check):
+    check("l1")

@@ -37,11 +37,6 @@ __device__ __forceinline__ unsigned int ld_relaxed_u32(const unsigned int* p) {
   return v;
 }
 
-// Polls after which a wait gives up: a poll is a round trip to L2, at least
-// 0.5 us, so no wait ends before 2 s of the kernel's own running time (time
-// during which the GPU runs another process does not count).
-constexpr int kBarrierPolls = 1 << 22;
-
 // A grid barrier for a cooperative launch (all blocks resident).  The count
 // word only grows (zero before the launch): thread 0 of each block adds one
 // and waits until the count reaches gridDim.x times the number of barriers

@@ -9,6 +9,12 @@
 
 namespace helm {
 
+// Polls after which a wait of the grid barrier gives up.  A poll is a round trip to
+// L2: 0.228 us on one block, 0.237 on 304 (measured at 2070 MHz), so no wait ends
+// before 2 s of the kernel's own running time (time during which the GPU runs
+// another process does not count).
+constexpr int kBarrierPolls = 9 << 20;
+
 // Dynamic shared memory of a block:
 //   table (where it fits): per round and owner warp its slice (-1: none) and that
 //     slice's position, per round and owner thread the row's length; without it

@@ -36,3 +36,7 @@ def test_every_number_of_rounds_has_a_plan(check):
 
 def test_blocks_leave_an_sm_its_l1(check):
     check("l1")
+
+
+def test_a_wait_lasts_two_seconds_of_polls(check):
+    check("wait")

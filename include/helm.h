@@ -208,7 +208,10 @@ typedef enum {
                                  whole FP64 solve of each method; the complex64
                                  inner solves of mixed precision up to some
                                  240,000 unknowns), else graph; the host-driven
-                                 loop if the graph cannot be built */
+                                 loop if the graph cannot be built.  Graph also
+                                 for matrices with long rows (FP64 above 262,144
+                                 entries, 192 beyond some 730,000 unknowns;
+                                 mixed precision above 128) */
   HELM_LAUNCH_GRAPH = 1,      /* CUDA graph with a device-driven while node;
                                  HELM_ERR_CUDA if it cannot be built */
   HELM_LAUNCH_PERSISTENT = 2, /* FP64 BiCGStab only (HELM_ERR_INVALID for

@@ -104,9 +104,10 @@ helm_status bicgstab_fp64(helm_csr A, const double2* b, double2* x, const helm_o
   unsigned int herr = 0;
 
   // persistent: the whole solve, restarts included, is one cooperative
-  // launch; HELM_LAUNCH_AUTO takes it wherever the device can run it
+  // launch; HELM_LAUNCH_AUTO takes it unless rows are long (persist_max_row)
+  // or the device cannot run it
   bool done = false;
-  if (o.launch == HELM_LAUNCH_PERSISTENT || o.launch == HELM_LAUNCH_AUTO) {
+  if (o.launch == HELM_LAUNCH_PERSISTENT || persist_default(A, sh, o)) {
     const void* fn = nullptr;
     int split = 1;
     with_shape(sh, [&](auto S) {

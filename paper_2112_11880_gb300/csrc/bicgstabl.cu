@@ -638,7 +638,7 @@ helm_status bicgstabl_fp64(helm_csr A, const double2* b, double2* x, const helm_
   SolverState* hs = A->state_host;
   HELM_CUDA_TRY(cudaMemsetAsync(A->dev_err, 0, sizeof(unsigned int), s));
   bool done = false;
-  if (o.launch == HELM_LAUNCH_AUTO) {
+  if (persist_default(A, sh, o)) {
     const void* fn = nullptr;
     int split = 1;
     with_shape(sh, [&](auto S) {

@@ -898,6 +898,13 @@ struct KShapes {
   int shape;    // SHAPE_*
 };
 
+// HELM_LAUNCH_AUTO takes a persistent kernel for this solve (where the device can).
+template <class V>
+inline bool persist_default(helm_csr A, const KShapes<V>& sh, const helm_opts& o) {
+  return o.launch == HELM_LAUNCH_AUTO &&
+         A->max_row <= persist_max_row(sh.shape == SHAPE_LARGE, std::is_same<V, float2>::value);
+}
+
 // A whole solve as one cooperative launch of `fn` on the shape that persist_fit
 // gave it; the final state is in A->state_host.  *done stays false (and nothing
 // has run) when the device did not take the launch.

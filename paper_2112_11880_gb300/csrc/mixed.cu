@@ -615,7 +615,7 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   PShape ps;
   const void* inner = nullptr;
   with_shape(sh.k, [&](auto S) { inner = reinterpret_cast<const void*>(&k_mx_inner<S.value>); });
-  bool persistent = o.launch == HELM_LAUNCH_AUTO && sh.k.shape != SHAPE_LARGE &&
+  bool persistent = persist_default(A, sh.k, o) && sh.k.shape != SHAPE_LARGE &&
                     persist_fit(inner, n, sh.k.grid, sh.k.threads, sh.k.bps, 1, Phases<float2>::kOwn, sizeof(float2),
                                 &ps);
   (void)cudaGetLastError();

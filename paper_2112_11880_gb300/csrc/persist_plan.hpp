@@ -89,4 +89,21 @@ inline bool persist_plan(int32_t n, int grid, int owners, int split, int want, s
   return true;
 }
 
+// Longest row up to which HELM_LAUNCH_AUTO runs a solve as a persistent kernel; the
+// graph beyond.  A product lasts as long as its longest row's chain of loads, and
+// the graph's pipeline is deeper (four entries a stage against three, or two on the
+// large shape).
+// Measured (one long row of L entries among rows of five; us per iteration,
+// persistent / graph; before persistent kernels):
+//   large shape, n = 1,000,000: BiCGStab L = 128 224 / 238 (234), 192 267 / 274
+//     (274), 256 314 / 310 (312), 1024 835 / 735 (791); TFQMR 192 280 / 268 (318),
+//     1024 852 / 736 (831); BiCGStab(2) 192 542 / 545 (660), 1024 1591 / 1471 (1652);
+//   complex64, n = 240,000: L = 64 50 / 56 (57), 128 67 / 67 (67), 192 90 / 83 (82),
+//     1024 336 / 249 (259);
+//   mid, n = 100,000: L = 1024 BiCGStab 384 / 352 (408), TFQMR 385 / 399 (434),
+//     BiCGStab(2) 836 / 729 (915): ahead of what was at every length.
+// Above 2^18 a step would come near the time that a wait lasts (1.1 s a product of a
+// row of 3.3 million entries; an entry with an imaginary part takes longer).
+inline int32_t persist_max_row(bool large, bool c64) { return c64 ? 128 : large ? 192 : 1 << 18; }
+
 }  // namespace helm

@@ -566,7 +566,7 @@ helm_status tfqmr_fp64(helm_csr A, const double2* b, double2* x, const helm_opts
   int32_t use_x0 = o.use_x0 ? 1 : 0, fresh = 1;
   HELM_CUDA_TRY(cudaMemsetAsync(A->dev_err, 0, sizeof(unsigned int), s));
   bool done = false;
-  if (o.launch == HELM_LAUNCH_AUTO) {
+  if (persist_default(A, sh, o)) {
     const void* fn = nullptr;
     int split = 1;
     with_shape(sh, [&](auto S) {

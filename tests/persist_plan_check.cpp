@@ -87,11 +87,23 @@ static void leaves_l1() {
   CHECK(helm::persist_room(233472, 232448, 1024, 200000, 2) == 0);
 }
 
+// By default a step of a persistent kernel stays well inside a wait's 2 s: at the
+// longest row that it takes, with 4 us an entry to spare; and the deeper pipeline of
+// the graph gets the long rows where the kernel's own is shallower.
+static void long_rows() {
+  for (bool large : {false, true})
+    for (bool c64 : {false, true}) CHECK(helm::persist_max_row(large, c64) * 4e-6 <= 1.1);
+  CHECK(helm::persist_max_row(false, false) > helm::persist_max_row(true, false));
+  CHECK(helm::persist_max_row(true, false) > helm::persist_max_row(false, true));
+  CHECK(helm::persist_max_row(false, true) >= 64);  // meshes of second order stay on it
+}
+
 int main(int argc, char** argv) {
   const char* what = argc > 1 ? argv[1] : "";
   if (!std::strcmp(what, "empty")) empty_system();
   else if (!std::strcmp(what, "rounds")) many_rounds();
   else if (!std::strcmp(what, "l1")) leaves_l1();
+  else if (!std::strcmp(what, "long")) long_rows();
   else if (!std::strcmp(what, "wait")) CHECK(helm::kBarrierPolls * 0.2277e-6 >= 2.0);
   else ++failures;
   if (failures == 0) std::printf("ok\n");

@@ -41,3 +41,21 @@ def test_a_step_of_more_than_a_second():
     assert out[0][1]["status"] == "not_converged" and out[0][1] == out[1][1]
     assert torch.equal(torch.view_as_real(out[0][0]), torch.view_as_real(out[1][0]))
     A.close()
+
+
+@pytest.mark.parametrize("n,length,precision", [
+    (300_000, 128, helm.HELM_PREC_MIXED), (200_000, 129, helm.HELM_PREC_MIXED), (200_000, 3000, helm.HELM_PREC_MIXED),
+    (15_000, 15_000, helm.HELM_PREC_FP64), (300_000, 1 << 18, helm.HELM_PREC_FP64),
+    (300_000, (1 << 18) + 1, helm.HELM_PREC_FP64), (1_000_000, 192, helm.HELM_PREC_FP64),
+    (1_000_000, 193, helm.HELM_PREC_FP64),
+])
+def test_forms_agree_on_both_sides_of_the_rule(n, length, precision):
+    A = helm.CsrMatrix(*long_row(n, length))
+    gen = torch.Generator(device=DEV).manual_seed(2)
+    b = torch.view_as_complex(torch.rand(n, 2, generator=gen, device=DEV, dtype=torch.float64))
+    for method in (helm.HELM_BICGSTAB, helm.HELM_TFQMR, helm.HELM_BICGSTABL)[: 1 if precision else 3]:
+        out = [helm.solve(A, b, tol=1e-10, maxit=60, method=method, precision=precision, launch=l)
+               for l in (helm.HELM_LAUNCH_GRAPH, helm.HELM_LAUNCH_AUTO)]
+        assert out[0][1]["status"] == "ok" and out[0][1] == out[1][1]
+        assert torch.equal(torch.view_as_real(out[0][0]), torch.view_as_real(out[1][0]))
+    A.close()

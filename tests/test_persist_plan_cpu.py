@@ -40,3 +40,7 @@ def test_blocks_leave_an_sm_its_l1(check):
 
 def test_a_wait_lasts_two_seconds_of_polls(check):
     check("wait")
+
+
+def test_long_rows_are_left_to_the_graph(check):
+    check("long")

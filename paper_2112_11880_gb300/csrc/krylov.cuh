@@ -255,6 +255,44 @@ __device__ __forceinline__ void sum_components(const double* partials, int G, in
   __syncthreads();
 }
 
+// put_block_partials and sum_components where a block is one warp, which would add
+// the components one after the other: the same sums, the components side by side
+// (graph kernels of meshes up to one slice per SM: us per iteration of the 15^3 box,
+// BiCGStab 36.4 -> 34.4, complex64 33.3 -> 31.8).
+template <int K>
+__device__ __forceinline__ void put_warp_partials(const double (&v)[K], double* partials) {
+  const int lane = threadIdx.x & 31;
+  const double ws = warp_sum_t<K>(v);
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if (lane == warp_sum_lane<K>(k)) partials[static_cast<size_t>(k) * gridDim.x + blockIdx.x] = ws;
+}
+template <int K>
+__device__ __forceinline__ void sum_warp_partials(const double* partials, int G, double (&tot)[K]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k < K; ++k) tot[k] = 0.0;
+#pragma unroll 1
+  for (int j0 = lane; j0 < G; j0 += 5 * 32) {
+    double w[K][5];
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+      for (int u = 0; u < 5; ++u)
+        w[k][u] = j0 + 32 * u < G ? ld_cg(&partials[static_cast<size_t>(k) * G + j0 + 32 * u]) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 5; ++u)
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        if (j0 + 32 * u < G) tot[k] += w[k][u];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+    for (int k = 0; k < K; ++k) tot[k] += __shfl_xor_sync(0xffffffffu, tot[k], off);
+}
+
 // Fixed-order totals of all blocks' partials, valid in thread 0: sum_components,
 // or thread j adds blocks j, j + T, ..., then the block tree.
 template <class V, int S, int K>
@@ -285,7 +323,9 @@ template <class V, int S, int K>
 __device__ __forceinline__ bool grid_total_last(double (&v)[K], double* partials, unsigned int* ticket, double* red,
                                                 double (&tot)[K]) {
   __shared__ bool s_last;
-  put_block_partials<V, S, K>(v, red, partials);
+  const bool one_warp = S != SHAPE_LARGE && blockDim.x == 32;
+  if (one_warp) put_warp_partials<K>(v, partials);
+  else put_block_partials<V, S, K>(v, red, partials);
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -294,7 +334,8 @@ __device__ __forceinline__ bool grid_total_last(double (&v)[K], double* partials
   __syncthreads();
   if (!s_last) return false;
   __threadfence();
-  sum_block_partials<V, S, K>(partials, gridDim.x, red, tot);
+  if (one_warp) sum_warp_partials<K>(partials, gridDim.x, tot);
+  else sum_block_partials<V, S, K>(partials, gridDim.x, red, tot);
   if (threadIdx.x == 0) *ticket = 0u;
   return true;
 }

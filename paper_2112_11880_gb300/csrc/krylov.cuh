@@ -615,10 +615,12 @@ struct Phases {
   }
 
   // P1: p = r + beta (p - omega v)
+  template <bool AHEAD>
   __device__ __forceinline__ void upd_p(V beta, V omega) const {
-    for_rows(q, n(), [&](int32_t i, int li) {
-      p.st_both(i, li, cfma(beta, cfms(omega, v.ld(i, li), p.ld(i, li)), r.ld(i, li)));
-    });
+    struct Ops { V v, p, r; };
+    for_rows_ld<AHEAD>(
+        q, n(), [&](int32_t i, int li) { return Ops{v.ld(i, li), p.ld(i, li), r.ld(i, li)}; },
+        [&](int32_t i, int li, const Ops& o) { p.st_both(i, li, cfma(beta, cfms(omega, o.v, o.p), o.r)); });
   }
 
   // P2: v = A p, (r^, v)
@@ -630,12 +632,16 @@ struct Phases {
   }
 
   // P3: s = r - alpha v, ||s||^2
+  template <bool AHEAD>
   __device__ __forceinline__ void upd_s(V alpha, double (&part)[4]) const {
-    for_rows(q, n(), [&](int32_t i, int li) {
-      const V sn = cfms(alpha, v.ld(i, li), r.ld(i, li));
-      s.st_both(i, li, sn);
-      part[0] = nrm_acc(part[0], sn);
-    });
+    struct Ops { V v, r; };
+    for_rows_ld<AHEAD>(
+        q, n(), [&](int32_t i, int li) { return Ops{v.ld(i, li), r.ld(i, li)}; },
+        [&](int32_t i, int li, const Ops& o) {
+          const V sn = cfms(alpha, o.v, o.r);
+          s.st_both(i, li, sn);
+          part[0] = nrm_acc(part[0], sn);
+        });
   }
 
   // P4: t = A s, (t, s), ||t||^2
@@ -649,21 +655,25 @@ struct Phases {
 
   // P5: x += alpha p + omega s, r = s - omega t; (r^, r), ||r||^2.  With sconv
   // (the solve stopped at s) only x += alpha p.
+  template <bool AHEAD>
   __device__ __forceinline__ void upd_xr(V alpha, V omega, bool sconv, double (&part)[4]) const {
     if (sconv) {
       for_rows(q, n(), [&](int32_t i, int li) { x.st(i, li, cfma(alpha, p.ld(i, li), x.ld(i, li))); });
       return;
     }
-    for_rows(q, n(), [&](int32_t i, int li) {
-      const V si = s.ld(i, li);
-      x.st(i, li, cfma(omega, si, cfma(alpha, p.ld(i, li), x.ld(i, li))));
-      const V ri = cfms(omega, t.ld(i, li), si);
-      r.st(i, li, ri);
-      const double2 d = dot_acc(make_double2(part[0], part[1]), rh.ld(i, li), ri);
-      part[0] = d.x;
-      part[1] = d.y;
-      part[2] = nrm_acc(part[2], ri);
-    });
+    struct Ops { V s, p, x, t, rh; };
+    for_rows_ld<AHEAD>(
+        q, n(),
+        [&](int32_t i, int li) { return Ops{s.ld(i, li), p.ld(i, li), x.ld(i, li), t.ld(i, li), rh.ld(i, li)}; },
+        [&](int32_t i, int li, const Ops& o) {
+          x.st(i, li, cfma(omega, o.s, cfma(alpha, o.p, o.x)));
+          const V ri = cfms(omega, o.t, o.s);
+          r.st(i, li, ri);
+          const double2 d = dot_acc(make_double2(part[0], part[1]), o.rh, ri);
+          part[0] = d.x;
+          part[1] = d.y;
+          part[2] = nrm_acc(part[2], ri);
+        });
   }
 };
 
@@ -716,7 +726,7 @@ HELM_SOLVER_KERNEL k_p(const __grid_constant__ KArgs<V> a) {
   const SolverState* st = a.st;
   if (st->status != ST_RUNNING || refine_step_pending<V>(st)) return;
   const PLayout lay = graph_layout(a.A.n);
-  Phases<V>(a, lay).upd_p(Prec<V>::cvt(st->beta), Prec<V>::cvt(st->omega));
+  Phases<V>(a, lay).template upd_p<true>(Prec<V>::cvt(st->beta), Prec<V>::cvt(st->omega));
 }
 
 // K2: v = A p, (r^, v) -> alpha
@@ -744,7 +754,7 @@ HELM_SOLVER_KERNEL k_s(const __grid_constant__ KArgs<V> a) {
   SolverState* st = a.st;
   if (st->status != ST_RUNNING || refine_step_pending<V>(st)) return;
   HELM_GRAPH_PHASES
-  ph.upd_s(Prec<V>::cvt(st->alpha), part);
+  ph.template upd_s<true>(Prec<V>::cvt(st->alpha), part);
   double part1[1] = {part[0]}, tot[1];
   if (!grid_total_last<V, S, 1>(part1, a.partials, a.tickets + TK_S, red, tot)) return;
   if (threadIdx.x != 0) return;
@@ -780,7 +790,7 @@ HELM_SOLVER_KERNEL k_xr(const __grid_constant__ KArgs<V> a) {
     return;
   }
   HELM_GRAPH_PHASES
-  ph.upd_xr(Prec<V>::cvt(st->alpha), Prec<V>::cvt(st->omega), st->phase == PH_SCONV, part);
+  ph.template upd_xr<true>(Prec<V>::cvt(st->alpha), Prec<V>::cvt(st->omega), st->phase == PH_SCONV, part);
   double part3[3] = {part[0], part[1], part[2]}, tot[3];
   if (!grid_total_last<V, S, 3>(part3, a.partials, a.tickets + TK_XR, red, tot)) return;
   if (threadIdx.x != 0) return;
@@ -828,11 +838,11 @@ __device__ __forceinline__ void persist_loop(const KArgs<V>& a, const PLayout& L
   while (step != STEP_END) {
     double part[4] = {0.0, 0.0, 0.0, 0.0};
     if (step == STEP_P) {
-      ph.upd_p(Prec<V>::cvt(sst.beta), Prec<V>::cvt(sst.omega));
+      ph.template upd_p<false>(Prec<V>::cvt(sst.beta), Prec<V>::cvt(sst.omega));
     } else if (step == STEP_S) {
-      ph.upd_s(Prec<V>::cvt(sst.alpha), part);
+      ph.template upd_s<false>(Prec<V>::cvt(sst.alpha), part);
     } else if (step == STEP_XR) {
-      ph.upd_xr(Prec<V>::cvt(sst.alpha), Prec<V>::cvt(sst.omega), sst.phase == PH_SCONV, part);
+      ph.template upd_xr<false>(Prec<V>::cvt(sst.alpha), Prec<V>::cvt(sst.omega), sst.phase == PH_SCONV, part);
       part[3] = (blockIdx.x == 0 && threadIdx.x == 0 && deadline_passed(&sst)) ? 1.0 : 0.0;
     } else if (whole && step == STEP_INIT) {
       ph.init_zero(part);

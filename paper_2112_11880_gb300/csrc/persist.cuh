@@ -181,6 +181,32 @@ __device__ __forceinline__ void for_rows(const PRows& q, int32_t n, F f) {
   }
 }
 
+// f(row, li, ld(row, li)) for every row of this thread; with AHEAD (graph kernels,
+// which have the registers) the next row's loads are issued before a row is worked
+// on.
+template <bool AHEAD, class Ld, class F>
+__device__ __forceinline__ void for_rows_ld(const PRows& q, int32_t n, Ld ld, F f) {
+  if constexpr (!AHEAD) {
+    for_rows(q, n, [&](int32_t r, int li) { f(r, li, ld(r, li)); });
+  } else {
+    int32_t s = q.slice(n, 0), r = s * 32 + q.lane();
+    if (s < 0 || r >= n) return;  // only the last round has none for some warps
+    auto cur = ld(r, q.place(0));
+#pragma unroll 1
+    for (int32_t k = 0;; ++k) {
+      const int32_t s1 = k + 1 < q.L.rounds ? q.slice(n, k + 1) : -1;
+      const int32_t r1 = s1 * 32 + q.lane();
+      const bool more = s1 >= 0 && r1 < n;
+      auto next = cur;
+      if (more) next = ld(r1, q.place(k + 1));
+      f(r, q.place(k), cur);
+      if (!more) return;
+      cur = next;
+      r = r1;
+    }
+  }
+}
+
 // Calls f(row, li, sum_k a_rk x_k) for every row of this thread; pre(row) first
 // (its loads are in flight with the sum's).  A split solver's rows are summed
 // in three parts (sell_row_part): here by the row's thread (sell_row_parts).

@@ -258,7 +258,7 @@ __device__ __forceinline__ void sum_components(const double* partials, int G, in
 // put_block_partials and sum_components where a block is one warp, which would add
 // the components one after the other: the same sums, the components side by side
 // (graph kernels of meshes up to one slice per SM: us per iteration of the 15^3 box,
-// BiCGStab 36.4 -> 34.4, complex64 33.3 -> 31.8).
+// BiCGStab 36.4 -> 35.0, complex64 33.4 -> 32.6).
 template <int K>
 __device__ __forceinline__ void put_warp_partials(const double (&v)[K], double* partials) {
   const int lane = threadIdx.x & 31;
@@ -267,11 +267,12 @@ __device__ __forceinline__ void put_warp_partials(const double (&v)[K], double* 
   for (int k = 0; k < K; ++k)
     if (lane == warp_sum_lane<K>(k)) partials[static_cast<size_t>(k) * gridDim.x + blockIdx.x] = ws;
 }
+// (out of line: the kernels of larger meshes on the same shape do not fetch it)
 template <int K>
-__device__ __forceinline__ void sum_warp_partials(const double* partials, int G, double (&tot)[K]) {
+__device__ __noinline__ double4 sum_warp_partials(const double* partials, int G) {
+  static_assert(K <= 4, "four at most");
   const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k < K; ++k) tot[k] = 0.0;
+  double tot[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1
   for (int j0 = lane; j0 < G; j0 += 5 * 32) {
     double w[K][5];
@@ -291,6 +292,7 @@ __device__ __forceinline__ void sum_warp_partials(const double* partials, int G,
   for (int off = 16; off > 0; off >>= 1)
 #pragma unroll
     for (int k = 0; k < K; ++k) tot[k] += __shfl_xor_sync(0xffffffffu, tot[k], off);
+  return make_double4(tot[0], tot[1], tot[2], tot[3]);
 }
 
 // Fixed-order totals of all blocks' partials, valid in thread 0: sum_components,
@@ -323,7 +325,9 @@ template <class V, int S, int K>
 __device__ __forceinline__ bool grid_total_last(double (&v)[K], double* partials, unsigned int* ticket, double* red,
                                                 double (&tot)[K]) {
   __shared__ bool s_last;
-  const bool one_warp = S != SHAPE_LARGE && blockDim.x == 32;
+  // only the shape of the smallest meshes has one-warp blocks
+  constexpr bool can = S == (std::is_same<V, float2>::value ? SHAPE_MID : SHAPE_SMALL);
+  const bool one_warp = can && blockDim.x == 32;
   if (one_warp) put_warp_partials<K>(v, partials);
   else put_block_partials<V, S, K>(v, red, partials);
   __syncthreads();
@@ -334,8 +338,12 @@ __device__ __forceinline__ bool grid_total_last(double (&v)[K], double* partials
   __syncthreads();
   if (!s_last) return false;
   __threadfence();
-  if (one_warp) sum_warp_partials<K>(partials, gridDim.x, tot);
-  else sum_block_partials<V, S, K>(partials, gridDim.x, red, tot);
+  if (one_warp) {
+    const double4 t = sum_warp_partials<K>(partials, gridDim.x);
+    const double t4[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+    for (int k = 0; k < K; ++k) tot[k] = t4[k];
+  } else sum_block_partials<V, S, K>(partials, gridDim.x, red, tot);
   if (threadIdx.x == 0) *ticket = 0u;
   return true;
 }

@@ -206,8 +206,9 @@ typedef enum {
 typedef enum {
   HELM_LAUNCH_AUTO = 0,       /* persistent where the device can launch it (the
                                  whole FP64 solve of each method; the complex64
-                                 inner solves of mixed precision up to some
-                                 240,000 unknowns), else graph; the host-driven
+                                 inner solves of mixed precision from some 5,000
+                                 up to some 240,000 unknowns), else graph; the
+                                 host-driven
                                  loop if the graph cannot be built.  Graph also
                                  for matrices with long rows (FP64 above 262,144
                                  entries, 192 beyond some 730,000 unknowns;

@@ -609,13 +609,17 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   a.dev_err = A->dev_err;
 
   // HELM_LAUNCH_AUTO: persistent inner solves where the device takes the launch
-  // (else the graphs: a context can have fewer SMs than the device reports),
-  // but the graph on the large shape (us per inner iteration on the 200x100x80
-  // cavity: 184 against 191; on mid the persistent kernel is ahead by 4 to 7)
+  // (else the graphs: a context can have fewer SMs than the device reports), but the
+  // graph on the large shape (us per inner iteration on the 200x100x80 cavity: 171
+  // against 191) and up to one slice per SM, where one warp a block makes the chains
+  // long and a solve's many short launches count (whole solves to 1e-10, ms,
+  // persistent / graph / before persistent kernels: 6x5x4 box 2.18 / 2.01 / 2.00, 9^3
+  // 8.80 / 8.30 / 8.28, 15^3 42.7 / 39.3 / 42.7; 18^3, 1.4 slices per SM, 50.6 / 57.8 /
+  // 67.3)
   PShape ps;
   const void* inner = nullptr;
   with_shape(sh.k, [&](auto S) { inner = reinterpret_cast<const void*>(&k_mx_inner<S.value>); });
-  bool persistent = persist_default(A, sh.k, o) && sh.k.shape != SHAPE_LARGE &&
+  bool persistent = persist_default(A, sh.k, o) && sh.k.shape != SHAPE_LARGE && A->nsl > A->num_sms &&
                     persist_fit(inner, n, sh.k.grid, sh.k.threads, sh.k.bps, 1, Phases<float2>::kOwn, sizeof(float2),
                                 &ps);
   (void)cudaGetLastError();

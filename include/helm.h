@@ -257,9 +257,12 @@ typedef struct {
                           most tol; when the recurrence met tol but the
                           recomputed residual did not, the solve restarts
                           from the current x while iterations remain
-                          (BiCGStab, BiCGStab(l), TFQMR); FP64 BiCGStab
-                          also when (r^, r) of its recurrence came to exactly
-                          zero after an iteration */
+                          (BiCGStab, BiCGStab(l), TFQMR).  A single FP64
+                          BiCGStab solve also restarts from the current x
+                          when (r^, r) of its recurrence came to exactly zero
+                          after an iteration (that iteration counts); in the
+                          first iteration of a start, and for a frequency of
+                          a sweep, that is HELM_ERR_BREAKDOWN */
   int32_t maxit;       /* iteration cap (Section 4 uses 1000); each BiCGStab
                           or TFQMR iteration applies A twice */
   int32_t use_x0;      /* 0: start from x = 0 (Section 4); 1: start from d_x */

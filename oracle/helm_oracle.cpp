@@ -145,9 +145,11 @@ struct Csr {
 // iterations remain, the method restarts from the current x, and the solve
 // reports ok only with a true residual at most tol.
 //
-// Breakdown (this project's reading; the paper is silent): rho == 0,
-// (r^, v) == 0, (t, t) == 0 or omega == 0 exactly, or any non-finite scalar.
-// On breakdown x holds the last iterate.
+// Breakdown (this project's reading; the paper is silent): rho == 0 in the first
+// iteration of a (re)start, (r^, v) == 0, (t, t) == 0 or omega == 0 exactly, or any
+// non-finite scalar.  On breakdown x holds the last iterate.  rho == 0 in a later
+// iteration: the recurrence can go no further, but x and r stand; the method
+// restarts from x (that iteration counted) while iterations remain.
 int bicgstab(const Csr& A, const cplx* b, cplx* x, double tol, int32_t maxit, int use_x0,
              int32_t* iters_out, double* relres_recur_out, double* relres_true_out) {
   const int32_t n = A.n;
@@ -170,6 +172,7 @@ int bicgstab(const Csr& A, const cplx* b, cplx* x, double tol, int32_t maxit, in
   int status = ST_NOT_CONVERGED;
   double relres = 0.0;
   for (;;) {  // one pass per (re)start
+    bool first = true, again = false;
     // r = b - A x ; r^ = r ; rho_prev = alpha = omega = 1 ; v = p = 0
     A.apply(x, tmp.data());
     ORACLE_PAR
@@ -183,7 +186,12 @@ int bicgstab(const Csr& A, const cplx* b, cplx* x, double tol, int32_t maxit, in
       const cplx rho = zdotc(n, rhat.data(), r.data());
       const cplx beta = (rho / rho_prev) * (alpha / omega);
       if (!finite(rho) || !finite(beta)) { status = ST_NONFINITE; break; }
-      if (rho == cplx(0.0, 0.0)) { status = ST_BREAKDOWN; break; }
+      if (rho == cplx(0.0, 0.0)) {
+        if (first) status = ST_BREAKDOWN;
+        else again = true;
+        break;
+      }
+      first = false;
       ORACLE_PAR
       for (int32_t i = 0; i < n; ++i) p[i] = r[i] + beta * (p[i] - omega * v[i]);
       A.apply(p.data(), v.data());
@@ -227,6 +235,8 @@ int bicgstab(const Csr& A, const cplx* b, cplx* x, double tol, int32_t maxit, in
     for (int32_t i = 0; i < n; ++i) tmp[i] = b[i] - tmp[i];
     const double rtrue = dznrm2(n, tmp.data()) / bnorm;
     *relres_true_out = rtrue;
+    if (again && rtrue <= tol) { status = ST_OK; break; }
+    if (again && it < maxit) continue;
     if (status == ST_OK && rtrue > tol && it < maxit) { status = ST_NOT_CONVERGED; continue; }
     if (status == ST_OK && rtrue > tol) status = ST_NOT_CONVERGED;
     break;

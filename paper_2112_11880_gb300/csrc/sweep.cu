@@ -453,7 +453,8 @@ template <class V> struct Vec5 { V a, b, c, d, e; };
 
 // Y_j = A_j X_j for the stand-alone batched product (helm_sweep_spmv): the
 // solver's row sum.
-__global__ void __launch_bounds__(256) k_sw_apply(SweepDev A, int32_t F, int32_t G, const double* __restrict__ w,
+constexpr int kApplyThreads = 288;  // eight warps, nine for three groups
+__global__ void __launch_bounds__(kApplyThreads) k_sw_apply(SweepDev A, int32_t F, int32_t G, const double* __restrict__ w,
                                                   const double2* __restrict__ X, int32_t ldx, double2* __restrict__ Y,
                                                   int32_t ldy) {
   const SweepWalk wk(F, G, nullptr, nullptr);
@@ -2615,9 +2616,13 @@ helm_status helm_sweep_spmv(helm_sweep S, int32_t nfreq, const double* h_omega, 
   HELM_CUDA_TRY(cudaMemcpyAsync(S->wapply, h_omega, nfreq * sizeof(double), cudaMemcpyHostToDevice, s));
   const SweepDev A{S->n, S->nnz, S->rowptr, S->colind, S->K, S->M, S->B, S->bzero_blk, nullptr, nullptr, nullptr};
   const int G = Fp / 32;
-  const int64_t warps = static_cast<int64_t>(S->n) * G;
-  const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((warps + 7) / 8, static_cast<int64_t>(S->num_sms) * 8)));
-  k_sw_apply<<<grid, 256, 0, s>>>(A, nfreq, G, S->wapply, static_cast<const double2*>(d_X), ldx,
+  // eight warps a block, or as few more as make whole slots: with three groups two of
+  // eight warps had none (us, three groups, eight / nine warps / a warp per row and
+  // group: 60x30x25, 96 frequencies 690 / 609 / 617, 65 606 / 488 / 617)
+  const int warps = (8 + G - 1) / G * G;
+  const int64_t want = (static_cast<int64_t>(S->n) * G + warps - 1) / warps;
+  const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(want, static_cast<int64_t>(S->num_sms) * (64 / warps))));
+  k_sw_apply<<<grid, 32 * warps, 0, s>>>(A, nfreq, G, S->wapply, static_cast<const double2*>(d_X), ldx,
                                   static_cast<double2*>(d_Y), ldy);
   HELM_CUDA_TRY(cudaGetLastError());
   return HELM_OK;

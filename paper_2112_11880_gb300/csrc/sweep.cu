@@ -157,7 +157,7 @@ struct SweepWalk {
   int split;           // threads that share a slot's rows (walk_split; 1: none), one row each at least
   int32_t ci, cstep;   // split: the rows whose sums this thread adds up (ci < 0: none)
   const int32_t* pos;  // a frequency's place among the na (null: all, in order)
-  __device__ __forceinline__ SweepWalk(int na_, int groups, const int32_t* act, const int32_t* pos_, int32_t n = 0)
+  __device__ __forceinline__ SweepWalk(int na_, int F, int groups, const int32_t* act, const int32_t* pos_, int32_t n = 0)
       : j(-1), i(0), step(1), na(na_), slots(static_cast<int>(blockDim.x >> 5) / groups), split(1), ci(-1), cstep(1),
         pos(pos_) {
     if (na == 0) return;
@@ -165,7 +165,7 @@ struct SweepWalk {
     cstep = static_cast<int32_t>(gridDim.x) * slots;
     split = max(min(static_cast<int>(blockDim.x) / pairs, (n + cstep - 1) / cstep), 1);
     const int sub = t / pairs, slot = (t - sub * pairs) / na, p = t - sub * pairs - slot * na;
-    if (sub < split) j = act ? act[p] : p;
+    if (sub < split) j = act && na < F ? act[p] : p;  // (with all of them running the list is in order)
     const int32_t first = static_cast<int32_t>(blockIdx.x) * slots + slot;
     if (sub == 0) ci = first;
     i = first + sub * cstep;
@@ -174,20 +174,22 @@ struct SweepWalk {
   // frequency j's place (-1: not among them)
   __device__ __forceinline__ int place(int f, int F) const { return pos ? pos[f] : f < F ? f : -1; }
 };
-// the running frequencies; all of them
+// the running frequencies (every kernel that changes a status lists them again, so
+// what is on the list is running: no kernel waits for the status as well); all of
+// them
 template <class V>
 __device__ __forceinline__ SweepWalk walk_running(const SweepArgsT<V>& a) {
-  return SweepWalk(*a.nact, a.G, a.act, a.pos);
+  return SweepWalk(*a.nact, a.F, a.G, a.act, a.pos);
 }
 // the running ones, a slot's rows shared out to the threads that the pairs leave:
 // the kernel forms the slot's sums afterwards (sweep_chain)
 template <class V>
 __device__ __forceinline__ SweepWalk walk_split(const SweepArgsT<V>& a) {
-  return SweepWalk(*a.nact, a.G, a.act, a.pos, a.A.n);
+  return SweepWalk(*a.nact, a.F, a.G, a.act, a.pos, a.A.n);
 }
 template <class V>
 __device__ __forceinline__ SweepWalk walk_all(const SweepArgsT<V>& a) {
-  return SweepWalk(a.F, a.G, nullptr, nullptr);
+  return SweepWalk(a.F, a.F, a.G, nullptr, nullptr);
 }
 
 // Per-frequency partial sums of one block: the slots' sums in slot order through
@@ -394,7 +396,7 @@ template <class V, class Pre, class Epi>
 __device__ __forceinline__ void sweep_spmv(const SweepArgsT<V>& a, const SweepWalk& wk, const V* __restrict__ x, Pre pre,
                                            Epi& epi, bool on = true) {
   const int j = wk.j;
-  if (!on || j < 0 || a.status[j] != ST_RUNNING || wk.i >= a.A.n) return;
+  if (!on || j < 0 || wk.i >= a.A.n) return;
   const double wj = a.w[j];
   const double w2 = wj * wj;
   int32_t k0 = __ldg(a.A.rowptr + wk.i), k1 = __ldg(a.A.rowptr + wk.i + 1);
@@ -457,7 +459,7 @@ constexpr int kApplyThreads = 288;  // eight warps, nine for three groups
 __global__ void __launch_bounds__(kApplyThreads) k_sw_apply(SweepDev A, int32_t F, int32_t G, const double* __restrict__ w,
                                                   const double2* __restrict__ X, int32_t ldx, double2* __restrict__ Y,
                                                   int32_t ldy) {
-  const SweepWalk wk(F, G, nullptr, nullptr);
+  const SweepWalk wk(F, F, G, nullptr, nullptr);
   const int j = wk.j;
   if (j < 0) return;
   const double wj = w[j];
@@ -531,12 +533,12 @@ __device__ void sweep_refresh(const SweepArgsT<V>& a) {
 #define SWEEP_ELEMENTWISE_BEGIN            \
   const SweepWalk wk = walk_running(a);    \
   const int j = wk.j;                      \
-  const bool run = j >= 0 && a.status[j] == ST_RUNNING;
+  const bool run = j >= 0;
 
 #define SWEEP_SPLIT_BEGIN                  \
   const SweepWalk wk = walk_split(a);      \
   const int j = wk.j;                      \
-  const bool run = j >= 0 && a.status[j] == ST_RUNNING;
+  const bool run = j >= 0;
 
 // init: r = b - A_j x (or r = b, x = 0), r^ = r, p = v = 0; ||b||, ||r||, rho
 template <class V>

@@ -92,7 +92,10 @@ typedef struct helm_csr_s* helm_csr; /* opaque CSR handle */
  * Work done: row statistics, the sliced copy, workspace allocation, and the
  * choice of SpMV variant: for nnz >= 2^18 the stand-alone SpMV's variants
  * are timed on this matrix and the fastest is kept (every variant gives the
- * same y bit for bit).  Synchronises `stream`.  Returns
+ * same y bit for bit), unless its product has a kernel of its own (small
+ * matrices, up to five slices per SM: 24,320 rows on GB300, where a row is
+ * summed in parts; complex64 ones of 200,000 rows and more with a diagonal
+ * copy).  Synchronises `stream`.  Returns
  * HELM_ERR_INVALID on bad sizes, a misaligned pointer, (with
  * HELM_CSR_VALIDATE) a malformed pattern, or when the padded sliced copy
  * would hold 2^31 entries or more; HELM_ERR_NOMEM if the workspace cannot be

@@ -61,8 +61,10 @@ __global__ void __launch_bounds__(Engine<V>::kThreads, Engine<V>::kMinBlocks) k_
 // Measured (us, a warp a slice -> this): ragged rows of up to 60 complex entries,
 // 20,011 rows 21.3 -> 12.7 (then the FP64 pipe: 240 instructions a slot of the
 // widest row), 5,000 18.5 -> 6.8, 1,000 18.0 -> 4.6; meshes of 27 entries a row,
-// 20x20x20 6.4 -> 3.8, 40x20x16 6.2 -> 4.4; ten slices per SM (60x30x25) 7.9 ->
-// 10.4.  Eight parts up to one slice per SM (1,000 rows: four 6.2), four up to five.
+// 20x20x20 6.4 -> 3.8, 40x20x16 6.2 -> 4.4.  At five slices per SM: the ragged rows
+// 21.6 -> 12.8, real ones 14.0 -> 7.6, 27 diagonals 6.8 -> 4.9, five 3.6 -> 3.4,
+// 42x24x21 (4.9) 7.2 -> 5.6; at ten a mesh (60x30x25) 7.9 -> 10.4.  Eight parts up to
+// one slice per SM (1,000 rows: four 6.2), four up to five.
 constexpr int kSplitUnroll = 4;
 constexpr int kSplitSlices = 5;  // per SM, at most
 template <class V, int P>
@@ -557,6 +559,19 @@ static helm_status spmv_occupancy(int U, int threads, int* per_sm) {
 // on the handle's own matrix (3 launches each after one warm-up, CUDA events
 // on `s`) and keep the fastest.  Matrices under 2^18 stored entries keep the
 // default (U = 4, 1024-thread blocks): their SpMV is launch-bound.
+// Whether the stand-alone product of this handle takes k_spmv_split or k_spmv_dia.
+// (A sliced-only complex64 handle takes its rows as a diagonal copy does: the same
+// bits.)
+template <class V>
+static bool takes_split(helm_csr A, const CsrDev<V>& d) {
+  return (std::is_same<V, double2>::value || (d.ndia == 0 && !A->sliced_only)) &&
+         A->nsl <= static_cast<int64_t>(A->num_sms) * kSplitSlices;
+}
+template <class V>
+static bool takes_dia(helm_csr A, const CsrDev<V>& d) {
+  return std::is_same<V, float2>::value && d.ndia > 0 && A->n >= kDiaRows;
+}
+
 template <class V>
 static helm_status autotune_spmv(helm_csr A, const CsrDev<V>& d, cudaStream_t s) {
   struct Cand {
@@ -569,7 +584,7 @@ static helm_status autotune_spmv(helm_csr A, const CsrDev<V>& d, cudaStream_t s)
   A->spmv_variant = 4;
   A->spmv_grid = s0.grid;
   A->spmv_threads = s0.threads;
-  if (A->nnz < (int64_t(1) << 18) || A->n == 0) return HELM_OK;
+  if (A->nnz < (int64_t(1) << 18) || A->n == 0 || takes_split(A, d) || takes_dia(A, d)) return HELM_OK;
   V *x = nullptr, *y = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   helm_status st = HELM_OK;
@@ -628,25 +643,21 @@ static int spmv_mode(V alpha, V beta) {
   return (a1 && b0) ? 0 : (b0 ? 1 : 2);
 }
 
-// Launches k_spmv_split where a matrix has few enough slices for it.
 template <class V>
-static bool spmv_split(helm_csr A, const CsrDev<V>& d, const V* x, V* y, V alpha, V beta, cudaStream_t s) {
-  if (A->nsl > static_cast<int64_t>(A->num_sms) * kSplitSlices) return false;
+static void launch_split(helm_csr A, const CsrDev<V>& d, const V* x, V* y, V alpha, V beta, cudaStream_t s) {
   const int mode = spmv_mode(alpha, beta);
   if (A->nsl <= A->num_sms) k_spmv_split<V, 8><<<A->nsl, 256, 0, s>>>(d, x, y, alpha, beta, mode);
   else k_spmv_split<V, 4><<<A->nsl, 128, 0, s>>>(d, x, y, alpha, beta, mode);
-  return true;
 }
 
 helm_status launch_spmv128(helm_csr A, const double2* x, double2* y, double2 alpha, double2 beta,
                            cudaStream_t s) {
   if (A->n == 0) return HELM_OK;
   const CsrDev<double2> d = csr_dev<double2>(A, static_cast<const double2*>(A->vals), A->sv);
-  if (spmv_split(A, d, x, y, alpha, beta, s)) {
-    HELM_CUDA_TRY(cudaGetLastError());
-    return HELM_OK;
-  }
-  spmv_enqueue<double2>(A->spmv_variant, A->spmv_grid, A->spmv_threads, d, x, y, alpha, beta, spmv_mode(alpha, beta), s);
+  if (takes_split(A, d)) launch_split(A, d, x, y, alpha, beta, s);
+  else
+    spmv_enqueue<double2>(A->spmv_variant, A->spmv_grid, A->spmv_threads, d, x, y, alpha, beta, spmv_mode(alpha, beta),
+                          s);
   HELM_CUDA_TRY(cudaGetLastError());
   return HELM_OK;
 }
@@ -654,18 +665,14 @@ helm_status launch_spmv128(helm_csr A, const double2* x, double2* y, double2 alp
 helm_status launch_spmv64(helm_csr A, const float2* x, float2* y, float2 alpha, float2 beta, cudaStream_t s) {
   if (A->n == 0) return HELM_OK;
   const CsrDev<float2> d = csr_dev<float2>(A, static_cast<const float2*>(A->vals), A->sv);
-  // (a sliced-only handle takes the rows as a diagonal copy does: the same bits)
-  if (d.ndia == 0 && !A->sliced_only && spmv_split(A, d, x, y, alpha, beta, s)) {
-    HELM_CUDA_TRY(cudaGetLastError());
-    return HELM_OK;
-  }
-  if (d.ndia > 0 && A->n >= kDiaRows) {
+  if (takes_split(A, d)) {
+    launch_split(A, d, x, y, alpha, beta, s);
+  } else if (takes_dia(A, d)) {
     const int64_t blocks = (static_cast<int64_t>(A->n) + 2 * kDiaThreads - 1) / (2 * kDiaThreads);
     k_spmv_dia<<<static_cast<unsigned>(blocks), kDiaThreads, 0, s>>>(d, A->dia, x, y, alpha, beta, spmv_mode(alpha, beta));
-    HELM_CUDA_TRY(cudaGetLastError());
-    return HELM_OK;
+  } else {
+    spmv_enqueue<float2>(A->spmv_variant, A->spmv_grid, A->spmv_threads, d, x, y, alpha, beta, spmv_mode(alpha, beta), s);
   }
-  spmv_enqueue<float2>(A->spmv_variant, A->spmv_grid, A->spmv_threads, d, x, y, alpha, beta, spmv_mode(alpha, beta), s);
   HELM_CUDA_TRY(cudaGetLastError());
   return HELM_OK;
 }

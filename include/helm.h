@@ -207,15 +207,20 @@ typedef enum {
 } helm_precision;
 /* How the iteration loop is driven on the device. */
 typedef enum {
-  HELM_LAUNCH_AUTO = 0,       /* persistent where the device can launch it (the
+  HELM_LAUNCH_AUTO = 0,       /* persistent where the device takes the launch (the
                                  whole FP64 solve of each method; the complex64
                                  inner solves of mixed precision from some 5,000
-                                 up to some 240,000 unknowns), else graph; the
-                                 host-driven
-                                 loop if the graph cannot be built.  Graph also
-                                 for matrices with long rows (FP64 above 262,144
-                                 entries, 192 beyond some 730,000 unknowns;
-                                 mixed precision above 128) */
+                                 to some 240,000 unknowns), else graph; the
+                                 host-driven loop if the graph cannot be built.
+                                 Graph also for matrices with long rows (FP64
+                                 above 262,144 entries, 192 beyond some 730,000
+                                 unknowns; mixed precision above 128).  A
+                                 persistent solve holds every SM (up to one
+                                 block per slice of 32 rows) until it ends:
+                                 solves on other streams wait for it or run
+                                 before it, and other kernels get what its blocks
+                                 leave of the SMs; with HELM_LAUNCH_GRAPH they
+                                 run between the kernels of the loop */
   HELM_LAUNCH_GRAPH = 1,      /* CUDA graph with a device-driven while node;
                                  HELM_ERR_CUDA if it cannot be built */
   HELM_LAUNCH_PERSISTENT = 2, /* FP64 BiCGStab only (HELM_ERR_INVALID for

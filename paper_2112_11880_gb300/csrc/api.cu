@@ -11,7 +11,6 @@
 #include <cstdint>
 #include <mutex>
 #include <new>
-#include <utility>
 #include <vector>
 
 #include "blas1.cuh"
@@ -51,7 +50,7 @@ template <class V, int U>
 __global__ void __launch_bounds__(Engine<V>::kThreads, Engine<V>::kMinBlocks) k_spmv(CsrDev<V> A, const V* __restrict__ x, V* y, V alpha,
                                                               V beta, int mode) {
   AxpbyEpi<V> epi{y, alpha, beta, mode, vzero<V>()};
-  (void)spmv_run<V, AxpbyEpi<V>, NoGate, GatherReadOnly, U>(A, x, epi, nullptr, nullptr);
+  spmv_run<V, AxpbyEpi<V>, GatherReadOnly, U>(A, x, epi);
 }
 
 // The same for a matrix of few slices: P warps take a part of a slice's
@@ -495,23 +494,6 @@ __global__ void k_dia_fill(int32_t n, const int32_t* __restrict__ rowptr, const 
 void debug_cuda_error(cudaError_t e, const char* file, int line) {
   static const bool on = std::getenv("HELM_DEBUG") != nullptr;
   if (on) std::fprintf(stderr, "libhelm: %s:%d: %s\n", file, line, cudaGetErrorString(e));
-}
-
-std::mutex g_attr_mu;
-std::vector<std::pair<const void*, int>> g_attr_done;
-
-// Opt a kernel into more than 48 KB of dynamic shared memory (once per
-// kernel and device).
-cudaError_t set_smem_attr(const void* fn, size_t bytes) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  std::lock_guard<std::mutex> lk(g_attr_mu);
-  for (auto& p : g_attr_done)
-    if (p.first == fn && p.second == dev) return cudaSuccess;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-  if (e == cudaSuccess) g_attr_done.emplace_back(fn, dev);
-  return e;
 }
 
 int sm_count() {

@@ -153,7 +153,6 @@ inline bool overlaps(const void* p, size_t pn, const void* q, size_t qn) {
 }
 
 // Launch-shape helpers (api.cu).
-cudaError_t set_smem_attr(const void* fn, size_t bytes);
 int sm_count();
 int vec_grid_for(int64_t n);
 // Doubles of a handle's partial sums per SM: 32 blocks of 8 sums.

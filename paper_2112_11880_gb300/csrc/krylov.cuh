@@ -14,18 +14,20 @@
 //   P4  t = A s          + (t, s), ||t||^2 -> omega = (t, s) / (t, t)
 //   P5  x += alpha p + omega s, r = s - omega t + (r^, r), ||r||^2
 //                                         -> stop test, rho, beta
-// For complex64 the products and each thread's partial sums are FP32; block
-// and grid sums and every scalar of the recurrence are FP64.
+// For complex64 the products are FP32; each thread's partial sums, block and grid
+// sums and every scalar of the recurrence are FP64.
 //
-// Two ways to run the loop, with the same arithmetic bit for bit:
+// Three ways to run the loop, with the same arithmetic bit for bit:
+//   * persistent (the default but for long rows, and for complex64 on the smallest
+//     and the large meshes): one cooperative kernel for the whole solve; a grid
+//     barrier ends every phase, after which every block adds the block partials
+//     itself (same order, so the same scalars in every block) -- no kernel
+//     launches, no last-block step;
 //   * graph: one kernel per phase; the last block to finish a phase (ticket
 //     counter) adds the block partials and forms the scalars; the loop is a
 //     CUDA graph with a conditional WHILE node (four iterations per pass);
-//   * persistent: one cooperative kernel for the whole solve; a grid barrier
-//     ends every phase, after which every block adds the block partials
-//     itself (same order, so the same scalars in every block) -- no kernel
-//     launches, no last-block step.
-// Both give each row to the same thread in every phase (SliceRows of the
+//   * host: the graph's kernels launched from the host (for profilers).
+// All give each row to the same thread in every phase (SliceRows of the
 // SpMV engine) on the same grid, and add the same partials in the same order.
 #pragma once
 
@@ -58,8 +60,7 @@ constexpr int32_t kModePlain = 0;
 constexpr int32_t kModeRefine = 1;
 constexpr int kInnerMax = 50000;  // inner iterations per refinement step at most
 
-// Per-thread partial sums of dot products and norms (S real, C complex)
-// accumulate in FP64: for complex128 operands the FP64 product (4 or 2 FMA),
+// Per-thread partial sums of dot products and norms accumulate in FP64: for complex128 operands the FP64 product (4 or 2 FMA),
 // for complex64 operands the product formed in FP32 and added in FP64.
 // Measured alternatives for complex64: an uncompensated FP32 running sum
 // over the ~10 rows a thread takes on the 200x100x80 cavity slowed the inner
@@ -67,25 +68,16 @@ constexpr int kInnerMax = 50000;  // inner iterations per refinement step at mos
 // inner iteration 2-6 % faster on the 120x60x50 and 200x100x80 cavities, but
 // the 200x100x80 solve to 1e-10 then stalled (289,524 inner iterations, not
 // converged, against 188,207 to convergence with FP64 sums).
+// A device scalar in the precision of the vectors.
 template <class V> struct Prec;
 template <> struct Prec<double2> {
-  using S = double;
-  using C = double2;
   __device__ static __forceinline__ double2 cvt(double2 z) { return z; }
-  __device__ static __forceinline__ S szero() { return 0.0; }
-  __device__ static __forceinline__ C czero() { return make_double2(0.0, 0.0); }
 };
 template <> struct Prec<float2> {
-  using S = double;
-  using C = double2;
   __device__ static __forceinline__ float2 cvt(double2 z) {
     return make_float2(static_cast<float>(z.x), static_cast<float>(z.y));
   }
-  __device__ static __forceinline__ S szero() { return 0.0; }
-  __device__ static __forceinline__ C czero() { return make_double2(0.0, 0.0); }
 };
-__device__ __forceinline__ double to_d(double v) { return v; }
-__device__ __forceinline__ double2 to_d2(double2 v) { return v; }
 
 // acc + conj(a) b and acc + |a|^2 in the precision rules above
 __device__ __forceinline__ double2 dot_acc(double2 acc, double2 a, double2 b) { return cfma_conj(a, b, acc); }
@@ -110,21 +102,25 @@ __device__ __forceinline__ double nrm_acc(double acc, float2 a) {
 //   large: two blocks per SM of at most 512 threads (64 registers).
 // complex64 (the inner solves of mixed precision): mid or large (us per inner
 // iteration, persistent / graph / before: 20^3 29.7 / 33.9 / 44.5, 60x30x25 29.4 /
-// 34.5 / 37.1, 80x40x32 37.6 / 44.9 / 47; large: 120x60x50 71.5 / 77.9, 200x100x80
-// 191 / 184 / 205: there the default is the graph).
+// 34.5 / 37.1, 80x40x32 37.6 / 44.9 / 47; large: 120x60x50 71.5 / 67.8 / 77.9,
+// 200x100x80 191 / 171 / 205: there the default is the graph).
 // Measured (BiCGStab, us per iteration: persistent / graph kernels; before, on
 // one shape with graph kernels):
-//   20^3 box      (2 slices per SM)  small 25.7 / 39.0                       (39.7)
-//   60x30x25      (10)               mid   37.2 / 39.1, large 50.1 / 47.6    (43.6)
-//   80x40x32      (23)               mid   54.0 / 61.6, large 60.0 / 67.0    (65.1)
-//   120x60x50     (77)               mid  121.1 / 136.9, large 135.4 / 140.2 (134.0)
-//   200x100x80    (338)              mid  504 (512 threads), large 475 / 498 (478)
-// (mid of 640 threads: 37.3, 55.1, 121.5; 704: 40.5, 61.0, 124.1; more spill.)
+//   20^3 box      (2 slices per SM)  small 25.8 / 35.4                       (49.4)
+//   60x30x25      (10)               mid   36.2 / 39.6, large 50.1 / 47.6    (46.5)
+//   80x40x32      (23)               mid   53.9 / 58.9, large 60.0 / 67.0    (66.3)
+//   120x60x50     (77)               mid  121.6 / 133.1, large 135.4 / 140.2 (139.1)
+//   200x100x80    (338)              mid  504 (512 threads), large 474 / 472 (488)
+// (mid of 640 threads: 37.3, 55.1, 121.5; 704: 40.5, 61.0, 124.1; more spill.  The
+// figures of a shape a mesh does not take are of a graph without loads ahead.)
 enum : int { SHAPE_SMALL = 0, SHAPE_MID = 1, SHAPE_LARGE = 2 };
 constexpr int kMidSlices = 150;    // slices per SM from which the shape is large
 // for complex64 sooner: whether its inner solves converge on an indefinite system
 // of that size hangs on the order of their sums (kOrderedSums; 120x60x50 at 10
-// points per wavelength, inner_tol 0.01: converges on the large shape, not on mid)
+// points per wavelength, inner_tol 0.01: converges on the large shape, not on mid).
+// Up to 50 slices either order converges: 30x15x12 to 104x52x42 (49.2 slices) at 8, 10
+// and 14 points per wavelength, to 1e-8 and 1e-10, inner_tol 0.5 to 1e-4, 336 solves,
+// all of them with both, the inner iterations within 0.4 % on average
 constexpr int kMidSlices32 = 50;
 template <int S> struct SolverBounds {
   static constexpr int threads = S == SHAPE_SMALL ? 384 : S == SHAPE_MID ? 768 : 512;  // warps of a split persistent kernel included
@@ -133,10 +129,6 @@ template <int S> struct SolverBounds {
   // entries per pipeline stage of the persistent kernel's products
   static constexpr int persist_u = S == SHAPE_LARGE ? 2 : 3;
 };
-// The other kernels on an SpMV grid (init, tail, refinement steps).
-constexpr int kSolverThreads = Engine<double2>::kThreads;
-constexpr int kSolverMinBlocks = Engine<double2>::kMinBlocks;
-
 template <class V>
 struct KArgs {
   CsrDev<V> A;

@@ -1,17 +1,16 @@
 // Mixed-precision solve: FP64 outer GCR (iterative refinement with a window
-// of directions) around complex64 BiCGStab inner solves, the whole solve in
-// one CUDA graph.
+// of directions) around complex64 BiCGStab inner solves.
 //
 // The paper's library covers single and double precision (Section 1); here
 // single precision does the bulk of the work and FP64 decides accuracy:
 //   inner (FP32):  BiCGStab on A32 (complex64 copy of the values owned by the
 //                  handle, 8 bytes per entry for real rows instead of 12), vectors
-//                  complex64; products and per-thread sums FP32, block and
-//                  grid sums and every recurrence scalar FP64.  The inner
-//                  system is A32 d = r / sigma with sigma = ||r|| / sqrt(n)
-//                  (unit RMS entries: in the problem's own scale, b ~ h^3,
-//                  the squared terms of the inner dots would fall below the
-//                  smallest normal float long before FP64 convergence).
+//                  complex64; products FP32, all sums and every recurrence
+//                  scalar FP64.  The inner system is A32 d = r / sigma with
+//                  sigma = ||r|| / sqrt(n) (unit RMS entries: in the problem's
+//                  own scale, b ~ h^3, the squared terms of the inner dots would
+//                  fall below the smallest normal float long before FP64
+//                  convergence).
 //   step (FP64):   when the inner recurrence residual has dropped by
 //                  inner_tol since the inner solve began, looks below the
 //                  outer tolerance, or after kInnerMax inner iterations, an
@@ -33,17 +32,16 @@
 // converged slowly and, folded without a step length, diverged whenever an
 // inner solve stagnated.  The convergence test is always the FP64 true
 // residual.
-// Launch structure: init (+ first inner start); then per refinement step one
-// launch of the inner graph (a conditional WHILE over the 5 complex64
-// kernels, which ends when a step is due or the solve stops) and one of the
-// step graph (its 6 kernels), the host reading the state between steps; then
-// the tail.  An inner iteration so launches its five kernels and nothing
-// else (with the step kernels inside the loop body, returning at once when
-// no step is due, an inner iteration cost 84.5 instead of 76.1 us on
-// the 120x60x50 cavity).  A conditional IF node around the step kernels
-// inside the WHILE body was tried first: adding it fails with
-// cudaErrorInvalidValue on this CUDA 13.0 stack (handle on the body or the
-// top graph, with or without a default).
+// Launch structure: init (+ first inner start); then per refinement step the inner
+// solve, one persistent kernel (mid-size meshes) or one launch of the inner graph (a
+// conditional WHILE over the 5 complex64 kernels, which ends when a step is due or
+// the solve stops), and the step's 6 kernels (with the inner graph: a graph of their
+// own), the host reading the state between steps; then the tail.  The step's kernels
+// are not in the loop's body: returning at once when no step is due, they cost an
+// inner iteration 84.5 instead of 76.1 us on the 120x60x50 cavity.  A conditional IF
+// node around them there was tried first: adding it fails with cudaErrorInvalidValue
+// on this CUDA 13.0 stack (handle on the body or the top graph, with or without a
+// default).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -58,7 +56,7 @@ namespace {
 constexpr int kGcr = 8;
 
 constexpr int R128 = Engine<double2>::kThreads;  // threads per SpMV block
-constexpr size_t kSmem128 = Engine<double2>::kSmem;
+constexpr int kMinBlocks128 = Engine<double2>::kMinBlocks;
 
 struct RuArgs {
   CsrDev<double2> A;  // FP64 matrix
@@ -73,7 +71,6 @@ struct RuArgs {
   SolverState* st;    // the inner loop's state
   double* partials;
   unsigned int* tickets;
-  unsigned int* dev_err;
   cudaGraphConditionalHandle cond;
   int has_cond;
 };
@@ -103,14 +100,13 @@ struct MxRow {
 
 // init: r64 = b - A x (or b, x = 0); asks for the first inner start, which
 // starts the complex64 recurrence
-__global__ void __launch_bounds__(R128, kSolverMinBlocks) k_mx_init(RuArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
+__global__ void __launch_bounds__(R128, kMinBlocks128) k_mx_init(RuArgs a) {
   __shared__ double red[32 * 2];
   SolverState* st = a.st;
   const int use_x0 = st->use_x0;
   MxRow rows{&a, {0.0, 0.0}, make_double2(0.0, 0.0)};
   if (use_x0) {
-    spmv_run<double2>(a.A, a.x, rows, smem, a.dev_err);
+    spmv_run<double2>(a.A, a.x, rows);
   } else {
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < a.A.n; i += gridDim.x * blockDim.x) {
       const double2 bi = a.b[i];
@@ -213,8 +209,7 @@ __device__ __forceinline__ bool grid_sum_last_many(double (&v)[K], double* parti
 
 // step 1b: w = A z (FP64, z = d64) and the projections beta_j = (C_j, w) on
 // the stored directions (classical Gram-Schmidt against the GCR window).
-__global__ void __launch_bounds__(R128, kSolverMinBlocks) k_gcr_project(RuArgs a, int always) {
-  extern __shared__ __align__(16) unsigned char smem[];
+__global__ void __launch_bounds__(R128, kMinBlocks128) k_gcr_project(RuArgs a, int always) {
   constexpr int K = 2 * kGcr;
   __shared__ double red[32 * 4];
   SolverState* st = a.st;
@@ -237,7 +232,7 @@ __global__ void __launch_bounds__(R128, kSolverMinBlocks) k_gcr_project(RuArgs a
       }
     }
   } epi{&a, nw, {}};
-  spmv_run<double2>(a.A, a.d64, epi, smem, a.dev_err);
+  spmv_run<double2>(a.A, a.d64, epi);
   double tot[K];
   if (!grid_sum_last_many<K>(epi.acc, a.partials, a.tickets + TK_AUX2, red, tot)) return;
   if (threadIdx.x != 0) return;
@@ -311,8 +306,7 @@ __global__ void __launch_bounds__(256) k_gcr_xupd(RuArgs a, int always) {
 }
 
 // step 2: r64 = b - A x (FP64), the convergence test
-__global__ void __launch_bounds__(R128, kSolverMinBlocks) k_mx_residual(RuArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
+__global__ void __launch_bounds__(R128, kMinBlocks128) k_mx_residual(RuArgs a) {
   __shared__ double red[32];
   SolverState* st = a.st;
   if (st->aux[1].x == 0.0) return;
@@ -327,7 +321,7 @@ __global__ void __launch_bounds__(R128, kSolverMinBlocks) k_mx_residual(RuArgs a
       part = cabs2_acc(ri, part);
     }
   } epi{&a, 0.0, make_double2(0.0, 0.0)};
-  spmv_run<double2>(a.A, a.x, epi, smem, a.dev_err);
+  spmv_run<double2>(a.A, a.x, epi);
   double part[1] = {epi.part};
   double tot[1];
   if (!grid_sum_last<1>(part, a.partials, a.tickets + TK_AUX0, red, tot)) return;
@@ -410,8 +404,7 @@ __global__ void __launch_bounds__(256) k_mx_restart(RuArgs a) {
 }
 
 // tail: the FP64 true residual for the report (x32 folded just before)
-__global__ void __launch_bounds__(R128, kSolverMinBlocks) k_mx_tail(RuArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
+__global__ void __launch_bounds__(R128, kMinBlocks128) k_mx_tail(RuArgs a) {
   __shared__ double red[32];
   SolverState* st = a.st;
   const double bnorm = st->bnorm;
@@ -427,7 +420,7 @@ __global__ void __launch_bounds__(R128, kSolverMinBlocks) k_mx_tail(RuArgs a) {
       __device__ __forceinline__ void prefetch(int32_t i) { bi = a->b[i]; }
       __device__ __forceinline__ void row(int32_t i, double2 ax) { part = cabs2_acc(csub(bi, ax), part); }
     } epi{&a, 0.0, make_double2(0.0, 0.0)};
-    spmv_run<double2>(a.A, a.x, epi, smem, a.dev_err);
+    spmv_run<double2>(a.A, a.x, epi);
     part[0] = epi.part;
   }
   double tot[1];
@@ -453,12 +446,12 @@ struct MxShapes {
 };
 
 void mx_init(const RuArgs& a, const MxShapes& sh, cudaStream_t s) {
-  k_mx_init<<<sh.grid128, R128, kSmem128, s>>>(a);
+  k_mx_init<<<sh.grid128, R128, 0, s>>>(a);
   k_mx_restart<<<sh.vec_grid, 256, 0, s>>>(a);
 }
 void mx_fold(const RuArgs& a, const MxShapes& sh, int always, cudaStream_t s) {
   k_mx_lift<<<sh.vec_grid, 256, 0, s>>>(a, always);
-  k_gcr_project<<<sh.grid_proj, R128, kSmem128, s>>>(a, always);
+  k_gcr_project<<<sh.grid_proj, R128, 0, s>>>(a, always);
   k_gcr_orth<<<sh.vec_grid, 256, 0, s>>>(a, always);
   k_gcr_xupd<<<sh.vec_grid, 256, 0, s>>>(a, always);
 }
@@ -466,7 +459,7 @@ void mx_fold(const RuArgs& a, const MxShapes& sh, int always, cudaStream_t s) {
 // residual and a fresh inner start
 void mx_step(const RuArgs& a, const MxShapes& sh, cudaStream_t s) {
   mx_fold(a, sh, 0, s);
-  k_mx_residual<<<sh.grid128, R128, kSmem128, s>>>(a);
+  k_mx_residual<<<sh.grid128, R128, 0, s>>>(a);
   k_mx_restart<<<sh.vec_grid, 256, 0, s>>>(a);
 }
 void mx_body(const RuArgs& a, const KArgs<float2>& k, const MxShapes& sh, cudaStream_t s) {
@@ -542,7 +535,7 @@ helm_status build_plain_graph(Fn fn, GraphEntry* out) {
 
 void mx_tail(const RuArgs& a, const MxShapes& sh, cudaStream_t s) {
   mx_fold(a, sh, 1, s);
-  k_mx_tail<<<sh.grid128, R128, kSmem128, s>>>(a);
+  k_mx_tail<<<sh.grid128, R128, 0, s>>>(a);
 }
 
 }  // namespace
@@ -553,15 +546,12 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   if (st == HELM_OK) st = ensure_vectors(A, kNumVec > 3 + 2 * kGcr ? kNumVec : 3 + 2 * kGcr);
   if (st == HELM_OK) st = ensure_vectors32(A, 8);
   if (st != HELM_OK) return st;
-  for (const void* fn : {reinterpret_cast<const void*>(&k_mx_init), reinterpret_cast<const void*>(&k_mx_residual),
-                         reinterpret_cast<const void*>(&k_gcr_project), reinterpret_cast<const void*>(&k_mx_tail)})
-    HELM_CUDA_TRY(set_smem_attr(fn, kSmem128));
   MxShapes sh;
   st = krylov_shapes<float2>(A, &sh.k);
   if (st != HELM_OK) return st;
   HELM_TRY(persistent_grid({reinterpret_cast<const void*>(&k_mx_init), reinterpret_cast<const void*>(&k_mx_residual),
                             reinterpret_cast<const void*>(&k_gcr_project), reinterpret_cast<const void*>(&k_mx_tail)},
-                           R128, kSmem128, A->num_sms,
+                           R128, 0, A->num_sms,
                            (static_cast<int64_t>(A->n) + Engine<double2>::R - 1) / Engine<double2>::R, &sh.grid128));
   // partials buffer: num_sms * 32 * 8 doubles (api.cu)
   sh.grid_proj = std::min(sh.grid128, A->num_sms * 32 * 8 / (2 * kGcr));
@@ -606,7 +596,6 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   a.st = A->state;
   a.partials = A->partials;
   a.tickets = A->tickets;
-  a.dev_err = A->dev_err;
 
   // HELM_LAUNCH_AUTO: persistent inner solves where the device takes the launch
   // (else the graphs: a context can have fewer SMs than the device reports), but the
@@ -617,9 +606,8 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   // 8.80 / 8.30 / 8.28, 15^3 42.7 / 39.3 / 42.7; 18^3, 1.4 slices per SM, 50.6 / 57.8 /
   // 67.3)
   PShape ps;
-  const void* inner = nullptr;
-  with_shape(sh.k, [&](auto S) { inner = reinterpret_cast<const void*>(&k_mx_inner<S.value>); });
-  bool persistent = persist_default(A, sh.k, o) && sh.k.shape != SHAPE_LARGE && A->nsl > A->num_sms &&
+  const void* inner = reinterpret_cast<const void*>(&k_mx_inner<SHAPE_MID>);
+  bool persistent = persist_default(A, sh.k, o) && sh.k.shape == SHAPE_MID && A->nsl > A->num_sms &&
                     persist_fit(inner, n, sh.k.grid, sh.k.threads, sh.k.bps, 1, Phases<float2>::kOwn, sizeof(float2),
                                 &ps);
   (void)cudaGetLastError();

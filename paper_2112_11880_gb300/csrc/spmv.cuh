@@ -18,9 +18,11 @@
 //     120x60x50 cavity), each adding i Im(a) x with 2 more FMA.
 //   Padding entries (rows shorter than the slice width) are never read: each
 //   lane stops at its own row length.
-// Row sums run in CSR order over the real parts, then over the imaginary
-// parts: for a row whose entries are all real the result is the CSR-order
-// FP64 sum bit for bit.
+// A row's sum runs in CSR order over the real parts, then over the imaginary
+// parts, so that for a row whose entries are all real it is the CSR-order FP64 sum
+// bit for bit.  Two users sum it in parts instead, each part so, the parts added in
+// order: the solvers on the smallest meshes (kParts) and the stand-alone product of
+// matrices of few slices (k_spmv_split).
 //
 // Schedule (SliceRows): rounds of consecutive slices, each round split into
 // equal contiguous sub-ranges, one per block (one block per SM), one slice
@@ -374,21 +376,11 @@ __device__ __forceinline__ float2 dia_row(const CsrDev<float2>& A, int32_t s, in
   return imag_row<float2, G>(A, ib, (A.isoff[s + 1] - ib) >> 5, lane, r, x, acc);
 }
 
-struct NoGate {
-  __device__ __forceinline__ bool operator()() const { return true; }
-};
-
 // Walk this thread's rows; for each row r < n call epi.prefetch(r) (before
 // the row's sum, so the epilogue's own loads are in flight with it) and then
-// epi.row(r, sum_k a_rk x_k).  gate() is called first by every thread; it
-// must return the same value in the whole block, and on false the engine
-// returns without reading x.  Returns true.  Called by all threads of the
-// block (blockDim a multiple of 32).  `smem` and `dev_err` are unused: the
-// engine needs no shared memory and no wait.
-template <class V, class Epi, class Gate = NoGate, class G = GatherReadOnly, int U = kSpmvUnroll>
-__device__ __forceinline__ bool spmv_run(const CsrDev<V>& A, const V* __restrict__ x, Epi& epi,
-                                         unsigned char* /*smem*/, unsigned int* /*dev_err*/, Gate gate = Gate()) {
-  if (!gate()) return true;
+// epi.row(r, sum_k a_rk x_k).
+template <class V, class Epi, class G = GatherReadOnly, int U = kSpmvUnroll>
+__device__ __forceinline__ void spmv_run(const CsrDev<V>& A, const V* __restrict__ x, Epi& epi) {
   for (SliceRows q(A.n); q.active(); q.advance()) {
     const int32_t r = q.row();
     int32_t len = 0;
@@ -405,19 +397,16 @@ __device__ __forceinline__ bool spmv_run(const CsrDev<V>& A, const V* __restrict
     }
     if (r < A.n) epi.row(r, acc);
   }
-  return true;
 }
 
-// Launch shape of every SpMV-shaped kernel: 1024 threads (32 warps), one
-// block per SM (64 registers per thread at most), and a small dynamic
-// shared-memory block that kernels use for their block sums.  Measured on
-// GB300 (120x60x50 cavity): with 256-thread blocks, four per SM, the warps'
+// Launch shape of the stand-alone product and the FP64 products of a refinement
+// step: 1024 threads (32 warps), one block per SM (64 registers per thread at most).
+// Measured on GB300 (120x60x50 cavity): with 256-thread blocks, four per SM, the warps'
 // slice counts differed by one round and SMs idled 19 % of the SpMV.
 template <class V> struct Engine {
   static constexpr int R = 32;  // rows per slice
   static constexpr int kThreads = 1024;
   static constexpr int kMinBlocks = 1;
-  static constexpr size_t kSmem = 32 * 8 * sizeof(double);
 };
 
 // Device view of one value array of a handle (the caller's values, the

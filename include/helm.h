@@ -83,8 +83,8 @@ typedef struct helm_csr_s* helm_csr; /* opaque CSR handle */
  * most 32 diagonals col - row = const (the longest row's), rows are sorted
  * without duplicates, and the diagonals hold at most 1.5 slots per stored
  * entry (a structured mesh in its natural numbering), the complex64 value
- * sets also get a diagonal copy of their real parts (float[diagonals][n], no
- * column index; 4 bytes per slot): the complex64 product, bound by HBM on
+ * sets also get a diagonal copy of their real parts (float[diagonals][n rounded
+ * up to 4], no column index; 4 bytes per slot): the complex64 product, bound by HBM on
  * GB300, reads it instead of the sliced copy, with the same result for
  * finite x (the diagonals are summed in column order, empty slots skipped).
  * complex128 products always read the sliced copy (their bound is the FP64
@@ -131,13 +131,15 @@ helm_status helm_spmv(helm_csr A, const double* alpha, const void* d_x, const do
  * helm_dot -- d_out = (x, y) = sum_i conj(x_i) y_i when conj_x != 0 (zdotc),
  * sum_i x_i y_i when conj_x == 0 (zdotu).  Section 3 computes the dot product
  * as an element-wise product followed by a block-wise sum of the products;
- * here each block sums its share in a fixed order and one block adds the block
- * partials in block order, so the result is bit-for-bit reproducible.
+ * here each block sums its share in a fixed order and one block adds the blocks'
+ * sums in a fixed order, so the result is bit-for-bit reproducible.
  *   n     : vector length, 0 <= n < 2^31 (n = 0 gives 0).
- *   dt    : element type of x and y; complex64 inputs are accumulated in
- *           double precision.
+ *   dt    : element type of x and y; complex64 products are formed in single
+ *           precision and added in double (beyond 32,768 elements a thread adds its
+ *           own few in single first).
  *   d_out : device complex128 (double[2]).
- * Asynchronous.  Uses stream-ordered scratch memory (cudaMallocAsync).
+ * Asynchronous.  Up to 32,768 elements one launch (one cluster of blocks) without
+ * scratch; beyond, two with stream-ordered scratch memory (cudaMallocAsync).
  */
 helm_status helm_dot(int64_t n, helm_dtype dt, const void* d_x, const void* d_y, int conj_x,
                      void* d_out, helm_stream_t stream);
@@ -150,7 +152,8 @@ helm_status helm_dot(int64_t n, helm_dtype dt, const void* d_x, const void* d_y,
  * real-time loops that must never enter the allocator, or hosts that embed
  * this library under their own device-memory manager.  The paper has no
  * counterpart; it exists only for those callers.
- *   Scratch: the per-block partial sums live in a fixed 64 KiB array compiled
+ *   Scratch: beyond 32,768 elements (up to there it needs none, and the notes on
+ *   sharing do not apply) the per-block partial sums live in a fixed 64 KiB array compiled
  *   into the library (a file-scope __device__ array of 2 x 4096 doubles).
  *   Every GPU that loads libhelm holds one copy of it until the process
  *   exits.  No call allocates or frees anything: no cudaMalloc, cudaFree or
@@ -174,7 +177,7 @@ helm_status helm_dot_noalloc(int64_t n, helm_dtype dt, const void* d_x, const vo
 /*
  * helm_nrm2 -- d_out = ||x||_2 = sqrt(sum_i |x_i|^2) (Section 3, Table 7).
  *   d_out : device double.
- * Asynchronous, deterministic, stream-ordered scratch as helm_dot.
+ * Asynchronous, deterministic, scratch as helm_dot.
  */
 helm_status helm_nrm2(int64_t n, helm_dtype dt, const void* d_x, double* d_out,
                       helm_stream_t stream);

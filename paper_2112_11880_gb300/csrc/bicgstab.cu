@@ -115,7 +115,7 @@ helm_status bicgstab_fp64(helm_csr A, const double2* b, double2* x, const helm_o
       split = SolverBounds<S.value>::parts;
     });
     PShape ps;
-    if (persist_fit(fn, n, sh.grid, sh.threads, sh.bps, split, Phases<V>::kOwn, sizeof(V), &ps)) {
+    if (persist_fit(fn, A, sh.grid, sh.threads, sh.bps, split, Phases<V>::kOwn, sizeof(V), &ps)) {
       void* args[] = {&a, &ps.L};
       HELM_TRY(run_persistent(A, fn, args, ps, o, s, &done));
     }

@@ -646,7 +646,7 @@ helm_status bicgstabl_fp64(helm_csr A, const double2* b, double2* x, const helm_
       split = SolverBounds<S.value>::parts;
     });
     PShape ps;
-    if (persist_fit(fn, A->n, sh.grid, sh.threads, sh.bps, split, slot_u(ell) + 1, sizeof(V), &ps)) {
+    if (persist_fit(fn, A, sh.grid, sh.threads, sh.bps, split, slot_u(ell) + 1, sizeof(V), &ps)) {
       void* args[] = {&a, &ps.L};
       HELM_TRY(run_persistent(A, fn, args, ps, o, s, &done));
     }

@@ -608,7 +608,7 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
   PShape ps;
   const void* inner = reinterpret_cast<const void*>(&k_mx_inner<SHAPE_MID>);
   bool persistent = persist_default(A, sh.k, o) && sh.k.shape == SHAPE_MID && A->nsl > A->num_sms &&
-                    persist_fit(inner, n, sh.k.grid, sh.k.threads, sh.k.bps, 1, Phases<float2>::kOwn, sizeof(float2),
+                    persist_fit(inner, A, sh.k.grid, sh.k.threads, sh.k.bps, 1, Phases<float2>::kOwn, sizeof(float2),
                                 &ps);
   (void)cudaGetLastError();
 

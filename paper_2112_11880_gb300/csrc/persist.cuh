@@ -336,12 +336,12 @@ struct PShape {
   size_t smem = 0;
 };
 
-// Fit a persistent kernel on a grid of `grid` blocks (bps per SM) of `owners`
-// owner threads, times `split` warps a slice: the table and as many of `want`
-// own vectors of `elem` bytes as there is room for.  False when the kernel
+// Fit a persistent kernel for the system A on a grid of `grid` blocks (bps per SM)
+// of `owners` owner threads, times `split` warps a slice: the table and as many of
+// `want` own vectors of `elem` bytes as there is room for.  False when the kernel
 // cannot run so.
-inline bool persist_fit(const void* fn, int32_t n, int grid, int owners, int bps, int split, int want, size_t elem,
-                        PShape* p) {
+inline bool persist_fit(const void* fn, const helm_csr_s* A, int grid, int owners, int bps, int split, int want,
+                        size_t elem, PShape* p) {
   int dev = 0, per_sm = 0, optin = 0, reserved = 0, coop = 0;
   cudaFuncAttributes fa;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -353,8 +353,8 @@ inline bool persist_fit(const void* fn, int32_t n, int grid, int owners, int bps
     return false;
   p->grid = grid;
   p->threads = owners * split;
-  const size_t room = persist_room(per_sm, optin, reserved, fa.sharedSizeBytes, bps);
-  if (!persist_plan(n, grid, owners, split, want, elem, room, &p->L, &p->smem)) return false;
+  const size_t room = persist_room(per_sm, optin, reserved, fa.sharedSizeBytes, bps, A->ndia > 0);
+  if (!persist_plan(A->n, grid, owners, split, want, elem, room, &p->L, &p->smem)) return false;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            optin - static_cast<int>(fa.sharedSizeBytes)) != cudaSuccess)
     return false;

@@ -53,17 +53,21 @@ inline size_t persist_layout(PLayout* L, size_t elem) {
 }
 
 // Shared memory a block may take, of `bps` blocks per SM that have `per_sm` bytes
-// between them: `reserved` and `fixed` (static) bytes go off each.  All blocks of
-// an SM stay within kPersistSmem, because what they leave of its 256 kB is L1, and
-// a warp's gathers from scattered columns each hold a line of it while they are in
-// flight: own vectors in shared memory gain next to nothing (120x60x50, us per
-// BiCGStab iteration with 16 / 48 / 112 / 227 kB per SM: 120 / 121 / 122 / 121), a
-// small L1 costs up to a factor of two where columns are scattered (27 a row, n =
-// 400,009: 141 / 141 / 143 / 251; TFQMR, 200,003: 90 / 88 / 89 / 141; BiCGStab,
-// 1,600,003: 477 / 478 / 505 / 1205).
+// between them: `reserved` and `fixed` (static) bytes go off each.  What the blocks of
+// an SM leave of its 256 kB is its L1, and each of a warp's gathers from scattered
+// columns holds a line of it while in flight; own vectors in shared memory gain 1 % at
+// most, a small L1 costs up to a factor of two.  So all blocks of an SM stay within
+// kPersistSmem, unless the columns of neighbouring rows are neighbours (`near`: the
+// matrix lies on few diagonals) and a block has the SM to itself.
+// Measured (us per iteration with 16 / 48 / 112 / 227 kB per SM): 27 random columns a
+// row, BiCGStab, n = 300,007 114 / 112 / 113 / 192, 400,009 141 / 141 / 143 / 251,
+// 1,600,003 477 / 478 / 505 / 1205; TFQMR, 200,003 90 / 88 / 89 / 141; meshes,
+// BiCGStab, 120x60x50 120 / 121 / 122 / 121, 200x100x80 466 / 468 / 472 / 469;
+// BiCGStab(2), 120x60x50 271 / 268 / 271 / 268.
 constexpr size_t kPersistSmem = 100 * 1024;
-inline size_t persist_room(size_t per_sm, size_t optin, size_t reserved, size_t fixed, int bps) {
-  const size_t block = std::min(std::min(per_sm, kPersistSmem) / bps - reserved, optin);
+inline size_t persist_room(size_t per_sm, size_t optin, size_t reserved, size_t fixed, int bps, bool near) {
+  const size_t sm = near && bps == 1 ? per_sm : std::min(per_sm, kPersistSmem);
+  const size_t block = std::min(sm / bps - reserved, optin);
   return block > fixed ? block - fixed : 0;
 }
 

@@ -574,7 +574,7 @@ helm_status tfqmr_fp64(helm_csr A, const double2* b, double2* x, const helm_opts
       split = SolverBounds<S.value>::parts;
     });
     PShape ps;
-    if (persist_fit(fn, A->n, sh.grid, sh.threads, sh.bps, split, TqPhases::kOwn, sizeof(V), &ps)) {
+    if (persist_fit(fn, A, sh.grid, sh.threads, sh.bps, split, TqPhases::kOwn, sizeof(V), &ps)) {
       void* args[] = {&a, &ps.L};
       HELM_TRY(run_persistent(A, fn, args, ps, o, s, &done));
     }

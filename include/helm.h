@@ -216,7 +216,8 @@ typedef enum {
                                  to some 240,000 unknowns), else graph; the
                                  host-driven loop if the graph cannot be built.
                                  Graph also for matrices with long rows (FP64
-                                 above 262,144 entries, 192 beyond some 730,000
+                                 above 37,000 to 262,144 entries, the fewer the
+                                 larger the system, above 192 beyond some 730,000
                                  unknowns; mixed precision above 128).  A
                                  persistent solve holds every SM (up to one
                                  block per slice of 32 rows) until it ends:

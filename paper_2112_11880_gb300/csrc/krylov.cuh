@@ -968,7 +968,8 @@ struct KShapes {
 template <class V>
 inline bool persist_default(helm_csr A, const KShapes<V>& sh, const helm_opts& o) {
   return o.launch == HELM_LAUNCH_AUTO &&
-         A->max_row <= persist_max_row(sh.shape == SHAPE_LARGE, std::is_same<V, float2>::value);
+         A->max_row <= persist_max_row(sh.shape == SHAPE_LARGE, std::is_same<V, float2>::value,
+                                       persist_rounds(A->n, sh.grid, sh.threads / 32));
 }
 
 // A whole solve as one cooperative launch of `fn` on the shape that persist_fit

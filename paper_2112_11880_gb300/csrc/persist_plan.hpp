@@ -106,8 +106,11 @@ inline bool persist_plan(int32_t n, int grid, int owners, int split, int want, s
 //     1024 336 / 249 (259);
 //   mid, n = 100,000: L = 1024 BiCGStab 384 / 352 (408), TFQMR 385 / 399 (434),
 //     BiCGStab(2) 836 / 729 (915): ahead of what was at every length.
-// Above 2^18 a step would come near the time that a wait lasts (1.1 s a product of a
-// row of 3.3 million entries; an entry with an imaginary part takes longer).
-inline int32_t persist_max_row(bool large, bool c64) { return c64 ? 128 : large ? 192 : 1 << 18; }
+// A warp takes a row in each of its rounds, and a step has to stay well inside the
+// time that a wait lasts: above 2^18 entries in all the graph (0.34 us an entry, 1.1 s
+// a product of a row of 3.3 million; an entry with an imaginary part another 1 us).
+inline int32_t persist_max_row(bool large, bool c64, int32_t rounds) {
+  return c64 ? 128 : large ? 192 : (1 << 18) / rounds;
+}
 
 }  // namespace helm

@@ -45,8 +45,8 @@ def test_a_step_of_more_than_a_second():
 
 @pytest.mark.parametrize("n,length,precision", [
     (300_000, 128, helm.HELM_PREC_MIXED), (200_000, 129, helm.HELM_PREC_MIXED), (200_000, 3000, helm.HELM_PREC_MIXED),
-    (15_000, 15_000, helm.HELM_PREC_FP64), (300_000, 1 << 18, helm.HELM_PREC_FP64),
-    (300_000, (1 << 18) + 1, helm.HELM_PREC_FP64), (1_000_000, 192, helm.HELM_PREC_FP64),
+    (15_000, 15_000, helm.HELM_PREC_FP64), (300_000, 1 << 16, helm.HELM_PREC_FP64),
+    (300_000, 1 << 18, helm.HELM_PREC_FP64), (1_000_000, 192, helm.HELM_PREC_FP64),
     (1_000_000, 193, helm.HELM_PREC_FP64),
 ])
 def test_forms_agree_on_both_sides_of_the_rule(n, length, precision):

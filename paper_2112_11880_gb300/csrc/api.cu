@@ -873,7 +873,7 @@ helm_status build_sell_vals(helm_csr A, const void* vals, helm_dtype dt, SellVal
 }
 
 // Graphs capture buffer addresses: drop them whenever a buffer is replaced.
-static void drop_graphs(helm_csr A) {
+void drop_graphs(helm_csr A) {
   for (auto& kv : A->graphs) {
     if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
     if (kv.second.graph) cudaGraphDestroy(kv.second.graph);

@@ -140,13 +140,7 @@ helm_status bicgstab_fp64(helm_csr A, const double2* b, double2* x, const helm_o
     } else {
       GraphEntry e;
       if (build_krylov_graph<V>(a, sh, tail, &e) == HELM_OK) {
-        if (A->graphs.size() >= 16) {  // bound the cache
-          for (auto& kv : A->graphs) {
-            cudaGraphExecDestroy(kv.second.exec);
-            cudaGraphDestroy(kv.second.graph);
-          }
-          A->graphs.clear();
-        }
+        bound_graphs(A, 1);
         g = &(A->graphs[key] = e);
       }
     }

@@ -672,8 +672,10 @@ helm_status bicgstabl_fp64(helm_csr A, const double2* b, double2* x, const helm_
             },
             [&](cudaGraphConditionalHandle c, cudaStream_t cs) { bl_body(with(c), sh, cs); },
             [&](cudaGraphConditionalHandle c, cudaStream_t cs) { bl_tail(with(c), sh, cs); },
-            &e) == HELM_OK)
+            &e) == HELM_OK) {
+      bound_graphs(A, 1);
       g = &(A->graphs[key] = e);
+    }
   }
 
   // an explicit graph request does not fall back to the host-driven loop

@@ -179,6 +179,15 @@ inline std::tuple<const void*, const void*, int> graph_key(const void* b, const 
   return std::make_tuple(b, x, 2 * tag + (o.precond == HELM_PRECOND_JACOBI ? 1 : 0));
 }
 
+// The graphs of a handle, one per (b, x, variant).  drop_graphs frees them all;
+// bound_graphs does so when `more` new ones would pass kMaxGraphs.  Called under the
+// handle's lock, with none of its graphs running (every solve waits for its own).
+constexpr size_t kMaxGraphs = 16;
+void drop_graphs(helm_csr A);
+inline void bound_graphs(helm_csr A, size_t more) {
+  if (A->graphs.size() + more > kMaxGraphs) drop_graphs(A);
+}
+
 helm_status ensure_jacobi(helm_csr A, cudaStream_t s);
 helm_status bicgstab_fp64(helm_csr A, const double2* b, double2* x, const helm_opts& o, helm_info* info,
                           cudaStream_t s);

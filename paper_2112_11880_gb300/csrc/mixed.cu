@@ -634,6 +634,7 @@ helm_status solve_mixed(helm_csr A, const double2* b, double2* x, const helm_opt
                             &ei) == HELM_OK;
       const bool ok_s = ok_i && build_plain_graph([&](cudaStream_t cs) { mx_step(a, sh, cs); }, &es) == HELM_OK;
       if (ok_i && ok_s) {
+        bound_graphs(A, 2);
         gi = &(A->graphs[ki] = ei);
         gs = &(A->graphs[ks] = es);
       } else {
